@@ -61,9 +61,11 @@ typedef struct {
   int32_t sketch_rows;     /* [0 = 400 if eps >= 1e-7, else 800] rows of the random sketch in the
                               pivoted QR (at least twice the largest rank) */
   double eps_op_factor;    /* [0 = 0.3 if eps >= 1e-7, else 0.1] skeleton tolerance = eps * factor */
-  int32_t m2l_mode;        /* [0] translations on: 0 = automatic (tensor cores if eps >= 1e-5, else
-                              FP32 CUDA cores), 1 = FP32 CUDA cores, 2 = tensor cores (tcgen05,
-                              scaled FP16 hi/lo split; adds about 2e-6 relative error) */
+  int32_t m2l_mode;        /* [0] translations on: 0 = automatic (tensor cores: the split of mode 2 if
+                              eps >= 1e-5, else the sliced form, which keeps the full FP32 or FP64
+                              precision; CUDA cores where neither applies), 1 = CUDA cores,
+                              2 = tensor cores (tcgen05, scaled FP16 hi/lo split; adds about 2e-6
+                              relative error) */
   int32_t host_threads;    /* [0 = all cores] threads for the skeleton precompute */
   const char* cache_dir;   /* [NULL = no disk cache] directory for skeleton files */
   int32_t tc_stages;       /* [0 = all] with m2l_mode 2, the translation families that run on
@@ -105,11 +107,12 @@ typedef struct {
                               whose target rank exceeds 128 then run on the FP32 CUDA cores. */
   int32_t arith;           /* [0] arithmetic of the apply: 0 = automatic (32 if eps >= 1e-6, else
                               64); 32 = the FP32 forms above (complex64 f and u); 64 = FP64
-                              throughout (translations, rows, check points and near field on
-                              the CUDA cores; operators kept in complex128), for eps down to
-                              1e-8.  With 64, f and u of every apply entry point are complex128
-                              [nrhs][N], m2l_mode 2 is refused and the other m2l / p2p / tc
-                              options are ignored; dfmm_solve takes arith 32 plans only. */
+                              throughout (rows, check points and near field on the CUDA cores,
+                              translations there with m2l_mode 1 and in FP64-exact slices on the
+                              tensor cores otherwise; operators kept in complex128), for eps down
+                              to 1e-8.  With 64, f and u of every apply entry point are complex128
+                              [nrhs][N], m2l_mode 2 is refused and the p2p / tc options are
+                              ignored; dfmm_solve takes arith 32 plans only. */
   int32_t skeleton_host;   /* [0] where the skeleton pivot selection (Sec. 2.1: pivoted QR of the
                               random sketch, then of the far samples) runs: 0 = on the GPU for all
                               representation types of the plan at once; 1 = host threads
@@ -217,8 +220,11 @@ typedef struct {
 int dfmm_plan_stats(dfmm_plan_t plan, dfmm_stats* out);
 
 /* Device bytes of the workspace that one apply with nrhs right-hand sides
- * needs (sorted densities and potentials, translation states, staging buffers
- * and work tables; the plan itself is not included).  -1 on a bad argument. */
+ * needs at least (sorted densities and potentials, translation states, staging
+ * buffers and work tables; the plan itself is not included).  Plans whose
+ * translations are sliced (automatic form below eps 1e-5) take a source buffer
+ * of their slices beside it where the memory at hand holds it, and run on the
+ * CUDA cores where it does not.  -1 on a bad argument. */
 int64_t dfmm_apply_workspace_bytes(dfmm_plan_t plan, int nrhs);
 
 /* Device bytes held by the plan (tree, lists, operators, evaluation rows);

@@ -93,6 +93,26 @@ void launch_split_cx(const float2* x, int64_t rows, int r, void* hi, void* lo, f
 void launch_gemm_stage_cx(const GemmArgs& a, const TcArgs& t, unsigned* status, bool one_acc, int kind,
                           cudaStream_t s);
 
+// Sliced tensor-core form (m2l_sl.cu): FP32 or FP64 products without loss of
+// precision on the FP16 tensor cores, for M, Kd multiples of 8 up to 512 and
+// dense source rows.  src / src_scale: the source buffer's slices
+// (launch_split_sl, sl_row_bytes per row) and per-row scales; img / op_scale:
+// the operator images (build_sl_image).  Scales are float, or double with fp64,
+// where every complex array holds complex128.  Tiles hold up to
+// gemm_tc_columns() columns.
+struct SlArgs {
+  const void* src;
+  const void* src_scale;
+  const void* img;
+  const void* op_scale;
+};
+bool gemm_sl_supported(int M, int Kd);
+int64_t sl_row_bytes(int r, bool fp64);
+int64_t sl_image_bytes(int M, int Kd, int nops, bool fp64);
+void build_sl_image(const float2* ops, int M, int Kd, int nops, void* img, void* scale, bool fp64, cudaStream_t s);
+void launch_split_sl(const float2* x, int64_t rows, int r, void* out, void* scale, bool fp64, cudaStream_t s);
+void launch_gemm_stage_sl(const GemmArgs& a, const SlArgs& t, unsigned* status, bool fp64, cudaStream_t s);
+
 // Permutes: fs[k][rhs] = f[rhs][perm[k]];  u[rhs][perm[k]] = us[k][rhs].
 void launch_permute_in(const float2* f, const int32_t* perm, int64_t N, int nrhs, float2* fs, cudaStream_t s);
 void launch_permute_out(const float2* us, const int32_t* perm, int64_t N, int nrhs, float2* u, cudaStream_t s);
@@ -112,6 +132,8 @@ struct P2CArgs {
   float2* out;               // [rows][nrhs][ld]
   int nrhs;
   const double* chk64;       // FP64 form: the check points, [nchk][3]
+  int halves;                // FP64 form: 1, or 2: each half of a row's check points is a row of its own,
+                             //   out[2 row + half][rhs][ld / 2]
   const float4* pts_lo;      // FP64 form: low parts of the local coordinates
 };
 void launch_p2c(const P2CArgs& a, cudaStream_t s);

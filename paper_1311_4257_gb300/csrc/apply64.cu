@@ -150,6 +150,7 @@ __global__ __launch_bounds__(C64_T) void p2c64_kernel(P2CArgs a) {
   const int4 job = a.jobs[blockIdx.x];
   const float4 sh = a.shifts[job.w];
   const double2* fs = c128(a.fs);
+  const int half = a.ld / a.halves;   // the row's length where its halves are rows of their own
   double2* out = c128(a.out) + (int64_t)job.z * a.nrhs * a.ld;
   for (int r0 = 0; r0 < a.nrhs; r0 += C64_NR) {
     const int nr = min(C64_NR, a.nrhs - r0);
@@ -181,7 +182,8 @@ __global__ __launch_bounds__(C64_T) void p2c64_kernel(P2CArgs a) {
           }
       }
       if (p < a.ld)
-        for (int k = 0; k < nr; ++k) out[(int64_t)(r0 + k) * a.ld + p] = live ? acc[k] : make_double2(0.0, 0.0);
+        for (int k = 0; k < nr; ++k)
+          out[(int64_t)((p / half) * a.nrhs + r0 + k) * half + p % half] = live ? acc[k] : make_double2(0.0, 0.0);
     }
   }
 }

@@ -8,9 +8,9 @@
 // operators and evaluation rows in FP64 (operators.cu).
 // Apply (one stream, no host synchronisation): permute in, P2M, LF-M2M, the
 // top V list, then per HF level HF-M2M and HF-M2L, HF-L2L, HF->LF L2L, LF-L2L
-// and LF-M2L (V), P2L (X), L2P, M2P (W), P2P (U), permute out.  The tensor-core
-// (m2l_cx.cu, m2l_tc.cu), FP32 (apply.cu) and FP64 (apply64.cu) kernels serve
-// the three arithmetic forms.  Also here: the allocation-free and captured
+// and LF-M2L (V), P2L (X), L2P, M2P (W), P2P (U), permute out.  The split
+// (m2l_cx.cu, m2l_tc.cu) and sliced (m2l_sl.cu) tensor-core, FP32 (apply.cu) and
+// FP64 (apply64.cu) kernels serve the arithmetic forms.  Also here: the allocation-free and captured
 // applies, the batched forms, dfmm_validate and the live-plan registry.
 #include "dfmm.h"
 
@@ -66,6 +66,8 @@ struct GemmPlan {
   int fam = 0;                     // profiling family
   __half* img = nullptr;           // tensor-core operator image (tensor form only)
   float* op_scale = nullptr;       // its per-operator power-of-two scales
+  void* sl_img = nullptr;          // sliced operator image (m2l_sl.cu; automatic form below eps 1e-5)
+  void* sl_scale = nullptr;        // its per-operator scales (float, double in the FP64 form)
   double flops_rhs = 0;            // algorithmic flops per right-hand side
   double bytes_fixed = 0;          // operators (bytes once per launch)
   double bytes_rhs = 0;            // unique source rows + target rows (read and write), per rhs
@@ -104,6 +106,7 @@ struct LFLevel {
   int R = 0, r = 0;
   int64_t nbox = 0;
   GemmPlan m2m, l2l, v, p2l;   // m2m from l+1, l2l from l-1 (LF or HF)
+  int p2l_halves = 1;          // operators the P2L projection's columns are divided over
   ChkPt* chk_b2 = nullptr;
   double* chk64 = nullptr;         // FP64 form: the check points b2, [2r][3]
   int4* p2l_jobs = nullptr;
@@ -135,6 +138,8 @@ struct Workspace {
   float2 *fs = nullptr, *us = nullptr, *p2l = nullptr;
   __half *ahi = nullptr, *alo = nullptr;                // split source buffer (tensor form)
   float* ascale = nullptr;                              // its per-row scales
+  void *sl = nullptr, *sl_scale = nullptr;              // sliced source buffer and its row scales (sliced form;
+                                                        // null: the stages run on the CUDA cores)
   std::vector<float2*> S, T;                            // per level (LF or HF states)
   std::vector<std::pair<void*, size_t>> zero;           // reset before each apply
   std::vector<std::pair<void*, size_t>> zero_late;      // reset on the side stream, first read by HF M2M
@@ -191,6 +196,7 @@ struct dfmm_plan_s {
   double K = 0, W = 0, eps = 0, eps_op = 0;
   dfmm_options opt{};
   bool fp64 = false;   // FP64 form (options.arith 64): complex128 densities, states and operators
+  bool sliced = false; // translations in the sliced tensor-core form (automatic form below eps 1e-5)
   int cw = 1;          // complex element width in float2 units (2 in the FP64 form)
   DevArena ar;
   TreeBuilder tree;
@@ -231,8 +237,6 @@ struct dfmm_plan_s {
 struct dfmm_graph_s {
   dfmm_plan_s* plan = nullptr;
   DevArena ar;
-  char* scratch = nullptr;
-  size_t bytes = 0;
   Workspace W;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -375,16 +379,16 @@ T* upload(const std::vector<T>& v, DevArena& ar, cudaStream_t s) {
   return d;
 }
 
-// conjugate transpose of a 2r x r matrix, columns scaled, padded to R x 2R:
-// complex64, or complex128 for the FP64 form
-float2* upload_projection(const std::vector<cd>& Q, int r, const double* colscale, int R, bool fp64, DevArena& ar,
+// conjugate transpose of a 2r x r matrix, padded to R x 2R and divided by columns
+// into `halves` operators: complex64, or complex128 for the FP64 form
+float2* upload_projection(const std::vector<cd>& Q, int r, int halves, int R, bool fp64, DevArena& ar,
                           cudaStream_t s) {
   std::vector<double2> h((size_t)R * 2 * R, make_double2(0, 0));
+  const int Kd = 2 * R / halves;
   for (int i = 0; i < r; ++i)
     for (int j = 0; j < 2 * r; ++j) {
-      cd v = std::conj(Q[(size_t)j * r + i]);
-      if (colscale) v *= colscale[j];
-      h[(size_t)i * 2 * R + j] = make_double2(v.real(), v.imag());
+      const cd v = std::conj(Q[(size_t)j * r + i]);
+      h[((size_t)(j / Kd) * R + i) * Kd + j % Kd] = make_double2(v.real(), v.imag());
     }
   if (fp64) return (float2*)upload(h, ar, s);
   std::vector<float2> f(h.size());
@@ -617,8 +621,11 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
     const int R = F.R;
     F.chk_b2 = upload_chk(rp.b2, 2 * rp.r, ar, s);
     if (P->fp64) F.chk64 = upload(rp.b2, ar, s);
-    F.p2l.M = R; F.p2l.Kd = 2 * R; F.p2l.nops = 1;
-    F.p2l.ops = upload_projection(rp.Qi, rp.r, nullptr, R, P->fp64, ar, s);
+    // the P2L projection, R x 2R; the sliced FP64 form takes it as two operators of R
+    // columns on the two halves of a check-point row, whose integer sums stay exact
+    F.p2l_halves = P->sliced && P->fp64 ? 2 : 1;
+    F.p2l.M = R; F.p2l.Kd = 2 * R / F.p2l_halves; F.p2l.nops = F.p2l_halves;
+    F.p2l.ops = upload_projection(rp.Qi, rp.r, F.p2l_halves, R, P->fp64, ar, s);
     std::vector<int4> jobs;
     std::vector<int32_t> op;
     std::vector<int2> pr;
@@ -639,8 +646,10 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
         for (int d = 0; d < 3; ++d) sh[d] = (float)(center(la, a, d) - center(lb, b, d));
         xs.push_back(make_float4(sh[0], sh[1], sh[2], 0.f));
         xj.push_back(make_int4(LV[la].h_first[a], LV[la].h_count[a], (int)xj.size(), (int)xs.size() - 1));
-        op.push_back(0);
-        pr.push_back(make_int2((int)xj.size() - 1, b));
+        for (int h = 0; h < F.p2l_halves; ++h) {
+          op.push_back(h);
+          pr.push_back(make_int2((int)(xj.size() - 1) * F.p2l_halves + h, b));
+        }
       }
       F.n_p2l = (int64_t)xj.size();
       for (auto& j : xj) F.npts_x += j.x >= 0 ? j.y : 0;
@@ -648,7 +657,7 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
       F.p2l_shifts = upload(xs, ar, s);
       F.p2l.fam = F_P2L_PROJ;
       F.p2l.flops_rhs = 8.0 * rp.r * 2 * rp.r * F.n_p2l;
-      F.p2l.src_rows = F.n_p2l;
+      F.p2l.src_rows = F.n_p2l * F.p2l_halves;
       F.p2l.dst_rows = LV[l].n;
       finish_gemm(F.p2l, op, pr, ar, s);
     }
@@ -1126,7 +1135,7 @@ int64_t max_source_rows(const dfmm_plan_s* P) {
   int64_t m = 1;
   for (int l = 0; l < P->nl; ++l) {
     if (l >= P->l_lf0) {
-      m = std::max({m, P->lf[l].nbox, P->lf[l].n_p2l});
+      m = std::max({m, P->lf[l].nbox, P->lf[l].n_p2l * P->lf[l].p2l_halves});
     } else if (P->l_top >= 0 && l >= P->l_top) {
       m = std::max(m, (int64_t)std::max(P->hf[l].out_keys.size(), P->hf[l].in_keys.size()));
     }
@@ -1146,6 +1155,22 @@ int64_t max_source_elems(const dfmm_plan_s* P) {
     } else if (P->l_top >= 0 && l >= P->l_top) {
       const HFLevel& H = P->hf[l];
       m = std::max(m, (int64_t)std::max(H.out_keys.size(), H.in_keys.size()) * H.R);
+    }
+  }
+  return m;
+}
+
+// Bytes of the sliced source buffer, per RHS (the row scales are max_sl_rows * nrhs values).
+int64_t max_slice_bytes(const dfmm_plan_s* P) {
+  int64_t m = 0;
+  for (int l = 0; l < P->nl; ++l) {
+    if (l >= P->l_lf0) {
+      const LFLevel& F = P->lf[l];
+      m = std::max(m, F.nbox * sl_row_bytes(F.R, P->fp64));
+      m = std::max(m, F.n_p2l * F.p2l_halves * sl_row_bytes(2 * F.R / F.p2l_halves, P->fp64));
+    } else if (P->l_top >= 0 && l >= P->l_top) {
+      const HFLevel& H = P->hf[l];
+      m = std::max(m, (int64_t)std::max(H.out_keys.size(), H.in_keys.size()) * sl_row_bytes(H.R, P->fp64));
     }
   }
   return m;
@@ -1192,6 +1217,16 @@ Workspace* get_workspace(dfmm_plan_s* P, cudaStream_t s, int nrhs) {
     W->alo = ar.alloc<__half>(e);
     W->ascale = ar.alloc<float>(max_source_rows(P) * nrhs);
   }
+  if (P->sliced) {
+    try {
+      W->sl = ar.alloc<char>(max_slice_bytes(P) * nrhs);
+      W->sl_scale = ar.alloc<double>(max_source_rows(P) * nrhs);
+    } catch (const Error& e) {   // no room for the slices: the stages run on the CUDA cores
+      if (e.code != DFMM_ERR_OOM) throw;
+      cudaGetLastError();
+      W->sl = W->sl_scale = nullptr;
+    }
+  }
   W->status = ar.alloc<unsigned>(1);
   W->zero.push_back({W->status, 4});   // reset by every apply; read by dfmm_sync_status
   DFMM_CUDA(cudaMemsetAsync(W->status, 0, 4, s));
@@ -1219,6 +1254,10 @@ bool on_tensor_cores(const dfmm_plan_s* P, const GemmPlan& g) {
 bool split_complex(const dfmm_plan_s* P, const GemmPlan& g) {
   return on_tensor_cores(P, g) && P->opt.tc_layout != 1 && gemm_cx_supported(g.M, g.Kd);
 }
+
+// whether a stage has the sliced form (m2l_sl.cu): operators sliced at plan time; it runs so
+// where the workspace holds the slices of its source
+bool sliced_stage(const GemmPlan& g) { return g.sl_img != nullptr; }
 
 // tile_order: 0 = by the 64 MB rule above, 1 = always by target block, 2 = always by operator.
 // block_bytes: target rows per block in the blocked order (8 MB unless the
@@ -1324,10 +1363,11 @@ struct Runner {
     if (g.npairs == 0) return;
     const bool tc = on_tensor_cores(P, g);
     const bool cx = tc && split_complex(P, g);
+    const bool sl = sliced_stage(g) && (count || W->sl);
     // the split arrays hold one source buffer in one layout (interleaved or split-complex)
     const int key = src_key < 0 ? -1 : 2 * src_key + (cx ? 1 : 0);
-    const bool split = tc && (key < 0 || key != split_key);
-    if (tc) split_key = key;
+    const bool split = (tc || sl) && (key < 0 || key != split_key);
+    if (tc || sl) split_key = key;
     if (count) { count[0] += split ? 2 : 1; return; }
     if (skip()) return;
     if (ctl && ctl->collect && cx) {   // the batched form merges this stage with the other plans' same stage
@@ -1335,7 +1375,7 @@ struct Runner {
                                        (first && g.dst_unique) ? 1 : 0});
       return;
     }
-    auto t = tiles_for(P, W, g, nrhs, tc ? gemm_tc_columns() : 64, s);
+    auto t = tiles_for(P, W, g, nrhs, tc || sl ? gemm_tc_columns() : 64, s);
     GemmArgs a;
     a.ops = g.ops;
     a.M = g.M;
@@ -1361,6 +1401,13 @@ struct Runner {
       TcArgs targs{g.img, g.op_scale, W->ahi, W->alo, W->ascale};
       if (cx) launch_gemm_stage_cx(a, targs, W->status, P->opt.tc_accumulate == 1, P->opt.tc_precision, s);
       else launch_gemm_stage_tc(a, targs, W->status, s);
+    } else if (sl) {
+      if (split) {
+        ProfScope ps(W, s, F_SPLIT, 0.0, (double)src_rows * nrhs * (src_ld * 8.0 * P->cw + sl_row_bytes(src_ld, P->fp64)));
+        launch_split_sl(src, src_rows * nrhs, src_ld, W->sl, W->sl_scale, P->fp64, s);
+      }
+      ProfScope ps(W, s, g.fam, g.flops_rhs * nrhs, g.bytes_fixed + g.bytes_rhs * nrhs);
+      launch_gemm_stage_sl(a, SlArgs{W->sl, W->sl_scale, g.sl_img, g.sl_scale}, W->status, P->fp64, s);
     } else {
       ProfScope ps(W, s, g.fam, g.flops_rhs * nrhs, g.bytes_fixed + g.bytes_rhs * nrhs);
       if (P->fp64) launch_gemm_stage64(a, s);
@@ -1487,11 +1534,12 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
         a.out = W->p2l;
         a.nrhs = nrhs;
         a.chk64 = F.chk64;
+        a.halves = F.p2l_halves;
         a.pts_lo = P->pts_lo;
         if (P->fp64) launch_p2c64(a, s);
         else launch_p2c(a, s);
       });
-      R.at(wave_lf_down(lw(l), 3)).gemm(F.p2l, count ? nullptr : W->p2l, 2 * F.R, F.n_p2l, T(l), F.R, -1);
+      R.at(wave_lf_down(lw(l), 3)).gemm(F.p2l, count ? nullptr : W->p2l, F.p2l.Kd, F.n_p2l * F.p2l_halves, T(l), F.R, -1);
     }
   }
   // 5. L2P at every leaf, M2P over the W list
@@ -1566,8 +1614,9 @@ std::vector<const GemmPlan*> all_gemms(dfmm_plan_s* P) {
 // [base, base + bytes): the device status word (at offset 0), state buffers,
 // staging buffers and the work tiles of every stage (copied in on `s`).  No device memory is allocated.  With
 // base == nullptr nothing is laid out or copied: the return value is the
-// number of bytes the layout needs.
-size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaStream_t s, Workspace& W) {
+// number of bytes the layout needs.  slices: with the sliced form's source
+// buffer; without it the plan's sliced stages run on the CUDA cores.
+size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaStream_t s, Workspace& W, bool slices) {
   size_t off = 0;
   auto take = [&](size_t n) -> char* {
     off = (off + 255) & ~(size_t)255;
@@ -1610,11 +1659,16 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
     W.alo = (__half*)take(e * 2);
     W.ascale = (float*)take((size_t)max_source_rows(P) * nrhs * 4);
   }
+  slices = slices && P->sliced;
+  if (slices) {
+    W.sl = take((size_t)max_slice_bytes(P) * nrhs);
+    W.sl_scale = take((size_t)max_source_rows(P) * nrhs * 8);
+  }
   std::vector<std::pair<const GemmPlan*, std::vector<int4>>> tl;
   std::vector<int> tl_cols;
   for (const GemmPlan* g : all_gemms(P)) {
     if (g->npairs == 0) continue;
-    const int cols = on_tensor_cores(P, *g) ? gemm_tc_columns() : 64;
+    const int cols = on_tensor_cores(P, *g) || (slices && sliced_stage(*g)) ? gemm_tc_columns() : 64;
     tl_cols.push_back(cols);
     tl.push_back({g, make_tiles(*g, nrhs, cols, P->opt.tile_order)});
   }
@@ -1632,10 +1686,28 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
   return off;
 }
 
-// Device bytes of one apply's workspace with nrhs right-hand sides.
-int64_t workspace_bytes(dfmm_plan_s* P, int nrhs) {
+// Device bytes of one apply's workspace with nrhs right-hand sides: the least an
+// apply runs in, or (slices) with room for the sliced form of plans that have it.
+int64_t workspace_bytes(dfmm_plan_s* P, int nrhs, bool slices) {
   Workspace W;
-  return (int64_t)carve_workspace(P, nrhs, nullptr, 0, nullptr, W);
+  return (int64_t)carve_workspace(P, nrhs, nullptr, 0, nullptr, W, slices);
+}
+
+// A carved workspace of its own in `ar`: with the slices, or where they do not fit the device, without.
+void own_workspace(dfmm_plan_s* P, int nrhs, DevArena& ar, cudaStream_t s, Workspace& W) {
+  bool slices = P->sliced;
+  size_t bytes = (size_t)workspace_bytes(P, nrhs, slices);
+  char* base = nullptr;
+  try {
+    base = ar.alloc<char>((int64_t)bytes);
+  } catch (const Error& e) {
+    if (!slices || e.code != DFMM_ERR_OOM) throw;
+    cudaGetLastError();
+    slices = false;
+    bytes = (size_t)workspace_bytes(P, nrhs, false);
+    base = ar.alloc<char>((int64_t)bytes);
+  }
+  carve_workspace(P, nrhs, base, bytes, s, W, slices);
 }
 
 // Operator images of every translation stage for the tensor-core form.
@@ -1651,6 +1723,28 @@ void build_images(dfmm_plan_s* P, cudaStream_t s) {
       g->img = P->ar.alloc<__half>(tc_image_elems(g->M, g->Kd, g->nops));
       build_tc_image(g->ops, g->M, g->Kd, g->nops, g->img, g->op_scale, s);
     }
+  }
+  DFMM_CUDA(cudaStreamSynchronize(s));
+  P->stats.plan_bytes = (int64_t)P->ar.bytes() + (P->close_keep ? (int64_t)P->close_keep->bytes() : 0);
+}
+
+// Sliced operator images of every translation stage that the form takes; a stage whose
+// image finds no room on the device stays on the CUDA cores.
+void build_slices(dfmm_plan_s* P, cudaStream_t s) {
+  for (const GemmPlan* gc : all_gemms(P)) {
+    GemmPlan* g = const_cast<GemmPlan*>(gc);
+    if (g->npairs == 0 || g->nops == 0 || !gemm_sl_supported(g->M, g->Kd)) continue;
+    try {
+      void* scale = P->ar.alloc<double>(g->nops);
+      void* img = P->ar.alloc<char>(sl_image_bytes(g->M, g->Kd, g->nops, P->fp64));
+      g->sl_scale = scale;
+      g->sl_img = img;
+    } catch (const Error& e) {
+      if (e.code != DFMM_ERR_OOM) throw;
+      cudaGetLastError();
+      continue;
+    }
+    build_sl_image(g->ops, g->M, g->Kd, g->nops, g->sl_img, g->sl_scale, P->fp64, s);
   }
   DFMM_CUDA(cudaStreamSynchronize(s));
   P->stats.plan_bytes = (int64_t)P->ar.bytes() + (P->close_keep ? (int64_t)P->close_keep->bytes() : 0);
@@ -1814,7 +1908,9 @@ int apply_with_scratch(dfmm_plan_s* P, const void* f, void* u, int nrhs, cudaStr
     DFMM_CUDA(cudaGetDevice(&dev));
     if (dev != P->device) return fail(DFMM_ERR_INVALID, "the plan belongs to another device");
     Workspace W;
-    carve_workspace(P, nrhs, (char*)scratch, bytes, stream, W);
+    // the sliced form where the scratch holds its source slices as well
+    const bool slices = P->sliced && (size_t)workspace_bytes(P, nrhs, true) <= bytes;
+    carve_workspace(P, nrhs, (char*)scratch, bytes, stream, W, slices);
     run_apply(P, (const float2*)f, (float2*)u, nrhs, stream, nullptr, &W);
     return DFMM_OK;
   });
@@ -2103,6 +2199,12 @@ int dfmm_plan(const double* points, int64_t N, double K, double eps, const dfmm_
     P->eps = eps;
     P->opt = o;
     P->fp64 = o.arith == 64;
+    // automatic translations below eps 1e-5: the sliced tensor-core form, at least
+    // as precise as the CUDA cores and faster from the smallest stages on (apply,
+    // sphere of 4 wavelengths, eps 1e-6: 0.21 against 0.49 ms; of 32: 3.7 against
+    // 19.5); m2l_mode 1 asks for the CUDA cores, which also serve what the form
+    // does not take
+    P->sliced = o.m2l_mode == 1 && (!opts || opts->m2l_mode == 0);
     P->cw = P->fp64 ? 2 : 1;
     P->stats.arith = o.arith;
     P->eps_op = eps * o.eps_op_factor;
@@ -2115,9 +2217,10 @@ int dfmm_plan(const double* points, int64_t N, double K, double eps, const dfmm_
     DFMM_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     struct SG { cudaStream_t s; ~SG() { cudaStreamDestroy(s); } } sg{s};
     build_plan(P.get(), points, s);
-    if (P->opt.m2l_mode == 2) {
+    if (P->opt.m2l_mode == 2 || P->sliced) {
       const double ti = now();
-      build_images(P.get(), s);
+      if (P->sliced) build_slices(P.get(), s);
+      else build_images(P.get(), s);
       DFMM_CUDA(cudaStreamSynchronize(s));
       P->stats.plan_phase_seconds[6] = now() - ti;
       P->stats.plan_seconds += P->stats.plan_phase_seconds[6];
@@ -2217,7 +2320,7 @@ int dfmm_plan_stats(dfmm_plan_t plan, dfmm_stats* out) {
 int64_t dfmm_apply_workspace_bytes(dfmm_plan_t plan, int nrhs) {
   if (!plan || nrhs < 1 || nrhs > 64) return -1;
   try {
-    return workspace_bytes(plan, nrhs);
+    return workspace_bytes(plan, nrhs, false);
   } catch (...) {
     return -1;
   }
@@ -2236,10 +2339,8 @@ int dfmm_graph_create(dfmm_plan_t plan, const void* f, void* u, int nrhs, cudaSt
     DFMM_CUDA(cudaGetDevice(&dev));
     if (dev != plan->device) return fail(DFMM_ERR_INVALID, "the plan belongs to another device");
     std::unique_ptr<dfmm_graph_s> G(new dfmm_graph_s());
-    G->bytes = (size_t)workspace_bytes(plan, nrhs);
-    G->scratch = G->ar.alloc<char>(G->bytes);
     // work tables are copied in here, outside the capture
-    carve_workspace(plan, nrhs, G->scratch, G->bytes, stream, G->W);
+    own_workspace(plan, nrhs, G->ar, stream, G->W);
     // one ordinary run first: initialises per-kernel launch attributes
     run_apply(plan, (const float2*)f, (float2*)u, nrhs, stream, nullptr, &G->W);
     DFMM_CUDA(cudaStreamSynchronize(stream));
@@ -2336,9 +2437,7 @@ int dfmm_batch_create(const dfmm_plan_t* plans, const void* const* f, void* cons
     // one carved workspace per plan (work tables copied in here, before any capture)
     for (int k = 0; k < count; ++k) {
       std::unique_ptr<Workspace> W(new Workspace());
-      const size_t bytes = (size_t)workspace_bytes(B->plans[k], B->nrhs[k]);
-      char* base = B->ar.alloc<char>((int64_t)bytes);
-      carve_workspace(B->plans[k], B->nrhs[k], base, bytes, stream, *W);
+      own_workspace(B->plans[k], B->nrhs[k], B->ar, stream, *W);
       B->ws.push_back(std::move(W));
     }
     B->status = B->ar.alloc<unsigned>(1);

@@ -34,6 +34,21 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t sbo) {
   return d;
 }
 
+// descriptor of a K-major tile with the 128-byte swizzle: rows of 128 bytes,
+// 8-row groups 1024 B apart, the 16-byte piece p of row r at r * 128 +
+// ((p ^ (r & 7)) << 4); the tile is 1024-byte aligned, saddr may add 32-byte K steps
+__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr) {
+  uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
+  d |= (uint64_t)1u << 16;
+  d |= (uint64_t)(1024u >> 4) << 32;
+  d |= (uint64_t)1u << 46;
+  d |= (uint64_t)2u << 61;
+  return d;
+}
+__host__ __device__ __forceinline__ uint32_t sw128_off(int row, int piece) {
+  return (uint32_t)(row * 128 + ((piece ^ (row & 7)) << 4));
+}
+
 // instruction descriptor, kind::f16: D f32, A and B f16, both K-major,
 // M = 128, N = n; neg_a negates A
 __device__ __forceinline__ uint32_t idesc_f16(int n, bool neg_a = false) {
