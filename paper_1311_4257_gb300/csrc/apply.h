@@ -38,6 +38,9 @@ struct GemmArgs {
 };
 
 void launch_gemm_stage(const GemmArgs& a, cudaStream_t s);
+// The same products in the same order for stages whose operators serve a few
+// columns each (gemm_few.cu); Kd a multiple of 8, tiles of up to 128 columns.
+void launch_gemm_stage_few(const GemmArgs& a, cudaStream_t s);
 
 // One stage of a multi-stage split-complex launch (the batched form runs the
 // same step of several plans in one launch): its tiles carry the stage's index
@@ -81,9 +84,9 @@ void compute_op_scales(const float2* ops, int64_t per_op, int nops, float* scale
 // (build_cx_image) and source rows split into real and imaginary halves
 // (launch_split_cx, rank r = row length in complex values).  Tiles hold up to
 // gemm_cx_columns() columns.
-bool gemm_cx_supported(int M, int Kd);
 int gemm_cx_columns();
 // kind: element type of the split, 0 = FP16, 1 = BF16, 2 = TF32 (4 bytes)
+bool gemm_cx_supported(int M, int Kd);
 int cx_elem_bytes(int kind);
 int64_t cx_image_bytes(int M, int Kd, int nops, int kind);
 void build_cx_image(const float2* ops, int M, int Kd, int nops, void* img, float* scale, int kind, cudaStream_t s);
@@ -97,7 +100,7 @@ void launch_gemm_stage_cx(const GemmArgs& a, const TcArgs& t, unsigned* status, 
 // precision on the FP16 tensor cores, for M, Kd multiples of 8 up to 512 and
 // dense source rows.  src / src_scale: the source buffer's slices
 // (launch_split_sl, sl_row_bytes per row) and per-row scales; img / op_scale:
-// the operator images (build_sl_image).  Scales are float, or double with fp64,
+// the operator images (build_sl_image, from the operators in FP64).  Scales are float, or double with fp64,
 // where every complex array holds complex128.  Tiles hold up to
 // gemm_tc_columns() columns.
 struct SlArgs {
@@ -109,7 +112,7 @@ struct SlArgs {
 bool gemm_sl_supported(int M, int Kd);
 int64_t sl_row_bytes(int r, bool fp64);
 int64_t sl_image_bytes(int M, int Kd, int nops, bool fp64);
-void build_sl_image(const float2* ops, int M, int Kd, int nops, void* img, void* scale, bool fp64, cudaStream_t s);
+void build_sl_image(const double2* ops, int M, int Kd, int nops, void* img, void* scale, bool fp64, cudaStream_t s);
 void launch_split_sl(const float2* x, int64_t rows, int r, void* out, void* scale, bool fp64, cudaStream_t s);
 void launch_gemm_stage_sl(const GemmArgs& a, const SlArgs& t, unsigned* status, bool fp64, cudaStream_t s);
 

@@ -77,6 +77,13 @@ struct GemmPlan {
 
 enum Fam { F_M2L_HF, F_M2L_LF, F_M2M, F_L2L, F_P2L_PROJ, F_P2M_EVAL, F_P2L_EVAL, F_L2P, F_M2P, F_P2P,
            F_PERMUTE, F_ZERO, F_SPLIT, F_COUNT };
+// columns (pairs x right-hand sides) per operator up to which a stage takes the few-column
+// form, on average over its operators: where its time crosses the split form's (3 columns: 13
+// against 26 us with the split of its source, sphere of 2 wavelengths, 40 points, eps 1e-5; 7
+// columns: 29 against 26), and the sliced form's and the CUDA-core stage's (8 columns: 43
+// against 89 and 172 us, eps 1e-6; 27 columns: both 80)
+constexpr int kFewColsSplit = 4, kFewCols = 12;
+
 const char* kFamName[F_COUNT] = {"m2l_hf", "m2l_lf", "m2m", "l2l", "p2l_proj", "p2m_eval",
                                  "p2l_eval", "l2p", "m2p", "p2p", "permute", "zero", "split"};
 
@@ -196,6 +203,7 @@ struct dfmm_plan_s {
   double K = 0, W = 0, eps = 0, eps_op = 0;
   dfmm_options opt{};
   bool fp64 = false;   // FP64 form (options.arith 64): complex128 densities, states and operators
+  bool few = false;    // stages of few columns per operator may run in their own form (gemm_few.cu)
   bool sliced = false; // translations in the sliced tensor-core form (automatic form below eps 1e-5)
   int cw = 1;          // complex element width in float2 units (2 in the FP64 form)
   DevArena ar;
@@ -394,6 +402,20 @@ float2* upload_projection(const std::vector<cd>& Q, int r, int halves, int R, bo
   std::vector<float2> f(h.size());
   for (size_t i = 0; i < h.size(); ++i) f[i] = make_float2((float)h[i].x, (float)h[i].y);
   return upload(f, ar, s);
+}
+
+// Room for the sliced operator images of a stage (m2l_sl.cu), if the plan takes the form
+// and the device has it; a stage without stays on the CUDA cores.
+bool alloc_slices(dfmm_plan_s* P, GemmPlan& g, DevArena& ar) {
+  if (!P->sliced || g.nops == 0 || !gemm_sl_supported(g.M, g.Kd)) return false;
+  try {
+    void* scale = ar.alloc<double>(g.nops);
+    g.sl_img = ar.alloc<char>(sl_image_bytes(g.M, g.Kd, g.nops, P->fp64));
+    g.sl_scale = scale;
+  } catch (const Error& e) {
+    if (e.code != DFMM_ERR_OOM) throw;
+  }
+  return g.sl_img != nullptr;
 }
 
 ChkPt* upload_chk(const std::vector<double>& pts, int n, DevArena& ar, cudaStream_t s) {
@@ -600,10 +622,16 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
   };
   // operator formation on the device (FP64 kernel blocks and products), timed
   // apart within phase 3
-  auto timed_form = [&](OpKind kind, const std::vector<OpSpec>& sp, const std::vector<DevRep>& dr, int Rt, int Rs,
-                        void* out, bool fp64) {
+  auto timed_form = [&](OpKind kind, const std::vector<OpSpec>& sp, const std::vector<DevRep>& dr, GemmPlan& g) {
     const double t = now();
-    form_ops(kind, sp, dr, Rt, Rs, out, fp64, ar, s);
+    OpSink sink;
+    if (alloc_slices(P, g, ar)) {
+      const int64_t per = sl_image_bytes(g.M, g.Kd, 1, P->fp64), sc = P->fp64 ? 8 : 4;
+      sink = [=, &g](const double2* ops, int first, int n) {
+        build_sl_image(ops, g.M, g.Kd, n, (char*)g.sl_img + first * per, (char*)g.sl_scale + first * sc, P->fp64, s);
+      };
+    }
+    form_ops(kind, sp, dr, g.M, g.Kd, g.ops, P->fp64, ar, s, sink);
     ph[7] += now() - t;
   };
   double m2l_flops = 0, other_flops = 0;
@@ -660,6 +688,12 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
       F.p2l.src_rows = F.n_p2l * F.p2l_halves;
       F.p2l.dst_rows = LV[l].n;
       finish_gemm(F.p2l, op, pr, ar, s);
+      if (F.p2l.npairs > 0 && alloc_slices(P, F.p2l, ar)) {
+        ArenaMark mk(ar);
+        const float2* p64 = upload_projection(rp.Qi, rp.r, F.p2l_halves, R, true, ar, s);
+        build_sl_image((const double2*)p64, F.p2l.M, F.p2l.Kd, F.p2l.nops, F.p2l.sl_img, F.p2l.sl_scale, P->fp64, s);
+        DFMM_CUDA(cudaStreamSynchronize(s));
+      }
     }
     // LF-M2L over the V list: one operator per offset
     {
@@ -685,7 +719,7 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
       F.v.M = R; F.v.Kd = R; F.v.nops = (int)specs.size();
       if (!specs.empty()) {
         F.v.ops = ar.alloc<float2>(((size_t)specs.size() * R * R) * P->cw);
-        timed_form(kOpM2L, specs, dreps, R, R, F.v.ops, P->fp64);
+        timed_form(kOpM2L, specs, dreps, F.v);
       }
       F.v.fam = F_M2L_LF;
       F.v.flops_rhs = 8.0 * rp.r * rp.r * V.n;
@@ -709,7 +743,7 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
       (void)C;
       F.m2m.M = R; F.m2m.Kd = Rc; F.m2m.nops = 8;
       F.m2m.ops = ar.alloc<float2>(((size_t)8 * R * Rc) * P->cw);
-      timed_form(kOpM2M, specs, dreps, R, Rc, F.m2m.ops, P->fp64);
+      timed_form(kOpM2M, specs, dreps, F.m2m);
       op.clear(); pr.clear();
       for (int64_t c = 0; c < Lc.n; ++c) {
         op.push_back(octant_of(&Lc.h_coords[3 * c]));
@@ -735,7 +769,7 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
       }
       F.l2l.M = R; F.l2l.Kd = Rp; F.l2l.nops = 8;
       F.l2l.ops = ar.alloc<float2>(((size_t)8 * R * Rp) * P->cw);
-      timed_form(kOpL2L, specs, dreps, R, Rp, F.l2l.ops, P->fp64);
+      timed_form(kOpL2L, specs, dreps, F.l2l);
       op.clear(); pr.clear();
       for (int64_t c = 0; c < LV[l].n; ++c) {
         op.push_back(octant_of(&LV[l].h_coords[3 * c]));
@@ -809,7 +843,7 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
         H.m2l.M = R; H.m2l.Kd = R; H.m2l.nops = (int)specs.size();
         if (!specs.empty()) {
           H.m2l.ops = ar.alloc<float2>(((size_t)specs.size() * R * R) * P->cw);
-          timed_form(kOpM2L, specs, dreps, R, R, H.m2l.ops, P->fp64);
+          timed_form(kOpM2L, specs, dreps, H.m2l);
         }
         H.m2l.src_rows = (int64_t)H.out_keys.size();
         H.m2l.dst_rows = (int64_t)H.in_keys.size();
@@ -835,7 +869,7 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
           }
         H.m2m.M = R; H.m2m.Kd = Rc; H.m2m.nops = (int)specs.size();
         H.m2m.ops = ar.alloc<float2>((std::max<size_t>(1, specs.size()) * R * Rc) * P->cw);
-        timed_form(kOpM2M, specs, dreps, R, Rc, H.m2m.ops, P->fp64);
+        timed_form(kOpM2M, specs, dreps, H.m2m);
         op.clear(); pr.clear();
         for (size_t k = 0; k < H.out_keys.size(); ++k) {
           int b = H.out_keys[k] / H.nd, d = H.out_keys[k] % H.nd;
@@ -877,7 +911,7 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
           }
         H.l2l.M = R; H.l2l.Kd = Hp.R; H.l2l.nops = (int)specs.size();
         H.l2l.ops = ar.alloc<float2>((std::max<size_t>(1, specs.size()) * R * Hp.R) * P->cw);
-        timed_form(kOpL2L, specs, dreps, R, Hp.R, H.l2l.ops, P->fp64);
+        timed_form(kOpL2L, specs, dreps, H.l2l);
         op.clear(); pr.clear();
         for (size_t k = 0; k < Hp.in_keys.size(); ++k) {
           int b = Hp.in_keys[k] / Hp.nd, d = Hp.in_keys[k] % Hp.nd;
@@ -917,7 +951,7 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
         }
       F.l2l.M = F.R; F.l2l.Kd = Hp.R; F.l2l.nops = (int)specs.size();
       F.l2l.ops = ar.alloc<float2>((std::max<size_t>(1, specs.size()) * F.R * Hp.R) * P->cw);
-      timed_form(kOpL2L, specs, dreps, F.R, Hp.R, F.l2l.ops, P->fp64);
+      timed_form(kOpL2L, specs, dreps, F.l2l);
       std::vector<int32_t> op;
       std::vector<int2> pr;
       for (size_t k = 0; k < Hp.in_keys.size(); ++k) {
@@ -1259,6 +1293,12 @@ bool split_complex(const dfmm_plan_s* P, const GemmPlan& g) {
 // where the workspace holds the slices of its source
 bool sliced_stage(const GemmPlan& g) { return g.sl_img != nullptr; }
 
+// whether a stage runs in the few-column form (gemm_few.cu): its operators serve so few
+// columns each that reading them bounds it
+bool few_columns(const dfmm_plan_s* P, const GemmPlan& g, int nrhs) {
+  return P->few && g.npairs * nrhs <= (int64_t)(P->opt.m2l_mode == 2 ? kFewColsSplit : kFewCols) * (int64_t)g.groups.size();
+}
+
 // tile_order: 0 = by the 64 MB rule above, 1 = always by target block, 2 = always by operator.
 // block_bytes: target rows per block in the blocked order (8 MB unless the
 // batched form's autotuner tries another size).
@@ -1361,9 +1401,10 @@ struct Runner {
   void gemm(const GemmPlan& g, const float2* src, int src_ld, int64_t src_rows, float2* dst, int dst_ld,
             int src_key, bool first = false) {
     if (g.npairs == 0) return;
-    const bool tc = on_tensor_cores(P, g);
+    const bool few = few_columns(P, g, nrhs);
+    const bool tc = !few && on_tensor_cores(P, g);
     const bool cx = tc && split_complex(P, g);
-    const bool sl = sliced_stage(g) && (count || W->sl);
+    const bool sl = !few && sliced_stage(g) && (count || W->sl);
     // the split arrays hold one source buffer in one layout (interleaved or split-complex)
     const int key = src_key < 0 ? -1 : 2 * src_key + (cx ? 1 : 0);
     const bool split = (tc || sl) && (key < 0 || key != split_key);
@@ -1375,7 +1416,7 @@ struct Runner {
                                        (first && g.dst_unique) ? 1 : 0});
       return;
     }
-    auto t = tiles_for(P, W, g, nrhs, tc || sl ? gemm_tc_columns() : 64, s);
+    auto t = tiles_for(P, W, g, nrhs, on_tensor_cores(P, g) || (sliced_stage(g) && W->sl) ? gemm_tc_columns() : 64, s);
     GemmArgs a;
     a.ops = g.ops;
     a.M = g.M;
@@ -1410,7 +1451,8 @@ struct Runner {
       launch_gemm_stage_sl(a, SlArgs{W->sl, W->sl_scale, g.sl_img, g.sl_scale}, W->status, P->fp64, s);
     } else {
       ProfScope ps(W, s, g.fam, g.flops_rhs * nrhs, g.bytes_fixed + g.bytes_rhs * nrhs);
-      if (P->fp64) launch_gemm_stage64(a, s);
+      if (few) launch_gemm_stage_few(a, s);
+      else if (P->fp64) launch_gemm_stage64(a, s);
       else launch_gemm_stage(a, s);
     }
   }
@@ -1723,28 +1765,6 @@ void build_images(dfmm_plan_s* P, cudaStream_t s) {
       g->img = P->ar.alloc<__half>(tc_image_elems(g->M, g->Kd, g->nops));
       build_tc_image(g->ops, g->M, g->Kd, g->nops, g->img, g->op_scale, s);
     }
-  }
-  DFMM_CUDA(cudaStreamSynchronize(s));
-  P->stats.plan_bytes = (int64_t)P->ar.bytes() + (P->close_keep ? (int64_t)P->close_keep->bytes() : 0);
-}
-
-// Sliced operator images of every translation stage that the form takes; a stage whose
-// image finds no room on the device stays on the CUDA cores.
-void build_slices(dfmm_plan_s* P, cudaStream_t s) {
-  for (const GemmPlan* gc : all_gemms(P)) {
-    GemmPlan* g = const_cast<GemmPlan*>(gc);
-    if (g->npairs == 0 || g->nops == 0 || !gemm_sl_supported(g->M, g->Kd)) continue;
-    try {
-      void* scale = P->ar.alloc<double>(g->nops);
-      void* img = P->ar.alloc<char>(sl_image_bytes(g->M, g->Kd, g->nops, P->fp64));
-      g->sl_scale = scale;
-      g->sl_img = img;
-    } catch (const Error& e) {
-      if (e.code != DFMM_ERR_OOM) throw;
-      cudaGetLastError();
-      continue;
-    }
-    build_sl_image(g->ops, g->M, g->Kd, g->nops, g->sl_img, g->sl_scale, P->fp64, s);
   }
   DFMM_CUDA(cudaStreamSynchronize(s));
   P->stats.plan_bytes = (int64_t)P->ar.bytes() + (P->close_keep ? (int64_t)P->close_keep->bytes() : 0);
@@ -2204,6 +2224,8 @@ int dfmm_plan(const double* points, int64_t N, double K, double eps, const dfmm_
     // sphere of 4 wavelengths, eps 1e-6: 0.21 against 0.49 ms; of 32: 3.7 against
     // 19.5); m2l_mode 1 asks for the CUDA cores, which also serve what the form
     // does not take
+    // m2l_mode 2 keeps every stage on the tensor cores, wait_test its waits
+    P->few = !P->fp64 && (!opts || opts->m2l_mode != 2) && !o.wait_test;
     P->sliced = o.m2l_mode == 1 && (!opts || opts->m2l_mode == 0);
     P->cw = P->fp64 ? 2 : 1;
     P->stats.arith = o.arith;
@@ -2217,10 +2239,9 @@ int dfmm_plan(const double* points, int64_t N, double K, double eps, const dfmm_
     DFMM_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     struct SG { cudaStream_t s; ~SG() { cudaStreamDestroy(s); } } sg{s};
     build_plan(P.get(), points, s);
-    if (P->opt.m2l_mode == 2 || P->sliced) {
+    if (P->opt.m2l_mode == 2) {
       const double ti = now();
-      if (P->sliced) build_slices(P.get(), s);
-      else build_images(P.get(), s);
+      build_images(P.get(), s);
       DFMM_CUDA(cudaStreamSynchronize(s));
       P->stats.plan_phase_seconds[6] = now() - ti;
       P->stats.plan_seconds += P->stats.plan_phase_seconds[6];

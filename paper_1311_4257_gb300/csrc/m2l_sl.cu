@@ -100,7 +100,7 @@ __device__ __forceinline__ void scale64(uint32_t mhi, double& s, double& inv) {
   inv = __hiloint2double((int)((2046u - e) << 20), 0);
 }
 
-__device__ __forceinline__ void slice(float v, __half* d) {
+__device__ __forceinline__ void slice(float v, __half (&d)[3]) {
   const float t = v * 128.f;
   const float d0 = rintf(t);
   const float r = (t - d0) * 256.f;               // |r| <= 128, exact
@@ -109,7 +109,17 @@ __device__ __forceinline__ void slice(float v, __half* d) {
   d[1] = h1;
   d[2] = __float2half_rn((r - __half2float(h1)) * 256.f);
 }
-__device__ __forceinline__ void slice(double v, __half* d) {
+// an operator's value as formed in FP64, to the same 2^-31: no rounding to FP32 in between
+__device__ __forceinline__ void slice(double v, __half (&d)[3]) {
+  const double t = v * 128.0;
+  const double d0 = rint(t);
+  const double r = (t - d0) * 256.0;
+  const __half h1 = __float2half_rn((float)r);
+  d[0] = __float2half_rn((float)d0);
+  d[1] = h1;
+  d[2] = __float2half_rn((float)((r - (double)__half2float(h1)) * 256.0));
+}
+__device__ __forceinline__ void slice(double v, __half (&d)[8]) {
   constexpr long long kBias = 64ll * (1ll + (1ll << 7) + (1ll << 14) + (1ll << 21) + (1ll << 28) + (1ll << 35) + (1ll << 42));
   const unsigned long long I = (unsigned long long)(__double2ll_rn(v * 36028797018963968.0) + kBias);   // 2^55 v
 #pragma unroll
@@ -175,53 +185,49 @@ __global__ __launch_bounds__(256) void split_sl_kernel(const T2* __restrict__ x,
   }
 }
 
-// scale[op]: a power of two >= the operator's largest magnitude
-template <int S, class T2, class T>
-__global__ __launch_bounds__(256) void op_scale_sl_kernel(const T2* __restrict__ ops, int64_t per_op,
+// scale[op]: a power of two above the largest magnitude of an operator formed in FP64
+template <class T>
+__global__ __launch_bounds__(256) void op_scale_sl_kernel(const double2* __restrict__ ops, int64_t per_op,
                                                           T* __restrict__ scale) {
   __shared__ uint32_t sm;
   if (threadIdx.x == 0) sm = 0;
   __syncthreads();
-  const T2* a = ops + (int64_t)blockIdx.x * per_op;
+  const double2* a = ops + (int64_t)blockIdx.x * per_op;
   uint32_t m = 0;
   for (int64_t q = threadIdx.x; q < per_op; q += blockDim.x) {
-    const T2 v = a[q];
-    uint32_t x, y;
-    if constexpr (S == 3) { x = __float_as_uint(v.x); y = __float_as_uint(v.y); }
-    else { x = (uint32_t)__double2hiint(v.x); y = (uint32_t)__double2hiint(v.y); }
-    m = max(m, max(x & 0x7fffffffu, y & 0x7fffffffu));
+    const double2 v = a[q];
+    m = max(m, max((uint32_t)__double2hiint(v.x) & 0x7fffffffu, (uint32_t)__double2hiint(v.y) & 0x7fffffffu));
   }
   atomicMax(&sm, m);
   __syncthreads();
   if (threadIdx.x == 0) {
-    T s, inv;
-    if constexpr (S == 3) scale32(sm, s, inv);
-    else scale64(sm, s, inv);
-    scale[blockIdx.x] = s;
+    double s, inv;
+    scale64(sm, s, inv);
+    scale[blockIdx.x] = (T)s;
   }
 }
 
 // Operator image [op][block][chunk][Tr, Ti][slice][row of the block][64], zero beyond M
 // and Kd, each row of 128 bytes swizzled as the MMA reads it: a chunk is one
 // bulk copy and the slices of Tr (or Ti) are one stacked operand.  One block per (op, chunk).
-template <int S, class T2, class T>
-__global__ __launch_bounds__(256) void op_image_sl_kernel(const T2* __restrict__ ops, const T* __restrict__ scale,
+template <int S, class T>
+__global__ __launch_bounds__(256) void op_image_sl_kernel(const double2* __restrict__ ops, const T* __restrict__ scale,
                                                           int M, int Kd, unsigned char* __restrict__ img) {
   const int nchunk = (Kd + SL_K - 1) / SL_K, Mp = round16(M), n = block_rows<S>(M);
   const int64_t op = blockIdx.x / nchunk;
   const int c = (int)(blockIdx.x % nchunk);
-  const T2* top = ops + op * (int64_t)M * Kd;
+  const double2* top = ops + op * (int64_t)M * Kd;
   unsigned char* base = img + op * (int64_t)nchunk * 2 * S * SL_ROW * Mp;
-  const T inv = T(1) / scale[op];
+  const double inv = 1.0 / (double)scale[op];
   for (int e = threadIdx.x; e < Mp * 8; e += blockDim.x) {
     const int p = e >> 3, pc = e & 7;
     const int blk = p / n, row = p - blk * n, nb = min(n, Mp - blk * n);
     unsigned char* o = base + (int64_t)blk * n * (nchunk * 2 * S * SL_ROW) + (int64_t)c * (2 * S * SL_ROW * nb);
-    T2 v[8];
+    double2 v[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int q = c * SL_K + 8 * pc + k;
-      v[k] = T2{T(0), T(0)};
+      v[k] = make_double2(0.0, 0.0);
       if (p < M && q < Kd) v[k] = top[(int64_t)p * Kd + q];
     }
 #pragma unroll
@@ -347,13 +353,14 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
     const int kp = round16(a.Kd);
     auto load_rows = [&](int4 tl, int* rows) {
       const int ncol = tl.z * a.nrhs;
+      const uint32_t mg = rhs_magic(a.nrhs);
 #pragma unroll
       for (int q = 0; q < RPT; ++q) {
         const int col = r0 + q * RSTEP;
         rows[q] = -1;
         if (col < ncol) {
-          if (a.nrhs == 1) rows[q] = a.pairs[tl.y + col].x;
-          else rows[q] = a.pairs[tl.y + col / a.nrhs].x * a.nrhs + col % a.nrhs;
+          const int pr = div_rhs(col, mg);
+          rows[q] = a.pairs[tl.y + pr].x * a.nrhs + (col - pr * a.nrhs);
         }
       }
     };
@@ -485,6 +492,7 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
       const int4 tile = a.tiles[it / nblk];
       const int blk = it % nblk, nb = min(n, Mp - blk * n);
       const int ncol = tile.z * a.nrhs;
+      const uint32_t mg = rhs_magic(a.nrhs);
       T* out[4];
       T cs[4];
 #pragma unroll
@@ -493,8 +501,9 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
         out[h] = nullptr;
         cs[h] = T(0);
         if (col < ncol) {
-          const int2 pr = a.pairs[tile.y + col / a.nrhs];
-          const int k = col % a.nrhs;
+          const int q = div_rhs(col, mg);
+          const int2 pr = a.pairs[tile.y + q];
+          const int k = col - q * a.nrhs;
           cs[h] = ((const T*)t.src_scale)[(int64_t)pr.x * a.nrhs + k];
           out[h] = (T*)((T2*)a.dst + ((int64_t)pr.y * a.nrhs + k) * a.dst_ld) + 2 * blk * n + 4 * (lane & 3);
         }
@@ -602,17 +611,17 @@ int64_t sl_row_bytes(int r, bool fp64) { return (int64_t)((r + SL_K - 1) / SL_K)
 
 int64_t sl_image_bytes(int M, int Kd, int nops, bool fp64) { return (int64_t)nops * round16(M) * sl_row_bytes(Kd, fp64); }
 
-void build_sl_image(const float2* ops, int M, int Kd, int nops, void* img, void* scale, bool fp64, cudaStream_t s) {
+void build_sl_image(const double2* ops, int M, int Kd, int nops, void* img, void* scale, bool fp64, cudaStream_t s) {
   if (nops == 0) return;
   if (!gemm_sl_supported(M, Kd)) throw Error(-5, "sliced stage needs ranks that are multiples of 8, <= 512");
   const unsigned blocks = (unsigned)((int64_t)nops * ((Kd + SL_K - 1) / SL_K));
+  unsigned char* p = (unsigned char*)img;
   if (fp64) {
-    const double2* o = (const double2*)ops;
-    op_scale_sl_kernel<8, double2, double><<<nops, 256, 0, s>>>(o, (int64_t)M * Kd, (double*)scale);
-    op_image_sl_kernel<8, double2, double><<<blocks, 256, 0, s>>>(o, (const double*)scale, M, Kd, (unsigned char*)img);
+    op_scale_sl_kernel<<<nops, 256, 0, s>>>(ops, (int64_t)M * Kd, (double*)scale);
+    op_image_sl_kernel<8><<<blocks, 256, 0, s>>>(ops, (const double*)scale, M, Kd, p);
   } else {
-    op_scale_sl_kernel<3, float2, float><<<nops, 256, 0, s>>>(ops, (int64_t)M * Kd, (float*)scale);
-    op_image_sl_kernel<3, float2, float><<<blocks, 256, 0, s>>>(ops, (const float*)scale, M, Kd, (unsigned char*)img);
+    op_scale_sl_kernel<<<nops, 256, 0, s>>>(ops, (int64_t)M * Kd, (float*)scale);
+    op_image_sl_kernel<3><<<blocks, 256, 0, s>>>(ops, (const float*)scale, M, Kd, p);
   }
   DFMM_CUDA(cudaGetLastError());
 }

@@ -141,6 +141,11 @@ __device__ __forceinline__ void tmem_ld16x256_x4(uint32_t ta, uint32_t* r) {
       : "r"(ta));
 }
 
+// column / nrhs for a tile column below 128 and 1 <= nrhs <= 64 by multiplication:
+// exact, since 127 * 63 < 2^16 (a division per gathered row took 3.5k clocks of a 12k-clock tile)
+__device__ __forceinline__ uint32_t rhs_magic(int nrhs) { return (65535u + (uint32_t)nrhs) / (uint32_t)nrhs; }
+__device__ __forceinline__ int div_rhs(int col, uint32_t magic) { return (int)(((uint32_t)col * magic) >> 16); }
+
 // fire-and-forget adds of two / four floats to global memory (no value returned)
 __device__ __forceinline__ void red_add2(float* p, float a, float b) {
   asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
