@@ -91,8 +91,7 @@ typedef struct {
                               or when a leaf has more than 127 near leaves. */
   int32_t tc_layout;       /* [0] tensor-core translations (m2l_mode 2): 0 = split-complex form
                               (Re y = Tr xr - Ti xi, Im y = Ti xr + Tr xi as four real products;
-                              ranks padded to 16) wherever the target rank is at most 128, the
-                              real-block form elsewhere; 1 = the real-block form [[Tr, -Ti],
+                              ranks padded to 16); 1 = the real-block form [[Tr, -Ti],
                               [Ti, Tr]] everywhere (ranks padded to 8). */
   int32_t tc_accumulate;   /* [0] split-complex form: 0 = automatic (1 if eps >= 1e-5, else 2);
                               1 = one tensor-memory accumulator per component, two buffers, so

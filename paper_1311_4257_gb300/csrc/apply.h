@@ -47,8 +47,7 @@ void launch_gemm_stage_few(const GemmArgs& a, cudaStream_t s);
 // in .w; all stages of a launch share M, Kd, dst_ld and the split's element type.
 struct CxStage {
   const int2* pairs;        // (src row, dst row)
-  const void* src_hi;       // split source rows (launch_split_cx)
-  const void* src_lo;
+  const void* src;          // split source rows (launch_split_cx)
   const float* src_scale;
   const void* img;          // operator image (build_cx_image)
   const float* op_scale;
@@ -61,7 +60,8 @@ struct CxStage {
 // must be multiples of 8, source rows dense (src_ld == Kd); tiles hold up to
 // gemm_tc_columns() columns.  img / op_scale: operator image and per-operator
 // power-of-two scales (build_tc_image); src_hi / src_lo / src_scale: the
-// source buffer split by launch_split (one scale per source row).
+// source buffer split by launch_split (one scale per source row); for the
+// split-complex form src_hi is the buffer of launch_split_cx and src_lo is not used.
 struct TcArgs {
   const __half* img;
   const float* op_scale;
@@ -85,12 +85,12 @@ void compute_op_scales(const float2* ops, int64_t per_op, int nops, float* scale
 // (launch_split_cx, rank r = row length in complex values).  Tiles hold up to
 // gemm_cx_columns() columns.
 int gemm_cx_columns();
-// kind: element type of the split, 0 = FP16, 1 = BF16, 2 = TF32 (4 bytes)
-bool gemm_cx_supported(int M, int Kd);
+// kind: element type of the split, 0 = FP16 (target ranks up to 256), 1 = BF16, 2 = TF32 (4 bytes; both up to 128)
+bool gemm_cx_supported(int M, int Kd, int kind);
 int cx_elem_bytes(int kind);
 int64_t cx_image_bytes(int M, int Kd, int nops, int kind);
 void build_cx_image(const float2* ops, int M, int Kd, int nops, void* img, float* scale, int kind, cudaStream_t s);
-void launch_split_cx(const float2* x, int64_t rows, int r, void* hi, void* lo, float* scale, int kind, cudaStream_t s);
+void launch_split_cx(const float2* x, int64_t rows, int r, void* out, float* scale, int kind, cudaStream_t s);
 // one_acc: one accumulator per component, double-buffered tensor memory (faster,
 // the cross terms accumulate with the large terms' truncation)
 void launch_gemm_stage_cx(const GemmArgs& a, const TcArgs& t, unsigned* status, bool one_acc, int kind,

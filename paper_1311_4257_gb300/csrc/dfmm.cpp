@@ -1247,8 +1247,8 @@ Workspace* get_workspace(dfmm_plan_s* P, cudaStream_t s, int nrhs) {
   if (P->opt.m2l_mode == 2) {
     // split arrays: 2 values per complex element, 2 bytes each (4 for the TF32 split)
     int64_t e = max_source_elems(P) * nrhs * 2 * (P->opt.tc_precision == 2 ? 2 : 1);
-    W->ahi = ar.alloc<__half>(e);
-    W->alo = ar.alloc<__half>(e);
+    W->ahi = ar.alloc<__half>(2 * e);   // hi and lo rows; the split-complex form interleaves them
+    W->alo = W->ahi + e;
     W->ascale = ar.alloc<float>(max_source_rows(P) * nrhs);
   }
   if (P->sliced) {
@@ -1280,13 +1280,13 @@ Workspace* get_workspace(dfmm_plan_s* P, cudaStream_t s, int nrhs) {
 bool on_tensor_cores(const dfmm_plan_s* P, const GemmPlan& g) {
   // the BF16 and TF32 splits exist in the split-complex form only: other stages stay on the CUDA cores
   return P->opt.m2l_mode == 2 && gemm_tc_supported(g.M, g.Kd) && (P->opt.tc_stages & kTcFamBit[g.fam]) != 0 &&
-         (P->opt.tc_precision == 0 || gemm_cx_supported(g.M, g.Kd));
+         (P->opt.tc_precision == 0 || gemm_cx_supported(g.M, g.Kd, P->opt.tc_precision));
 }
 
 // whether a tensor-core stage takes the split-complex form (m2l_cx.cu): target
 // rank at most 128 and ranks that are multiples of 16; else the real-block form
 bool split_complex(const dfmm_plan_s* P, const GemmPlan& g) {
-  return on_tensor_cores(P, g) && P->opt.tc_layout != 1 && gemm_cx_supported(g.M, g.Kd);
+  return on_tensor_cores(P, g) && P->opt.tc_layout != 1 && gemm_cx_supported(g.M, g.Kd, P->opt.tc_precision);
 }
 
 // whether a stage has the sliced form (m2l_sl.cu): operators sliced at plan time; it runs so
@@ -1435,7 +1435,7 @@ struct Runner {
     if (tc) {
       if (split) {
         ProfScope ps(W, s, F_SPLIT, 0.0, (double)src_rows * nrhs * src_ld * 16);
-        if (cx) launch_split_cx(src, src_rows * nrhs, src_ld, W->ahi, W->alo, W->ascale, P->opt.tc_precision, s);
+        if (cx) launch_split_cx(src, src_rows * nrhs, src_ld, W->ahi, W->ascale, P->opt.tc_precision, s);
         else launch_split(src, src_rows * nrhs, src_ld, W->ahi, W->alo, W->ascale, s);
       }
       ProfScope ps(W, s, g.fam, g.flops_rhs * nrhs, g.bytes_fixed + g.bytes_rhs * nrhs);
@@ -1697,8 +1697,8 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
   W.p2l = (float2*)take(p2l_rows * nrhs * cb);
   if (P->opt.m2l_mode == 2) {
     size_t e = (size_t)max_source_elems(P) * nrhs * 2 * (P->opt.tc_precision == 2 ? 2 : 1);
-    W.ahi = (__half*)take(e * 2);
-    W.alo = (__half*)take(e * 2);
+    W.ahi = (__half*)take(e * 4);
+    W.alo = W.ahi + e;
     W.ascale = (float*)take((size_t)max_source_rows(P) * nrhs * 4);
   }
   slices = slices && P->sliced;
@@ -2047,8 +2047,7 @@ dfmm_batch_s::Merged& merged_for(dfmm_batch_s* B, int64_t wave, int M, int Kd, i
     const WaveGemm& w = list[i];
     CxStage c;
     c.pairs = w.g->pairs;
-    c.src_hi = w.W->ahi;
-    c.src_lo = w.W->alo;
+    c.src = w.W->ahi;
     c.src_scale = w.W->ascale;
     c.img = w.g->img;
     c.op_scale = w.g->op_scale;
@@ -2106,7 +2105,7 @@ std::pair<int64_t, int64_t> batch_run(dfmm_batch_s* B, cudaStream_t s, int force
       dfmm_batch_s::Merged& m = merged_for(B, wv, sh[0], sh[1], sh[2], sh[3], list, s);
       for (auto& w : list)
         if (w.split) {
-          launch_split_cx(w.src, w.src_rows * w.nrhs, w.src_ld, w.W->ahi, w.W->alo, w.W->ascale,
+          launch_split_cx(w.src, w.src_rows * w.nrhs, w.src_ld, w.W->ahi, w.W->ascale,
                           w.P->opt.tc_precision, s);
           ++launches;
         }
