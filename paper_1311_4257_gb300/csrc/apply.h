@@ -138,6 +138,7 @@ struct P2CArgs {
   int halves;                // FP64 form: 1, or 2: each half of a row's check points is a row of its own,
                              //   out[2 row + half][rhs][ld / 2]
   const float4* pts_lo;      // FP64 form: low parts of the local coordinates
+  const double2* trig;       // FP64 form: build_trig_table
 };
 void launch_p2c(const P2CArgs& a, cudaStream_t s);
 
@@ -199,6 +200,7 @@ struct P2PArgs {
   const int32_t* close_off;  // [N + 1]
   const int32_t* close_j;    // source point of each correction
   const float2* close_w;     // G(p_i, p_j) - (the FP32 form's value for the pair)
+  const double2* trig;       // FP64 form only: build_trig_table
 };
 // Double-float coordinates throughout (any accuracy).
 void launch_p2p(const P2PArgs& a, cudaStream_t s);
@@ -215,6 +217,9 @@ void launch_p2p_close(const P2PArgs& a, float delta, int32_t* cnt, unsigned* deg
 // every complex array (operators, rows, states, densities, potentials)
 // holding complex128 (double2) elements at the same indices.  Representation
 // ranks up to 512; the check-point form needs P2CArgs.chk64 and .pts_lo.
+// trig_table_bytes() bytes of exp(2 pi i k / n), which the kernel evaluations read.
+int trig_table_bytes();
+void build_trig_table(void* t, cudaStream_t s);
 void launch_gemm_stage64(const GemmArgs& a, cudaStream_t s);
 void launch_permute_in64(const float2* f, const int32_t* perm, int64_t N, int nrhs, float2* fs, cudaStream_t s);
 void launch_permute_out64(const float2* us, const int32_t* perm, int64_t N, int nrhs, float2* u, cudaStream_t s);

@@ -233,6 +233,7 @@ struct dfmm_plan_s {
   std::unique_ptr<DevArena> close_keep;   // their storage (allocated after a scratch mark of the plan arena)
   int64_t n_leaves = 0;
   float4* zero_shift = nullptr;
+  double2* trig = nullptr;        // FP64 form: table of the kernel evaluations
   std::unique_ptr<RepSet> reps;
   std::vector<std::array<int64_t, 3>> rep_ranks;   // (level, cell, rank)
   dfmm_stats stats{};
@@ -637,6 +638,10 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
   double m2l_flops = 0, other_flops = 0;
   auto center = [&](int l, int64_t b, int d) { return -0.5 * P->W + (LV[l].h_coords[3 * b + d] + 0.5) * LV[l].w; };
   P->zero_shift = upload(std::vector<float4>{make_float4(0, 0, 0, 0)}, ar, s);
+  if (P->fp64) {
+    P->trig = (double2*)ar.alloc<char>(trig_table_bytes());
+    build_trig_table(P->trig, s);
+  }
 
   phase(2);
   // ---- LF levels
@@ -1577,6 +1582,7 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
         a.nrhs = nrhs;
         a.chk64 = F.chk64;
         a.halves = F.p2l_halves;
+        a.trig = P->trig;
         a.pts_lo = P->pts_lo;
         if (P->fp64) launch_p2c64(a, s);
         else launch_p2c(a, s);
@@ -1634,6 +1640,7 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
     a.close_off = P->close_off;
     a.close_j = P->close_j;
     a.close_w = P->close_w;
+    a.trig = P->trig;
     if (P->fp64) launch_p2p64(a, s);
     else if (P->opt.p2p_mode == 2) launch_p2p_fast(a, N, s);
     else launch_p2p(a, s);
