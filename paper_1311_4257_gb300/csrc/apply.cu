@@ -18,6 +18,7 @@
 //    exact plan-time corrections of the close pairs (p2p_close_kernel,
 //    p2p_close_apply_kernel); p2p_kernel: the same on double-float coordinates.
 #include "apply.h"
+#include "pdl.h"
 
 #include <type_traits>
 
@@ -41,6 +42,7 @@ __device__ __forceinline__ void red_add2(float* p, float a, float b) {
 }
 
 __global__ __launch_bounds__(256) void gemm_stage_kernel(GemmArgs a) {
+  pdl_begin();
   __shared__ float2 As[BK][BM + 1];
   __shared__ float2 Bs[BK][BN + 1];
   __shared__ const float2* srcp[BN];
@@ -115,17 +117,41 @@ __global__ __launch_bounds__(256) void gemm_stage_kernel(GemmArgs a) {
   }
 }
 
-__global__ void permute_in_kernel(const float2* __restrict__ f, const int32_t* __restrict__ perm, int64_t N,
-                                  int nrhs, float2* __restrict__ fs) {
-  int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= N * nrhs) return;
-  int64_t k = e / nrhs;
-  int r = (int)(e % nrhs);
-  fs[e] = f[(int64_t)r * N + perm[k]];
+// Blocks below nperm permute; each of the others clears 16 KB of one of the ranges.  One
+// launch where the memsets of a small apply cost 3 us each.
+constexpr int64_t kZeroChunk = 16384;
+
+template <class T2>
+__global__ __launch_bounds__(256) void permute_in_kernel(const T2* f, const int32_t* perm, int64_t N, int nrhs, T2* fs,
+                                                         int64_t nperm, ZeroRanges z) {
+  pdl_begin();
+  int64_t b = blockIdx.x;
+  if (b < nperm) {
+    if (b == 0 && threadIdx.x == 0 && z.status) *z.status = 0u;
+    const int64_t e = b * 256 + threadIdx.x;
+    if (e >= N * nrhs) return;
+    const int64_t k = e / nrhs;
+    fs[e] = f[(e - k * nrhs) * N + perm[k]];
+    return;
+  }
+  b -= nperm;
+  for (int i = 0; i < z.n; ++i) {
+    const int64_t nb = (z.r[i].bytes + kZeroChunk - 1) / kZeroChunk;
+    if (b < nb) {
+      const int64_t lo = b * kZeroChunk, hi = lo + kZeroChunk < z.r[i].bytes ? lo + kZeroChunk : z.r[i].bytes;
+      char* p = (char*)z.r[i].p;
+      for (int64_t o = lo + 16 * threadIdx.x; o < hi; o += 16 * 256) {
+        if (o + 16 <= hi) *(float4*)(p + o) = make_float4(0.f, 0.f, 0.f, 0.f);
+        else *(float2*)(p + o) = make_float2(0.f, 0.f);
+      }
+      return;
+    }
+    b -= nb;
+  }
 }
 
-__global__ void permute_out_kernel(const float2* __restrict__ us, const int32_t* __restrict__ perm, int64_t N,
-                                   int nrhs, float2* __restrict__ u) {
+__global__ void permute_out_kernel(const float2* us, const int32_t* perm, int64_t N, int nrhs, float2* u) {
+  pdl_begin();
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= N * nrhs) return;
   int64_t k = e / nrhs;
@@ -160,6 +186,7 @@ constexpr int P2C_JOBS = 8;   // rounds of side-by-side jobs per block
 // sides are accumulated per pass.
 template <int NR>
 __global__ __launch_bounds__(P2C_THREADS) void p2c_kernel(P2CArgs a, int tpj) {
+  pdl_begin();
   __shared__ float4 sp[P2C_CHUNK];
   __shared__ float2 sf[P2C_CHUNK][NR];
   const int jp = blockDim.x / tpj;
@@ -233,6 +260,7 @@ __global__ __launch_bounds__(P2C_THREADS) void p2c_kernel(P2CArgs a, int tpj) {
 }
 
 __global__ __launch_bounds__(256) void rows_kernel(RowsArgs a) {
+  pdl_begin();
   const int4 job = a.jobs[blockIdx.x];
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const float2* st = a.state + (int64_t)job.w * a.nrhs * a.R;
@@ -263,8 +291,7 @@ __global__ __launch_bounds__(256) void rows_kernel(RowsArgs a) {
       }
       if (lane == 0) {
         float2* u = a.us + (int64_t)(job.x + i) * a.nrhs + k;
-        if (a.atomic) atomicAdd(u, sum);
-        else { float2 o = *u; *u = make_float2(o.x + sum.x, o.y + sum.y); }
+        red_add2((float*)u, sum.x, sum.y);
       }
     }
   }
@@ -279,6 +306,7 @@ constexpr int L2P_ROWS = 2;
 
 template <int Q>
 __global__ __launch_bounds__(256) void l2p_kernel(L2PArgs a) {
+  pdl_begin();
   const int64_t r0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * L2P_ROWS;
   const int lane = threadIdx.x & 31;
   if (r0 >= a.nrows) return;
@@ -307,7 +335,7 @@ __global__ __launch_bounds__(256) void l2p_kernel(L2PArgs a) {
       for (int t = 0; t < Q; ++t) {
         const int q = lane + 32 * t;
         if (q < R2) {
-          const float4 sv = __ldg(st + (int64_t)k * R2 + q);
+          const float4 sv = st[(int64_t)k * R2 + q];
           acc.x = fmaf(v[j][t].x, sv.x, fmaf(-v[j][t].y, sv.y, acc.x));
           acc.y = fmaf(v[j][t].x, sv.y, fmaf(v[j][t].y, sv.x, acc.y));
           acc.x = fmaf(v[j][t].z, sv.z, fmaf(-v[j][t].w, sv.w, acc.x));
@@ -320,9 +348,7 @@ __global__ __launch_bounds__(256) void l2p_kernel(L2PArgs a) {
         acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
       }
       if (lane == 0) {
-        float2* u = a.us + (int64_t)m[j].x * a.nrhs + k;
-        const float2 o = *u;
-        *u = make_float2(o.x + acc.x, o.y + acc.y);
+        red_add2((float*)(a.us + (int64_t)m[j].x * a.nrhs + k), acc.x, acc.y);   // beside the near field
       }
     }
   }
@@ -337,6 +363,7 @@ __global__ __launch_bounds__(256) void l2p_kernel(L2PArgs a) {
 // (more rows in flight) fit on an SM.
 template <int Q, int KB>
 __global__ __launch_bounds__(256) void p2m_rows_kernel(P2MRowsArgs a) {
+  pdl_begin();
   const int64_t jw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (jw >= a.njobs) return;
@@ -367,7 +394,7 @@ __global__ __launch_bounds__(256) void p2m_rows_kernel(P2MRowsArgs a) {
 #pragma unroll
         for (int kk = 0; kk < KB; ++kk) {
           if (kk >= nk) break;
-          const float2 f = __ldg(a.fs + (int64_t)(job.x + i + j) * a.nrhs + k0 + kk);
+          const float2 f = a.fs[(int64_t)(job.x + i + j) * a.nrhs + k0 + kk];
 #pragma unroll
           for (int t = 0; t < Q; ++t) {
             float4& c = acc[kk][t];
@@ -416,6 +443,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // right-hand sides are accumulated per pass.
 template <int NR>
 __global__ __launch_bounds__(P2P_THREADS) void p2p_kernel(P2PArgs a) {
+  pdl_begin();
   __shared__ float4 syh[P2P_CHUNK];
   __shared__ float4 syl[P2P_CHUNK];
   __shared__ float2 sf[P2P_CHUNK][NR];
@@ -520,9 +548,7 @@ __global__ __launch_bounds__(P2P_THREADS) void p2p_kernel(P2PArgs a) {
             sum.x += v.x;
             sum.y += v.y;
           }
-          float2* uu = a.us + (int64_t)(lr.x + t0 + threadIdx.x) * a.nrhs + r0 + k;
-          float2 o = *uu;
-          *uu = make_float2(o.x + sum.x, o.y + sum.y);
+          red_add2((float*)(a.us + (int64_t)(lr.x + t0 + threadIdx.x) * a.nrhs + r0 + k), sum.x, sum.y);
         }
       }
       __syncthreads();
@@ -569,6 +595,7 @@ __device__ __forceinline__ float4 shifted(float4 v, float4 sh) {
 // pass.
 template <int NR>
 __global__ __launch_bounds__(PF_THREADS) void p2p_fast_kernel(P2PArgs a) {
+  pdl_begin();
   __shared__ float4 sy[PF_CHUNK];
   __shared__ float2 sf[PF_CHUNK][NR];
   __shared__ float2 red[PF_THREADS][2][NR];
@@ -668,6 +695,7 @@ __global__ __launch_bounds__(PF_THREADS) void p2p_fast_kernel(P2PArgs a) {
 // Exact corrections of the close pairs of the FP32 form, one thread per
 // target point: us[i] += sum_c w_c f[j_c].
 __global__ void p2p_close_apply_kernel(P2PArgs a, int64_t npoints) {
+  pdl_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= npoints) return;
   const int c0 = a.close_off[i], c1 = a.close_off[i + 1];
@@ -680,9 +708,7 @@ __global__ void p2p_close_apply_kernel(P2PArgs a, int64_t npoints) {
       sum.x = fmaf(w.x, f.x, fmaf(-w.y, f.y, sum.x));
       sum.y = fmaf(w.x, f.y, fmaf(w.y, f.x, sum.y));
     }
-    float2* uu = a.us + i * a.nrhs + k;
-    const float2 o = *uu;
-    *uu = make_float2(o.x + sum.x, o.y + sum.y);
+    red_add2((float*)(a.us + i * a.nrhs + k), sum.x, sum.y);
   }
 }
 
@@ -732,74 +758,80 @@ __global__ void p2p_close_kernel(P2PArgs a, float delta2, int32_t* cnt, unsigned
 
 }  // namespace
 
-void launch_gemm_stage(const GemmArgs& a, cudaStream_t s) {
+void launch_gemm_stage(const GemmArgs& a, LaunchStream s) {
   if (a.ntiles == 0) return;
   dim3 grid((unsigned)a.ntiles, (unsigned)((a.M + BM - 1) / BM));
-  gemm_stage_kernel<<<grid, 256, 0, s>>>(a);
+  launch_pdl(gemm_stage_kernel, grid, 256, 0, s, a);
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_permute_in(const float2* f, const int32_t* perm, int64_t N, int nrhs, float2* fs, cudaStream_t s) {
+void launch_permute_in(const float2* f, const int32_t* perm, int64_t N, int nrhs, float2* fs, const ZeroRanges& z,
+                       bool fp64, LaunchStream s) {
+  const int64_t nperm = (N * nrhs + 255) / 256;
+  int64_t blocks = nperm;
+  for (int i = 0; i < z.n; ++i) blocks += (z.r[i].bytes + kZeroChunk - 1) / kZeroChunk;
+  if (fp64)
+    launch_pdl(permute_in_kernel<double2>, (unsigned)blocks, 256, 0, s, (const double2*)f, perm, N, nrhs, (double2*)fs, nperm, z);
+  else
+    launch_pdl(permute_in_kernel<float2>, (unsigned)blocks, 256, 0, s, f, perm, N, nrhs, fs, nperm, z);
+  DFMM_CUDA(cudaGetLastError());
+}
+
+void launch_permute_out(const float2* us, const int32_t* perm, int64_t N, int nrhs, float2* u, LaunchStream s) {
   int64_t n = N * nrhs;
-  permute_in_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(f, perm, N, nrhs, fs);
+  launch_pdl(permute_out_kernel, (unsigned)((n + 255) / 256), 256, 0, s, us, perm, N, nrhs, u);
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_permute_out(const float2* us, const int32_t* perm, int64_t N, int nrhs, float2* u, cudaStream_t s) {
-  int64_t n = N * nrhs;
-  permute_out_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(us, perm, N, nrhs, u);
-  DFMM_CUDA(cudaGetLastError());
-}
-
-void launch_p2c(const P2CArgs& a, cudaStream_t s) {
+void launch_p2c(const P2CArgs& a, LaunchStream s) {
   if (a.njobs == 0) return;
   const int tpj = max(32, (min(a.nchk, P2C_THREADS) + 31) / 32 * 32);
   const int jp = P2C_THREADS / tpj;
   const unsigned grid = (unsigned)((a.njobs + (int64_t)jp * P2C_JOBS - 1) / ((int64_t)jp * P2C_JOBS));
-  if (a.nrhs == 1) p2c_kernel<1><<<grid, jp * tpj, 0, s>>>(a, tpj);
-  else if (a.nrhs == 2) p2c_kernel<2><<<grid, jp * tpj, 0, s>>>(a, tpj);
-  else if (a.nrhs <= 4) p2c_kernel<4><<<grid, jp * tpj, 0, s>>>(a, tpj);
-  else p2c_kernel<8><<<grid, jp * tpj, 0, s>>>(a, tpj);
+  if (a.nrhs == 1) launch_pdl(p2c_kernel<1>, grid, jp * tpj, 0, s, a, tpj);
+  else if (a.nrhs == 2) launch_pdl(p2c_kernel<2>, grid, jp * tpj, 0, s, a, tpj);
+  else if (a.nrhs <= 4) launch_pdl(p2c_kernel<4>, grid, jp * tpj, 0, s, a, tpj);
+  else launch_pdl(p2c_kernel<8>, grid, jp * tpj, 0, s, a, tpj);
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_rows(const RowsArgs& a, cudaStream_t s) {
+void launch_rows(const RowsArgs& a, LaunchStream s) {
   if (a.njobs == 0) return;
   if (a.R > 256 || a.R % 2) throw Error(-5, "representation rank must be even and at most 256");
-  rows_kernel<<<(unsigned)a.njobs, 256, 0, s>>>(a);
+  launch_pdl(rows_kernel, (unsigned)a.njobs, 256, 0, s, a);
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_l2p(const L2PArgs& a, cudaStream_t s) {
+void launch_l2p(const L2PArgs& a, LaunchStream s) {
   if (a.nrows == 0) return;
   if (a.R > 256 || a.R % 2) throw Error(-5, "representation rank must be even and at most 256");
   const unsigned grid = (unsigned)((a.nrows + 8 * L2P_ROWS - 1) / (8 * L2P_ROWS));
-  if (a.R <= 128) l2p_kernel<2><<<grid, 256, 0, s>>>(a);
-  else l2p_kernel<4><<<grid, 256, 0, s>>>(a);
+  if (a.R <= 128) launch_pdl(l2p_kernel<2>, grid, 256, 0, s, a);
+  else launch_pdl(l2p_kernel<4>, grid, 256, 0, s, a);
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_p2m_rows(const P2MRowsArgs& a, cudaStream_t s) {
+void launch_p2m_rows(const P2MRowsArgs& a, LaunchStream s) {
   if (a.njobs == 0) return;
   if (a.R > 256 || a.R % 2) throw Error(-5, "representation rank must be even and at most 256");
   const unsigned grid = (unsigned)((a.njobs + 7) / 8);
   if (a.nrhs == 1) {
-    if (a.R <= 128) p2m_rows_kernel<2, 1><<<grid, 256, 0, s>>>(a);
-    else p2m_rows_kernel<4, 1><<<grid, 256, 0, s>>>(a);
+    if (a.R <= 128) launch_pdl(p2m_rows_kernel<2, 1>, grid, 256, 0, s, a);
+    else launch_pdl(p2m_rows_kernel<4, 1>, grid, 256, 0, s, a);
   } else {
-    if (a.R <= 128) p2m_rows_kernel<2, 4><<<grid, 256, 0, s>>>(a);
-    else p2m_rows_kernel<4, 4><<<grid, 256, 0, s>>>(a);
+    if (a.R <= 128) launch_pdl(p2m_rows_kernel<2, 4>, grid, 256, 0, s, a);
+    else launch_pdl(p2m_rows_kernel<4, 4>, grid, 256, 0, s, a);
   }
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_p2p_fast(const P2PArgs& a, int64_t npoints, cudaStream_t s) {
+void launch_p2p_fast(const P2PArgs& a, int64_t npoints, LaunchStream s) {
   if (a.nleaves == 0) return;
-  if (a.nrhs == 1) p2p_fast_kernel<1><<<(unsigned)a.nleaves, PF_THREADS, 0, s>>>(a);
-  else if (a.nrhs == 2) p2p_fast_kernel<2><<<(unsigned)a.nleaves, PF_THREADS, 0, s>>>(a);
-  else p2p_fast_kernel<4><<<(unsigned)a.nleaves, PF_THREADS, 0, s>>>(a);
+  if (a.nrhs == 1) launch_pdl(p2p_fast_kernel<1>, (unsigned)a.nleaves, PF_THREADS, 0, s, a);
+  else if (a.nrhs == 2) launch_pdl(p2p_fast_kernel<2>, (unsigned)a.nleaves, PF_THREADS, 0, s, a);
+  else launch_pdl(p2p_fast_kernel<4>, (unsigned)a.nleaves, PF_THREADS, 0, s, a);
   DFMM_CUDA(cudaGetLastError());
-  p2p_close_apply_kernel<<<(unsigned)((npoints + 255) / 256), 256, 0, s>>>(a, npoints);
+  launch_pdl(p2p_close_apply_kernel, (unsigned)((npoints + 255) / 256), 256, 0, s, a, npoints);
   DFMM_CUDA(cudaGetLastError());
 }
 
@@ -810,11 +842,11 @@ void launch_p2p_close(const P2PArgs& a, float delta, int32_t* cnt, unsigned* deg
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_p2p(const P2PArgs& a, cudaStream_t s) {
+void launch_p2p(const P2PArgs& a, LaunchStream s) {
   if (a.nleaves == 0) return;
-  if (a.nrhs == 1) p2p_kernel<1><<<(unsigned)a.nleaves, P2P_THREADS, 0, s>>>(a);
-  else if (a.nrhs == 2) p2p_kernel<2><<<(unsigned)a.nleaves, P2P_THREADS, 0, s>>>(a);
-  else p2p_kernel<4><<<(unsigned)a.nleaves, P2P_THREADS, 0, s>>>(a);
+  if (a.nrhs == 1) launch_pdl(p2p_kernel<1>, (unsigned)a.nleaves, P2P_THREADS, 0, s, a);
+  else if (a.nrhs == 2) launch_pdl(p2p_kernel<2>, (unsigned)a.nleaves, P2P_THREADS, 0, s, a);
+  else launch_pdl(p2p_kernel<4>, (unsigned)a.nleaves, P2P_THREADS, 0, s, a);
   DFMM_CUDA(cudaGetLastError());
 }
 

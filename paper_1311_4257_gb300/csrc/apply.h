@@ -5,6 +5,7 @@
 #include <cuda_fp16.h>
 
 #include "common.h"
+#include "pdl.h"
 
 namespace dfmm {
 
@@ -37,10 +38,10 @@ struct GemmArgs {
                             //    nullptr: one stage given by the fields above and TcArgs
 };
 
-void launch_gemm_stage(const GemmArgs& a, cudaStream_t s);
+void launch_gemm_stage(const GemmArgs& a, LaunchStream s);
 // The same products in the same order for stages whose operators serve a few
 // columns each (gemm_few.cu); Kd a multiple of 8, tiles of up to 128 columns.
-void launch_gemm_stage_few(const GemmArgs& a, cudaStream_t s);
+void launch_gemm_stage_few(const GemmArgs& a, LaunchStream s);
 
 // One stage of a multi-stage split-complex launch (the batched form runs the
 // same step of several plans in one launch): its tiles carry the stage's index
@@ -69,12 +70,12 @@ struct TcArgs {
   const __half* src_lo;
   const float* src_scale;
 };
-void launch_gemm_stage_tc(const GemmArgs& a, const TcArgs& t, unsigned* status, cudaStream_t s);
+void launch_gemm_stage_tc(const GemmArgs& a, const TcArgs& t, unsigned* status, LaunchStream s);
 int gemm_tc_columns();
 bool gemm_tc_supported(int M, int Kd);
 int64_t tc_image_elems(int M, int Kd, int nops);
 void build_tc_image(const float2* ops, int M, int Kd, int nops, __half* img, float* scale, cudaStream_t s);
-void launch_split(const float2* x, int64_t rows, int ld, __half* hi, __half* lo, float* scale, cudaStream_t s);
+void launch_split(const float2* x, int64_t rows, int ld, __half* hi, __half* lo, float* scale, LaunchStream s);
 // scale[op] = smallest power of two >= max |entry| of operator op (per_op complex entries each)
 void compute_op_scales(const float2* ops, int64_t per_op, int nops, float* scale, cudaStream_t s);
 
@@ -90,11 +91,11 @@ bool gemm_cx_supported(int M, int Kd, int kind);
 int cx_elem_bytes(int kind);
 int64_t cx_image_bytes(int M, int Kd, int nops, int kind);
 void build_cx_image(const float2* ops, int M, int Kd, int nops, void* img, float* scale, int kind, cudaStream_t s);
-void launch_split_cx(const float2* x, int64_t rows, int r, void* out, float* scale, int kind, cudaStream_t s);
+void launch_split_cx(const float2* x, int64_t rows, int r, void* out, float* scale, int kind, LaunchStream s);
 // one_acc: one accumulator per component, double-buffered tensor memory (faster,
 // the cross terms accumulate with the large terms' truncation)
 void launch_gemm_stage_cx(const GemmArgs& a, const TcArgs& t, unsigned* status, bool one_acc, int kind,
-                          cudaStream_t s);
+                          LaunchStream s);
 
 // Sliced tensor-core form (m2l_sl.cu): FP32 or FP64 products without loss of
 // precision on the FP16 tensor cores, for M, Kd multiples of 8 up to 512 and
@@ -113,12 +114,20 @@ bool gemm_sl_supported(int M, int Kd);
 int64_t sl_row_bytes(int r, bool fp64);
 int64_t sl_image_bytes(int M, int Kd, int nops, bool fp64);
 void build_sl_image(const double2* ops, int M, int Kd, int nops, void* img, void* scale, bool fp64, cudaStream_t s);
-void launch_split_sl(const float2* x, int64_t rows, int r, void* out, void* scale, bool fp64, cudaStream_t s);
-void launch_gemm_stage_sl(const GemmArgs& a, const SlArgs& t, unsigned* status, bool fp64, cudaStream_t s);
+void launch_split_sl(const float2* x, int64_t rows, int r, void* out, void* scale, bool fp64, LaunchStream s);
+void launch_gemm_stage_sl(const GemmArgs& a, const SlArgs& t, unsigned* status, bool fp64, LaunchStream s);
 
-// Permutes: fs[k][rhs] = f[rhs][perm[k]];  u[rhs][perm[k]] = us[k][rhs].
-void launch_permute_in(const float2* f, const int32_t* perm, int64_t N, int nrhs, float2* fs, cudaStream_t s);
-void launch_permute_out(const float2* us, const int32_t* perm, int64_t N, int nrhs, float2* u, cudaStream_t s);
+// Permutes: fs[k][rhs] = f[rhs][perm[k]];  u[rhs][perm[k]] = us[k][rhs].  The first also
+// clears z's ranges and the status word (fp64: complex128 at f, fs).
+struct ZeroRanges {
+  static constexpr int kMax = 48;   // two state arrays per level and us
+  struct { void* p; int64_t bytes; } r[kMax];   // 16-byte aligned, whole multiples of 8 bytes
+  int n = 0;
+  unsigned* status = nullptr;       // cleared if set
+};
+void launch_permute_in(const float2* f, const int32_t* perm, int64_t N, int nrhs, float2* fs, const ZeroRanges& z,
+                       bool fp64, LaunchStream s);
+void launch_permute_out(const float2* us, const int32_t* perm, int64_t N, int nrhs, float2* u, LaunchStream s);
 
 // Kernel evaluation from points to check points (P2M, and P2L with the
 // target box's check points): out[row][rhs][p] = sum_i G(c + x_p - y_i) f_i.
@@ -140,7 +149,7 @@ struct P2CArgs {
   const float4* pts_lo;      // FP64 form: low parts of the local coordinates
   const double2* trig;       // FP64 form: build_trig_table
 };
-void launch_p2c(const P2CArgs& a, cudaStream_t s);
+void launch_p2c(const P2CArgs& a, LaunchStream s);
 
 // Rows applied to states: us[i][rhs] += sum_q rows[row_i][q] state[srow][rhs][q].
 struct RowsArgs {
@@ -149,10 +158,9 @@ struct RowsArgs {
   const float2* rows;        // [..][R]
   const float2* state;       // [..][nrhs][R]
   int R, nrhs;
-  float2* us;                // [N][nrhs]
-  int atomic;
+  float2* us;                // [N][nrhs], added to atomically (as by every launch that adds to us)
 };
-void launch_rows(const RowsArgs& a, cudaStream_t s);
+void launch_rows(const RowsArgs& a, LaunchStream s);
 
 // L2P, one warp per point: us[p_r][rhs] += sum_q rows[r][q] state[s_r][rhs][q]
 // for every row r, with (p_r, s_r) = map[r] (each point has one row).
@@ -164,7 +172,7 @@ struct L2PArgs {
   int R, nrhs;               // R even, <= 256
   float2* us;                // [N][nrhs]
 };
-void launch_l2p(const L2PArgs& a, cudaStream_t s);
+void launch_l2p(const L2PArgs& a, LaunchStream s);
 
 // P2M through per-point rows: for every leaf job (first point, count, first
 // row, box) and right-hand side k, state[box][k][q] = sum_i rows[row + i][q]
@@ -177,7 +185,7 @@ struct P2MRowsArgs {
   float2* state;             // [boxes][nrhs][R]
   int R, nrhs;               // R <= 256
 };
-void launch_p2m_rows(const P2MRowsArgs& a, cudaStream_t s);
+void launch_p2m_rows(const P2MRowsArgs& a, LaunchStream s);
 
 // Near field: us[i] += sum over U-list source leaves of G(p_i, p_j) f_j,
 // skipping p_j == p_i.
@@ -203,9 +211,9 @@ struct P2PArgs {
   const double2* trig;       // FP64 form only: build_trig_table
 };
 // Double-float coordinates throughout (any accuracy).
-void launch_p2p(const P2PArgs& a, cudaStream_t s);
+void launch_p2p(const P2PArgs& a, LaunchStream s);
 // FP32 coordinates (high parts) throughout, then the close-pair corrections.
-void launch_p2p_fast(const P2PArgs& a, int64_t npoints, cudaStream_t s);
+void launch_p2p_fast(const P2PArgs& a, int64_t npoints, LaunchStream s);
 // Close pairs of the FP32 form: every (target i, source j) of the U lists with
 // FP32 distance below delta and p_j != p_i.  Pass 1 (off == nullptr): counts per
 // target point into cnt[N], and sets *degenerate if two distinct points have FP32
@@ -220,13 +228,12 @@ void launch_p2p_close(const P2PArgs& a, float delta, int32_t* cnt, unsigned* deg
 // trig_table_bytes() bytes of exp(2 pi i k / n), which the kernel evaluations read.
 int trig_table_bytes();
 void build_trig_table(void* t, cudaStream_t s);
-void launch_gemm_stage64(const GemmArgs& a, cudaStream_t s);
-void launch_permute_in64(const float2* f, const int32_t* perm, int64_t N, int nrhs, float2* fs, cudaStream_t s);
-void launch_permute_out64(const float2* us, const int32_t* perm, int64_t N, int nrhs, float2* u, cudaStream_t s);
-void launch_p2c64(const P2CArgs& a, cudaStream_t s);
-void launch_rows64(const RowsArgs& a, cudaStream_t s);
-void launch_l2p64(const L2PArgs& a, cudaStream_t s);
-void launch_p2m_rows64(const P2MRowsArgs& a, cudaStream_t s);
-void launch_p2p64(const P2PArgs& a, cudaStream_t s);
+void launch_gemm_stage64(const GemmArgs& a, LaunchStream s);
+void launch_permute_out64(const float2* us, const int32_t* perm, int64_t N, int nrhs, float2* u, LaunchStream s);
+void launch_p2c64(const P2CArgs& a, LaunchStream s);
+void launch_rows64(const RowsArgs& a, LaunchStream s);
+void launch_l2p64(const L2PArgs& a, LaunchStream s);
+void launch_p2m_rows64(const P2MRowsArgs& a, LaunchStream s);
+void launch_p2p64(const P2PArgs& a, LaunchStream s);
 
 }  // namespace dfmm

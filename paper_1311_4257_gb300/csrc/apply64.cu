@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "apply.h"
+#include "pdl.h"
 
 namespace dfmm {
 
@@ -83,14 +84,9 @@ __device__ __forceinline__ double3 point64(const float4* hi, const float4* lo, i
                       ((double)h.z + (double)l.z) + (double)sh.z);
 }
 
-__device__ __forceinline__ void add_to(double2* p, double2 v, bool atomic) {
-  if (atomic) {
-    atomicAdd(&p->x, v.x);
-    atomicAdd(&p->y, v.y);
-  } else {
-    const double2 o = *p;
-    *p = make_double2(o.x + v.x, o.y + v.y);
-  }
+__device__ __forceinline__ void add_to(double2* p, double2 v) {
+  atomicAdd(&p->x, v.x);
+  atomicAdd(&p->y, v.y);
 }
 
 // y[dst] += T_op x[src] over a stage's pairs: one CTA computes a 64-row x
@@ -99,6 +95,7 @@ __device__ __forceinline__ void add_to(double2* p, double2 v, bool atomic) {
 constexpr int GM = 64, GN = 64, GK = 8;
 
 __global__ __launch_bounds__(256) void gemm64_kernel(GemmArgs a) {
+  pdl_begin();
   __shared__ double2 As[GK][GM + 1];
   __shared__ double2 Bs[GK][GN + 1];
   __shared__ const double2* srcp[GN];
@@ -160,20 +157,13 @@ __global__ __launch_bounds__(256) void gemm64_kernel(GemmArgs a) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int r = row0 + ty * 4 + i;
-      if (r < a.M) add_to(dstp[c] + r, acc[i][j], true);
+      if (r < a.M) add_to(dstp[c] + r, acc[i][j]);
     }
   }
 }
 
-__global__ void permute_in64_kernel(const double2* __restrict__ f, const int32_t* __restrict__ perm, int64_t N,
-                                    int nrhs, double2* __restrict__ fs) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= N * nrhs) return;
-  fs[e] = f[(e % nrhs) * N + perm[e / nrhs]];
-}
-
-__global__ void permute_out64_kernel(const double2* __restrict__ us, const int32_t* __restrict__ perm, int64_t N,
-                                     int nrhs, double2* __restrict__ u) {
+__global__ void permute_out64_kernel(const double2* us, const int32_t* perm, int64_t N, int nrhs, double2* u) {
+  pdl_begin();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= N * nrhs) return;
   u[(e % nrhs) * N + perm[e / nrhs]] = us[e];
@@ -194,6 +184,7 @@ void by_rhs(int nrhs, F&& f) {
 // shared memory C64_T at a time; padding entries up to ld are written as zeros.
 template <int NR>
 __global__ __launch_bounds__(C64_T) void p2c64_kernel(P2CArgs a) {
+  pdl_begin();
   __shared__ double3 sp[C64_T];
   __shared__ double2 sf[C64_T][NR];
   __shared__ double2 trig[kTrig];
@@ -266,8 +257,7 @@ __device__ __forceinline__ double warp_sums(double (&v)[N]) {
 constexpr int R64_MAX = 512;         // largest rank of the FP64 row kernels
 
 template <int NR>
-__device__ __forceinline__ void row_dot(const double2* row, const double2* st, int R, int nrhs, double2* u,
-                                        bool atomic) {
+__device__ __forceinline__ void row_dot(const double2* row, const double2* st, int R, int nrhs, double2* u) {
   const int lane = threadIdx.x & 31;
   for (int k0 = 0; k0 < nrhs; k0 += NR) {
     double2 sum[NR];
@@ -286,31 +276,28 @@ __device__ __forceinline__ void row_dot(const double2* row, const double2* st, i
     for (int k = 0; k < NR; ++k) { v[2 * k] = sum[k].x; v[2 * k + 1] = sum[k].y; }
     const double t = warp_sums<2 * NR>(v);
     const int slot = warp_slot<2 * NR>();
-    if (lane % (16 / NR) == 0 && k0 + (slot >> 1) < nrhs) {
-      double* p = (double*)(u + k0) + slot;
-      if (atomic) atomicAdd(p, t);
-      else *p += t;
-    }
+    if (lane % (16 / NR) == 0 && k0 + (slot >> 1) < nrhs) atomicAdd((double*)(u + k0) + slot, t);
   }
 }
 
 template <int NR>
 __global__ __launch_bounds__(256) void rows64_kernel(RowsArgs a) {
+  pdl_begin();
   const int4 job = a.jobs[blockIdx.x];
   const int warp = threadIdx.x / 32;
   const double2* st = c128(a.state) + (int64_t)job.w * a.nrhs * a.R;
   for (int i = warp; i < job.y; i += 8)
-    row_dot<NR>(c128(a.rows) + (int64_t)(job.z + i) * a.R, st, a.R, a.nrhs, c128(a.us) + (int64_t)(job.x + i) * a.nrhs,
-                a.atomic != 0);
+    row_dot<NR>(c128(a.rows) + (int64_t)(job.z + i) * a.R, st, a.R, a.nrhs, c128(a.us) + (int64_t)(job.x + i) * a.nrhs);
 }
 
 template <int NR>
 __global__ __launch_bounds__(256) void l2p64_kernel(L2PArgs a) {
+  pdl_begin();
   const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (r >= a.nrows) return;
   const int2 m = a.map[r];
   row_dot<NR>(c128(a.rows) + r * a.R, c128(a.state) + (int64_t)m.y * a.nrhs * a.R, a.R, a.nrhs,
-              c128(a.us) + (int64_t)m.x * a.nrhs, false);
+              c128(a.us) + (int64_t)m.x * a.nrhs);
 }
 
 // P2M through rows: state[box][k][q] = sum_i rows[row + i][q] fs[first + i][k].  One
@@ -319,6 +306,7 @@ __global__ __launch_bounds__(256) void l2p64_kernel(L2PArgs a) {
 // small bodies two warps per SM).
 template <int NR>
 __global__ __launch_bounds__(C64_T) void p2m64_kernel(P2MRowsArgs a) {
+  pdl_begin();
   const int4 job = a.jobs[blockIdx.x];
   const int q = blockIdx.y * C64_T + threadIdx.x;
   if (q >= a.R) return;
@@ -357,6 +345,7 @@ __global__ __launch_bounds__(C64_T) void p2m64_kernel(P2MRowsArgs a) {
 // added at the end, so that a leaf of a dozen points fills the block.
 template <int NR>
 __global__ __launch_bounds__(C64_T) void p2p64_kernel(P2PArgs a) {
+  pdl_begin();
   __shared__ double3 sp[C64_T];
   __shared__ double2 sf[C64_T][NR];
   __shared__ double2 red[C64_T][NR];
@@ -419,7 +408,7 @@ __global__ __launch_bounds__(C64_T) void p2p64_kernel(P2PArgs a) {
             sum.x += v.x;
             sum.y += v.y;
           }
-          add_to(us + (int64_t)(lr.x + t0 + threadIdx.x) * a.nrhs + r0 + k, sum, gridDim.y > 1);
+          add_to(us + (int64_t)(lr.x + t0 + threadIdx.x) * a.nrhs + r0 + k, sum);
         }
     }
   }
@@ -431,10 +420,10 @@ void check_rank(int R) {
 
 }  // namespace
 
-void launch_gemm_stage64(const GemmArgs& a, cudaStream_t s) {
+void launch_gemm_stage64(const GemmArgs& a, LaunchStream s) {
   if (a.ntiles == 0) return;
   const dim3 grid((unsigned)a.ntiles, (unsigned)((a.M + GM - 1) / GM));
-  gemm64_kernel<<<grid, 256, 0, s>>>(a);
+  launch_pdl(gemm64_kernel, grid, 256, 0, s, a);
   DFMM_CUDA(cudaGetLastError());
 }
 
@@ -445,53 +434,47 @@ void build_trig_table(void* t, cudaStream_t s) {
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_permute_in64(const float2* f, const int32_t* perm, int64_t N, int nrhs, float2* fs, cudaStream_t s) {
+void launch_permute_out64(const float2* us, const int32_t* perm, int64_t N, int nrhs, float2* u, LaunchStream s) {
   const int64_t n = N * nrhs;
-  permute_in64_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const double2*)f, perm, N, nrhs, (double2*)fs);
+  launch_pdl(permute_out64_kernel, (unsigned)((n + 255) / 256), 256, 0, s, (const double2*)us, perm, N, nrhs, (double2*)u);
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_permute_out64(const float2* us, const int32_t* perm, int64_t N, int nrhs, float2* u, cudaStream_t s) {
-  const int64_t n = N * nrhs;
-  permute_out64_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const double2*)us, perm, N, nrhs, (double2*)u);
-  DFMM_CUDA(cudaGetLastError());
-}
-
-void launch_p2c64(const P2CArgs& a, cudaStream_t s) {
+void launch_p2c64(const P2CArgs& a, LaunchStream s) {
   if (a.njobs == 0) return;
   if (!a.chk64 || !a.pts_lo || !a.trig) throw Error(-5, "FP64 check-point evaluation needs FP64 check points");
   const dim3 grid((unsigned)a.njobs, (unsigned)((a.ld + C64_T - 1) / C64_T));
-  by_rhs(a.nrhs, [&](auto nr) { p2c64_kernel<nr()><<<grid, C64_T, 0, s>>>(a); });
+  by_rhs(a.nrhs, [&](auto nr) { launch_pdl(p2c64_kernel<nr()>, grid, C64_T, 0, s, a); });
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_rows64(const RowsArgs& a, cudaStream_t s) {
+void launch_rows64(const RowsArgs& a, LaunchStream s) {
   if (a.njobs == 0) return;
   check_rank(a.R);
-  by_rhs(a.nrhs, [&](auto nr) { rows64_kernel<nr()><<<(unsigned)a.njobs, 256, 0, s>>>(a); });
+  by_rhs(a.nrhs, [&](auto nr) { launch_pdl(rows64_kernel<nr()>, (unsigned)a.njobs, 256, 0, s, a); });
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_l2p64(const L2PArgs& a, cudaStream_t s) {
+void launch_l2p64(const L2PArgs& a, LaunchStream s) {
   if (a.nrows == 0) return;
   check_rank(a.R);
-  by_rhs(a.nrhs, [&](auto nr) { l2p64_kernel<nr()><<<(unsigned)((a.nrows + 7) / 8), 256, 0, s>>>(a); });
+  by_rhs(a.nrhs, [&](auto nr) { launch_pdl(l2p64_kernel<nr()>, (unsigned)((a.nrows + 7) / 8), 256, 0, s, a); });
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_p2m_rows64(const P2MRowsArgs& a, cudaStream_t s) {
+void launch_p2m_rows64(const P2MRowsArgs& a, LaunchStream s) {
   if (a.njobs == 0) return;
   check_rank(a.R);
   const dim3 grid((unsigned)a.njobs, (unsigned)((a.R + C64_T - 1) / C64_T));
-  by_rhs(a.nrhs, [&](auto nr) { p2m64_kernel<nr()><<<grid, C64_T, 0, s>>>(a); });
+  by_rhs(a.nrhs, [&](auto nr) { launch_pdl(p2m64_kernel<nr()>, grid, C64_T, 0, s, a); });
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_p2p64(const P2PArgs& a, cudaStream_t s) {
+void launch_p2p64(const P2PArgs& a, LaunchStream s) {
   if (a.nleaves == 0) return;
   // enough blocks for the SMs to even out: four per leaf where the leaves alone are few
   const dim3 grid((unsigned)a.nleaves, a.nleaves < 152 * 32 ? 4u : 1u);
-  by_rhs(a.nrhs, [&](auto nr) { p2p64_kernel<nr()><<<grid, C64_T, 0, s>>>(a); });
+  by_rhs(a.nrhs, [&](auto nr) { launch_pdl(p2p64_kernel<nr()>, grid, C64_T, 0, s, a); });
   DFMM_CUDA(cudaGetLastError());
 }
 

@@ -77,6 +77,13 @@ struct GemmPlan {
 
 enum Fam { F_M2L_HF, F_M2L_LF, F_M2M, F_L2L, F_P2L_PROJ, F_P2M_EVAL, F_P2L_EVAL, F_L2P, F_M2P, F_P2P,
            F_PERMUTE, F_ZERO, F_SPLIT, F_COUNT };
+// Bytes up to which the first launch clears what the apply adds into (sphere of 32 wavelengths,
+// 140 MB: 1.35 against 1.36 ms with memsets; torus of 40, 3 right-hand sides, 210 MB: 1.68
+// against 1.66), points x right-hand sides up to which the near field runs beside the far field
+// (sphere of 16, 80,000: 380 against 397 us; of 24, 181,000: 856 both ways), and up to which
+// kernels are placed early (pdl.h).
+constexpr int64_t kFusedZero = 160 << 20, kBesideNear = 200000, kEarlyLaunch = 1000000;
+
 // columns (pairs x right-hand sides) per operator up to which a stage takes the few-column
 // form, on average over its operators: where its time crosses the split form's (3 columns: 13
 // against 26 us with the split of its source, sphere of 2 wavelengths, 40 points, eps 1e-5; 7
@@ -150,7 +157,8 @@ struct Workspace {
   std::vector<float2*> S, T;                            // per level (LF or HF states)
   std::vector<std::pair<void*, size_t>> zero;           // reset before each apply
   std::vector<std::pair<void*, size_t>> zero_late;      // reset on the side stream, first read by HF M2M
-  cudaStream_t side = nullptr;                          // for zero_late, beside P2M and the V list
+  cudaStream_t side = nullptr;                          // for zero_late, beside P2M and the V list, or the near field
+  bool may_fork = false;                                // the workspace lives on, so it may own the side stream
   cudaEvent_t fork = nullptr, join = nullptr;
   std::map<std::pair<const void*, int>, std::pair<int4*, int64_t>> tiles;   // key (stage, nrhs * 1024 + columns)
   float2 *f_dev = nullptr, *u_dev = nullptr;            // staging for host applies
@@ -1222,6 +1230,7 @@ Workspace* get_workspace(dfmm_plan_s* P, cudaStream_t s, int nrhs) {
   slot.reset(new Workspace());
   Workspace* W = slot.get();
   W->nrhs = nrhs;
+  W->may_fork = true;
   DevArena& ar = W->ar;
   const int64_t N = P->N;
   const int64_t cw = P->cw;   // float2 units per complex element
@@ -1369,7 +1378,7 @@ struct WaveCtl {
 struct Runner {
   dfmm_plan_s* P;
   Workspace* W;
-  cudaStream_t s;
+  LaunchStream s;
   int nrhs;
   int64_t* count;   // dry run: count launches only
   WaveCtl* ctl = nullptr;
@@ -1480,9 +1489,10 @@ inline int64_t wave_lf_down(int64_t lw, int k) { return 5000 + (64 - lw) * 8 + k
 inline int64_t wave_l2p(int64_t lw) { return 6000 + (64 - lw); }
 constexpr int64_t kWaveM2P = 6500, kWaveP2P = 7000, kWaveEnd = 8000;
 
-void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_t s, int64_t* count = nullptr,
+void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_t stream, int64_t* count = nullptr,
                Workspace* ext = nullptr, WaveCtl* ctl = nullptr) {
-  Workspace* W = count ? nullptr : (ext ? ext : get_workspace(P, s, nrhs));
+  Workspace* W = count ? nullptr : (ext ? ext : get_workspace(P, stream, nrhs));
+  const LaunchStream s(stream, P->N * nrhs <= kEarlyLaunch);
   Runner R{P, W, s, nrhs, count};
   R.ctl = ctl;
   const int64_t lW = (int64_t)std::llround(std::log2(P->W));
@@ -1491,8 +1501,21 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
   const int nl = P->nl;
   auto S = [&](int l) { return count ? (float2*)nullptr : W->S[l]; };
   auto T = [&](int l) { return count ? (float2*)nullptr : W->T[l]; };
-  const bool late = !count && !ctl && !W->zero_late.empty();
-  if (late) {   // HF states: reset on a side stream while P2M and the V list run
+  // What the apply adds into is cleared first: by the first launch where that is little, else by
+  // memsets, those of the HF states on a side stream while P2M and the V list run.
+  ZeroRanges z;
+  int64_t zbytes = 0;
+  if (!count)
+    for (auto* list : {&W->zero, &W->zero_late})
+      for (auto& r : *list) {
+        if (r.first == W->status) { z.status = W->status; continue; }
+        if (z.n < ZeroRanges::kMax) { z.r[z.n].p = r.first; z.r[z.n].bytes = (int64_t)r.second; }
+        ++z.n;
+        zbytes += (int64_t)r.second;
+      }
+  const bool fused = zbytes <= kFusedZero && z.n <= ZeroRanges::kMax;
+  const bool late = !count && !ctl && !fused && !W->zero_late.empty();
+  auto fork_side = [&] {
     if (!W->side) {
       DFMM_CUDA(cudaStreamCreateWithFlags(&W->side, cudaStreamNonBlocking));
       DFMM_CUDA(cudaEventCreateWithFlags(&W->fork, cudaEventDisableTiming));
@@ -1500,19 +1523,51 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
     }
     DFMM_CUDA(cudaEventRecord(W->fork, s));
     DFMM_CUDA(cudaStreamWaitEvent(W->side, W->fork, 0));
-    for (auto& z : W->zero_late) DFMM_CUDA(cudaMemsetAsync(z.first, 0, z.second, W->side));
+  };
+  if (late) {
+    fork_side();
+    for (auto& r : W->zero_late) DFMM_CUDA(cudaMemsetAsync(r.first, 0, r.second, W->side));
     DFMM_CUDA(cudaEventRecord(W->join, W->side));
   }
-  if (!count && !R.at(kWaveStart).skip()) {
+  if (!count && !fused && !R.at(kWaveStart).skip()) {
     ProfScope ps(W, s, F_ZERO, 0.0, 0.0);
-    for (auto& z : W->zero) DFMM_CUDA(cudaMemsetAsync(z.first, 0, z.second, s));
+    for (auto& r : W->zero) DFMM_CUDA(cudaMemsetAsync(r.first, 0, r.second, s));
     if (ctl)   // the batched form resets every state in line
-      for (auto& z : W->zero_late) DFMM_CUDA(cudaMemsetAsync(z.first, 0, z.second, s));
+      for (auto& r : W->zero_late) DFMM_CUDA(cudaMemsetAsync(r.first, 0, r.second, s));
   }
-  R.at(kWaveStart).launch(F_PERMUTE, 0.0, 20.0 * N * nrhs, [&] {
-    if (P->fp64) launch_permute_in64(f, P->perm, N, nrhs, W->fs, s);
-    else launch_permute_in(f, P->perm, N, nrhs, W->fs, s);
-  });
+  if (!fused) {
+    z.n = 0;
+    z.status = nullptr;
+  }
+  R.at(kWaveStart).launch(F_PERMUTE, 0.0, 20.0 * N * nrhs, [&] { launch_permute_in(f, P->perm, N, nrhs, W->fs, z, P->fp64, s); });
+  auto near_field = [&](cudaStream_t st) {
+    P2PArgs a;
+    a.leaf_range = P->p2p_range;
+    a.nleaves = P->n_leaves;
+    a.u_off = P->p2p_off;
+    a.u_src = P->p2p_src;
+    a.u_shift = P->p2p_shift;
+    a.flat = P->p2p_flat;
+    a.pts = P->pts_local;
+    a.pts_lo = P->pts_lo;
+    a.fs = W->fs;
+    a.us = W->us;
+    a.nrhs = nrhs;
+    a.close_off = P->close_off;
+    a.close_j = P->close_j;
+    a.close_w = P->close_w;
+    a.trig = P->trig;
+    if (P->fp64) launch_p2p64(a, st);
+    else if (P->opt.p2p_mode == 2) launch_p2p_fast(a, N, st);
+    else launch_p2p(a, st);
+  };
+  // a small apply leaves the device half empty: its near field runs beside the far field
+  const bool beside = !count && !ctl && fused && W->may_fork && !W->prof && N * nrhs <= kBesideNear;
+  if (beside) {
+    fork_side();
+    near_field(W->side);
+    DFMM_CUDA(cudaEventRecord(W->join, W->side));
+  }
   // 1. LF upward: P2M at leaves, LF-M2M from the level below
   for (int l = nl - 1; l >= P->l_lf0; --l) {
     LFLevel& F = P->lf[l];
@@ -1618,33 +1673,15 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
       a.R = g.R;
       a.nrhs = nrhs;
       a.us = W->us;
-      a.atomic = 1;
       if (P->fp64) launch_rows64(a, s);
       else launch_rows(a, s);
     });
   }
   // 6. near field
-  R.at(kWaveP2P).launch(F_P2P, (double)P->stats.p2p_interactions * (16.0 + 8.0 * nrhs), (double)N * (32.0 + 24.0 * nrhs), [&] {
-    P2PArgs a;
-    a.leaf_range = P->p2p_range;
-    a.nleaves = P->n_leaves;
-    a.u_off = P->p2p_off;
-    a.u_src = P->p2p_src;
-    a.u_shift = P->p2p_shift;
-    a.flat = P->p2p_flat;
-    a.pts = P->pts_local;
-    a.pts_lo = P->pts_lo;
-    a.fs = W->fs;
-    a.us = W->us;
-    a.nrhs = nrhs;
-    a.close_off = P->close_off;
-    a.close_j = P->close_j;
-    a.close_w = P->close_w;
-    a.trig = P->trig;
-    if (P->fp64) launch_p2p64(a, s);
-    else if (P->opt.p2p_mode == 2) launch_p2p_fast(a, N, s);
-    else launch_p2p(a, s);
-  });
+  if (beside) DFMM_CUDA(cudaStreamWaitEvent(s, W->join, 0));
+  else
+    R.at(kWaveP2P).launch(F_P2P, (double)P->stats.p2p_interactions * (16.0 + 8.0 * nrhs),
+                          (double)N * (32.0 + 24.0 * nrhs), [&] { near_field(s); });
   R.at(kWaveEnd).launch(F_PERMUTE, 0.0, 20.0 * N * nrhs, [&] {
     if (P->fp64) launch_permute_out64(W->us, P->perm, N, nrhs, u, s);
     else launch_permute_out(W->us, P->perm, N, nrhs, u, s);
@@ -2368,6 +2405,7 @@ int dfmm_graph_create(dfmm_plan_t plan, const void* f, void* u, int nrhs, cudaSt
     std::unique_ptr<dfmm_graph_s> G(new dfmm_graph_s());
     // work tables are copied in here, outside the capture
     own_workspace(plan, nrhs, G->ar, stream, G->W);
+    G->W.may_fork = true;
     // one ordinary run first: initialises per-kernel launch attributes
     run_apply(plan, (const float2*)f, (float2*)u, nrhs, stream, nullptr, &G->W);
     DFMM_CUDA(cudaStreamSynchronize(stream));

@@ -10,6 +10,7 @@
 // in the order of the CUDA-core stage kernel (gemm_stage_kernel): the result is
 // its to the bit, up to the order of the additions to dst.
 #include "apply.h"
+#include "pdl.h"
 #include "tcgen05.cuh"
 
 namespace dfmm {
@@ -43,6 +44,7 @@ __device__ __forceinline__ void chunk(const unsigned char* ar, const unsigned ch
 }
 
 __global__ __launch_bounds__(FW_THREADS) void gemm_few_kernel(GemmArgs a) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x;
   const int4 tile = a.tiles[blockIdx.x];
@@ -112,11 +114,11 @@ __global__ __launch_bounds__(FW_THREADS) void gemm_few_kernel(GemmArgs a) {
 
 }  // namespace
 
-void launch_gemm_stage_few(const GemmArgs& a, cudaStream_t s) {
+void launch_gemm_stage_few(const GemmArgs& a, LaunchStream s) {
   if (a.ntiles == 0) return;
   if (a.Kd % 8 || a.src_ld % 2) throw Error(-5, "few-column stage needs source ranks that are multiples of 8");
   const dim3 grid((unsigned)a.ntiles, (unsigned)((a.M + FW_ROWS - 1) / FW_ROWS));
-  gemm_few_kernel<<<grid, FW_THREADS, FW_SMEM, s>>>(a);
+  launch_pdl(gemm_few_kernel, grid, FW_THREADS, FW_SMEM, s, a);
   DFMM_CUDA(cudaGetLastError());
 }
 

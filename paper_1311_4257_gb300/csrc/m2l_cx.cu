@@ -57,6 +57,7 @@
 #include <algorithm>
 
 #include "apply.h"
+#include "pdl.h"
 #include "tcgen05.cuh"
 
 namespace dfmm {
@@ -148,8 +149,8 @@ template <class T> __device__ __forceinline__ void store4(unsigned char* o, cons
 // long as what is left; a row takes 8 r bytes, 16 r for TF32).  One warp per row, four complex
 // values per lane and step.
 template <int KIND>
-__global__ __launch_bounds__(256) void split_cx_kernel(const float* __restrict__ x, int64_t rows, int r,
-                                                       unsigned char* __restrict__ out, float* __restrict__ scale) {
+__global__ __launch_bounds__(256) void split_cx_kernel(const float* x, int64_t rows, int r, unsigned char* out, float* scale) {
+  pdl_begin();
   using E = Elem<KIND>;
   using T = typename E::T;
   constexpr int EB = elem_bytes<KIND>(), BKE = seg_elems<KIND>();
@@ -273,6 +274,7 @@ struct CxRing {   // position in a ring of shared-memory slots, and the parity o
 
 template <int KIND, bool ONE>
 __global__ __launch_bounds__(CX_THREADS, 1) void gemm_cx_kernel(GemmArgs a, TcArgs t, int nblk, unsigned* status) {
+  pdl_begin();
   constexpr int EB = elem_bytes<KIND>(), BKE = seg_elems<KIND>(), KSTEP = kstep_elems<KIND>();
   constexpr int RSTEP = CX_PRODUCERS / 8, RPT = CX_M / RSTEP;
   extern __shared__ unsigned char smem_raw[];
@@ -614,20 +616,20 @@ void build_cx_image(const float2* ops, int M, int Kd, int nops, void* img, float
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_split_cx(const float2* x, int64_t rows, int r, void* out, float* scale, int kind, cudaStream_t s) {
+void launch_split_cx(const float2* x, int64_t rows, int r, void* out, float* scale, int kind, LaunchStream s) {
   if (rows == 0) return;
   if (r % 16) throw Error(-5, "split-complex source rows need a rank that is a multiple of 16");
   const unsigned grid = (unsigned)((rows * 32 + 255) / 256);
   const float* xf = (const float*)x;
   unsigned char* o = (unsigned char*)out;
-  if (kind == 0) split_cx_kernel<0><<<grid, 256, 0, s>>>(xf, rows, r, o, scale);
-  else if (kind == 1) split_cx_kernel<1><<<grid, 256, 0, s>>>(xf, rows, r, o, scale);
-  else split_cx_kernel<2><<<grid, 256, 0, s>>>(xf, rows, r, o, scale);
+  if (kind == 0) launch_pdl(split_cx_kernel<0>, grid, 256, 0, s, xf, rows, r, o, scale);
+  else if (kind == 1) launch_pdl(split_cx_kernel<1>, grid, 256, 0, s, xf, rows, r, o, scale);
+  else launch_pdl(split_cx_kernel<2>, grid, 256, 0, s, xf, rows, r, o, scale);
   DFMM_CUDA(cudaGetLastError());
 }
 
 template <int KIND, bool ONE>
-void launch_cx(const GemmArgs& a, const TcArgs& t, int nblk, unsigned* status, unsigned grid, cudaStream_t s) {
+void launch_cx(const GemmArgs& a, const TcArgs& t, int nblk, unsigned* status, unsigned grid, LaunchStream s) {
   static bool attr[64] = {false};
   int dev = 0;
   DFMM_CUDA(cudaGetDevice(&dev));
@@ -636,11 +638,11 @@ void launch_cx(const GemmArgs& a, const TcArgs& t, int nblk, unsigned* status, u
     DFMM_CUDA(cudaFuncSetAttribute(gemm_cx_kernel<KIND, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, CX_SMEM));
     attr[dev] = true;
   }
-  gemm_cx_kernel<KIND, ONE><<<grid, CX_THREADS, CX_SMEM, s>>>(a, t, nblk, status);
+  launch_pdl(gemm_cx_kernel<KIND, ONE>, grid, CX_THREADS, CX_SMEM, s, a, t, nblk, status);
 }
 
 void launch_gemm_stage_cx(const GemmArgs& a, const TcArgs& t, unsigned* status, bool one_acc, int kind,
-                          cudaStream_t s) {
+                          LaunchStream s) {
   if (a.ntiles == 0) return;
   if (!gemm_cx_supported(a.M, a.Kd, kind) || a.src_ld != a.Kd)
     throw Error(-5, "split-complex stage needs ranks that are multiples of 16, <= 256, and dense source rows");

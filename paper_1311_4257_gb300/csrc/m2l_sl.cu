@@ -44,6 +44,7 @@
 #include <algorithm>
 
 #include "apply.h"
+#include "pdl.h"
 #include "tcgen05.cuh"
 
 namespace dfmm {
@@ -145,8 +146,8 @@ __device__ __forceinline__ void store_pieces(unsigned char* out, const __half (*
 // multiple of 16 with zeros; what is left of the last chunk is not read), one scale per row.  One warp per row; a lane takes 8
 // complex values, i.e. one 16-byte piece of every slice.
 template <int S, class T2, class T>
-__global__ __launch_bounds__(256) void split_sl_kernel(const T2* __restrict__ x, int64_t rows, int r,
-                                                       unsigned char* __restrict__ out, T* __restrict__ scale) {
+__global__ __launch_bounds__(256) void split_sl_kernel(const T2* x, int64_t rows, int r, unsigned char* out, T* scale) {
+  pdl_begin();
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
@@ -299,6 +300,7 @@ struct Ring {   // position in a ring of shared-memory slots, and the parity of 
 // lets its own copies and MMAs land, frees its tensor memory and returns.
 template <int S, class T2, class T>
 __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlArgs t, int nblk, unsigned* status) {
+  pdl_begin();
   constexpr int NA = Cfg<S>::NA, NB = Cfg<S>::NB;
   constexpr int RPT = SL_M * 8 / SL_PRODUCERS;   // rows per producer thread
   extern __shared__ unsigned char smem_raw[];
@@ -584,7 +586,7 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
 }
 
 template <int S, class T2, class T>
-void launch_sl(const GemmArgs& a, const SlArgs& t, unsigned* status, cudaStream_t s) {
+void launch_sl(const GemmArgs& a, const SlArgs& t, unsigned* status, LaunchStream s) {
   static bool attr[64] = {false};
   static int nsm[64] = {0};
   int dev = 0;
@@ -598,8 +600,7 @@ void launch_sl(const GemmArgs& a, const SlArgs& t, unsigned* status, cudaStream_
   const int n = block_rows<S>(a.M), nblk = (a.M + n - 1) / n;
   const int64_t items = a.ntiles * nblk;
   if (items > INT32_MAX - 1024) throw Error(-5, "translation stage has too many work items");
-  gemm_sl_kernel<S, T2, T><<<(unsigned)std::min<int64_t>(items, nsm[dev]), SL_THREADS, sl_smem<S>(), s>>>(a, t, nblk,
-                                                                                                          status);
+  launch_pdl(gemm_sl_kernel<S, T2, T>, (unsigned)std::min<int64_t>(items, nsm[dev]), SL_THREADS, sl_smem<S>(), s, a, t, nblk, status);
   DFMM_CUDA(cudaGetLastError());
 }
 
@@ -626,17 +627,17 @@ void build_sl_image(const double2* ops, int M, int Kd, int nops, void* img, void
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_split_sl(const float2* x, int64_t rows, int r, void* out, void* scale, bool fp64, cudaStream_t s) {
+void launch_split_sl(const float2* x, int64_t rows, int r, void* out, void* scale, bool fp64, LaunchStream s) {
   if (rows == 0) return;
   const unsigned grid = (unsigned)((rows * 32 + 255) / 256);
   if (fp64)
-    split_sl_kernel<8, double2, double><<<grid, 256, 0, s>>>((const double2*)x, rows, r, (unsigned char*)out, (double*)scale);
+    launch_pdl(split_sl_kernel<8, double2, double>, grid, 256, 0, s, (const double2*)x, rows, r, (unsigned char*)out, (double*)scale);
   else
-    split_sl_kernel<3, float2, float><<<grid, 256, 0, s>>>(x, rows, r, (unsigned char*)out, (float*)scale);
+    launch_pdl(split_sl_kernel<3, float2, float>, grid, 256, 0, s, x, rows, r, (unsigned char*)out, (float*)scale);
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_gemm_stage_sl(const GemmArgs& a, const SlArgs& t, unsigned* status, bool fp64, cudaStream_t s) {
+void launch_gemm_stage_sl(const GemmArgs& a, const SlArgs& t, unsigned* status, bool fp64, LaunchStream s) {
   if (a.ntiles == 0) return;
   if (!gemm_sl_supported(a.M, a.Kd) || a.src_ld != a.Kd)
     throw Error(-5, "sliced stage needs ranks that are multiples of 8, <= 512, and dense source rows");

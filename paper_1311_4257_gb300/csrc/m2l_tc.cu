@@ -433,14 +433,14 @@ void build_tc_image(const float2* ops, int M, int Kd, int nops, __half* img, flo
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_split(const float2* x, int64_t rows, int ld, __half* hi, __half* lo, float* scale, cudaStream_t s) {
+void launch_split(const float2* x, int64_t rows, int ld, __half* hi, __half* lo, float* scale, LaunchStream s) {
   if (rows == 0) return;
   const int64_t threads = rows * 32;
   split_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>((const float*)x, rows, 2 * ld, hi, lo, scale);
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_gemm_stage_tc(const GemmArgs& a, const TcArgs& t, unsigned* status, cudaStream_t s) {
+void launch_gemm_stage_tc(const GemmArgs& a, const TcArgs& t, unsigned* status, LaunchStream s) {
   if (a.ntiles == 0) return;
   if (!gemm_tc_supported(a.M, a.Kd) || a.src_ld != a.Kd)
     throw Error(-5, "tensor-core stage needs ranks padded to a multiple of 8 and dense source rows");
