@@ -45,7 +45,7 @@ typedef enum {
   DFMM_ERR_INVALID = -1,      /* bad argument (null pointer, N < 1, nrhs < 1, ...) */
   DFMM_ERR_DOMAIN = -2,       /* a point lies outside the root box |x|_inf <= K/2 */
   DFMM_ERR_OOM = -3,          /* device or host allocation failed */
-  DFMM_ERR_CUDA = -4,         /* a CUDA runtime / cuBLAS call failed */
+  DFMM_ERR_CUDA = -4,         /* a CUDA runtime call failed */
   DFMM_ERR_UNSUPPORTED = -5,  /* eps outside [1e-8, 1e-2], K outside (0, 4096] */
   DFMM_ERR_TIMEOUT = -6,      /* a device-side bounded wait gave up */
   DFMM_ERR_DEVICE = -7,       /* a device-side check failed (status word set) */

@@ -15,7 +15,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libdfmm.so")
 
-SOURCES = ["sort.cu", "tree.cu", "operators.cu", "apply.cu", "apply64.cu", "skeleton_gpu.cu", "validate.cu", "m2l_tc.cu", "m2l_cx.cu", "m2l_sl.cu", "gemm_few.cu", "noalloc.cu", "probes.cu", "skeleton.cpp", "dfmm.cpp",
+SOURCES = ["sort.cu", "tree.cu", "operators.cu", "apply.cu", "apply64.cu", "skeleton_gpu.cu", "validate.cu", "m2l_tc.cu", "m2l_cx.cu", "m2l_sl.cu", "gemm_few.cu", "noalloc.cu", "probes.cu", "krylov.cu", "skeleton.cpp", "dfmm.cpp",
            "serve.cpp", "solve.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -72,7 +72,7 @@ def build(verbose: bool = False) -> str:
     linked = open(stamp).read() if os.path.exists(stamp) else ""
     if cmds or not os.path.exists(LIB) or linked != "\n".join(objs) or \
             any(os.path.getmtime(o) > os.path.getmtime(LIB) for o in objs):
-        link = [nvcc(), "-shared", "-o", LIB] + objs + ARCH + ["-lcublas", "-lcudart"]
+        link = [nvcc(), "-shared", "-o", LIB] + objs + ARCH + ["-lcudart"]
         res = subprocess.run(link, capture_output=True, text=True)
         if res.returncode != 0:
             raise RuntimeError("link failed:\n" + res.stdout + res.stderr)

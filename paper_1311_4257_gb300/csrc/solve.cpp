@@ -7,18 +7,19 @@
 // Krylov method applies G once); this is that outer loop, with the matvec
 // through dfmm_apply on the caller's stream.  The Krylov basis lives on the
 // device (complex64); each new vector is orthogonalised by classical
-// Gram-Schmidt done twice (two GEMVs against the basis per pass), the small
+// Gram-Schmidt done twice (two kernels per pass, krylov.cu), the small
 // Hessenberg least-squares problem is solved on the host in double precision
-// with Givens rotations.
-#include <cublas_v2.h>
-
+// with Givens rotations; the host waits once per iteration.
 #include <cmath>
 #include <complex>
+#include <cstring>
+#include <string>
 #include <vector>
 
 #include "common.h"
 #include "dfmm.h"
 #include "internal.h"
+#include "krylov.h"
 
 namespace {
 
@@ -31,18 +32,7 @@ struct DevBuf {
   }
 };
 
-struct Blas {
-  cublasHandle_t h = nullptr;
-  ~Blas() {
-    if (h) cublasDestroy(h);
-  }
-};
-
-void check(cublasStatus_t st, const char* what) {
-  if (st != CUBLAS_STATUS_SUCCESS) throw dfmm::Error(DFMM_ERR_CUDA, std::string("cuBLAS failed: ") + what);
-}
-
-cuComplex c32(cd z) { return make_cuComplex((float)z.real(), (float)z.imag()); }
+float2 c32(cd z) { return make_float2((float)z.real(), (float)z.imag()); }
 
 }  // namespace
 
@@ -61,74 +51,80 @@ extern "C" int dfmm_solve(dfmm_plan_t plan, double alpha_re, double alpha_im, do
     const int64_t N = st.N;
     const int m = restart;
     const cd alpha(alpha_re, alpha_im), beta(beta_re, beta_im);
+    // basis, one vector, and beside the kernels' scratch what the host reads back in one copy: the
+    // norm of the new vector and its products with the basis in the two passes
     DevBuf Vb, wb, hb;
-    if (cudaMalloc(&Vb.p, (size_t)(m + 1) * N * sizeof(cuComplex)) != cudaSuccess ||
-        cudaMalloc(&wb.p, (size_t)N * sizeof(cuComplex)) != cudaSuccess ||
-        cudaMalloc(&hb.p, (size_t)(m + 1) * sizeof(cuComplex)) != cudaSuccess) {
+    const int64_t scratch = (dfmm::krylov_scratch_bytes(N, m + 1) + 255) & ~(int64_t)255;
+    const size_t back = sizeof(double) + 2 * (size_t)(m + 1) * sizeof(float2);
+    if (cudaMalloc(&Vb.p, (size_t)(m + 1) * N * sizeof(float2)) != cudaSuccess ||
+        cudaMalloc(&wb.p, (size_t)N * sizeof(float2)) != cudaSuccess ||
+        cudaMalloc(&hb.p, scratch + back) != cudaSuccess) {
       cudaGetLastError();
       return dfmm::set_error(DFMM_ERR_OOM, "GMRES workspace allocation failed");
     }
-    cuComplex* V = (cuComplex*)Vb.p;
-    cuComplex* w = (cuComplex*)wb.p;
-    cuComplex* hd = (cuComplex*)hb.p;
-    cuComplex* xv = (cuComplex*)x;
-    const cuComplex* bv = (const cuComplex*)b;
-    Blas B;
-    check(cublasCreate(&B.h), "create");
-    check(cublasSetStream(B.h, stream), "set stream");
-    const cuComplex one = make_cuComplex(1.f, 0.f), zero = make_cuComplex(0.f, 0.f), mone = make_cuComplex(-1.f, 0.f);
-    const cuComplex ca = c32(alpha), cb = c32(beta);
+    DFMM_CUDA(cudaMemsetAsync(hb.p, 0, 256, stream));
+    float2* V = (float2*)Vb.p;
+    float2* w = (float2*)wb.p;
+    double* nd = (double*)((char*)hb.p + scratch);
+    float2* hd = (float2*)(nd + 1);
+    float2* xv = (float2*)x;
+    const float2* bv = (const float2*)b;
+    const float2 ca = c32(alpha), cb = c32(beta);
+    std::vector<char> hback(back);
+    auto read_back = [&](size_t bytes) {
+      DFMM_CUDA(cudaMemcpyAsync(hback.data(), nd, bytes, cudaMemcpyDeviceToHost, stream));
+      DFMM_CUDA(cudaStreamSynchronize(stream));
+      double r;
+      std::memcpy(&r, hback.data(), sizeof r);
+      return r;
+    };
 
-    // out = (alpha I + beta G) v
-    auto matvec = [&](const cuComplex* v, cuComplex* out) {
+    auto apply = [&](const float2* v, float2* out) {
       const int rc = dfmm_apply(plan, v, out, 1, stream);
       if (rc != DFMM_OK) throw dfmm::Error(rc, dfmm_last_error());
-      check(cublasCscal(B.h, (int)N, &cb, out, 1), "scal");
-      check(cublasCaxpy(B.h, (int)N, &ca, v, 1, out, 1), "axpy");
     };
-    auto nrm = [&](const cuComplex* v) {
-      float r = 0.f;
-      check(cublasScnrm2(B.h, (int)N, v, 1, &r), "nrm2");
-      return (double)r;
+    auto nrm = [&](float2* v) {
+      dfmm::krylov_update(V, 0, nullptr, v, nd, hb.p, N, stream);
+      return read_back(sizeof(double));
     };
     // r = b - A x into dst
-    auto residual = [&](cuComplex* dst) {
-      matvec(xv, w);
-      DFMM_CUDA(cudaMemcpyAsync(dst, bv, (size_t)N * sizeof(cuComplex), cudaMemcpyDeviceToDevice, stream));
-      check(cublasCaxpy(B.h, (int)N, &mone, w, 1, dst, 1), "axpy");
+    auto residual = [&](float2* dst) {
+      apply(xv, w);
+      dfmm::krylov_combine(c32(-alpha), xv, c32(-beta), w, make_float2(1.f, 0.f), bv, dst, N, stream);
     };
 
-    const double bnorm = nrm(bv);
+    const double bnorm = nrm((float2*)bv);   // no columns: only read
     int done = 0;
     double rr = 0.0;
     if (bnorm == 0.0) {
-      DFMM_CUDA(cudaMemsetAsync(xv, 0, (size_t)N * sizeof(cuComplex), stream));
+      DFMM_CUDA(cudaMemsetAsync(xv, 0, (size_t)N * sizeof(float2), stream));
     } else {
       std::vector<cd> H((size_t)(m + 1) * m), g(m + 1), cs(m), sn(m), y(m);
-      std::vector<cuComplex> hh(m + 1), yc(m);
+      std::vector<float2> yc(m);
       while (done < maxit) {
         residual(V);
         const double beta0 = nrm(V);
         rr = beta0 / bnorm;
         if (rr <= tol) break;
-        const float inv0 = (float)(1.0 / beta0);
-        check(cublasCsscal(B.h, (int)N, &inv0, V, 1), "scal");
+        dfmm::krylov_scale(V, nd, N, stream);
         std::fill(H.begin(), H.end(), cd(0));
         std::fill(g.begin(), g.end(), cd(0));
         g[0] = beta0;
         int k = 0;
         for (int j = 0; j < m && done < maxit; ++j) {
-          cuComplex* vj = V + (size_t)(j + 1) * N;
-          matvec(V + (size_t)j * N, vj);
-          for (int pass = 0; pass < 2; ++pass) {   // classical Gram-Schmidt, twice
-            check(cublasCgemv(B.h, CUBLAS_OP_C, (int)N, j + 1, &one, V, (int)N, vj, 1, &zero, hd, 1), "gemv");
-            DFMM_CUDA(cudaMemcpyAsync(hh.data(), hd, (size_t)(j + 1) * sizeof(cuComplex), cudaMemcpyDeviceToHost,
-                                      stream));
-            DFMM_CUDA(cudaStreamSynchronize(stream));
-            for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] += cd(hh[i].x, hh[i].y);
-            check(cublasCgemv(B.h, CUBLAS_OP_N, (int)N, j + 1, &mone, V, (int)N, hd, 1, &one, vj, 1), "gemv");
-          }
-          const double hn = nrm(vj);
+          const float2* v = V + (size_t)j * N;
+          float2* vj = V + (size_t)(j + 1) * N;
+          // vj = (alpha I + beta G) v, orthogonalised by classical Gram-Schmidt, twice
+          apply(v, w);
+          dfmm::krylov_dots(V, j + 1, vj, w, cb, v, ca, hd, hb.p, N, stream);
+          dfmm::krylov_update(V, j + 1, hd, vj, nd, hb.p, N, stream);
+          dfmm::krylov_dots(V, j + 1, vj, nullptr, cb, nullptr, ca, hd + m + 1, hb.p, N, stream);
+          dfmm::krylov_update(V, j + 1, hd + m + 1, vj, nd, hb.p, N, stream);
+          dfmm::krylov_scale(vj, nd, N, stream);
+          const double hn = read_back(back);
+          const float2* hh = (const float2*)(hback.data() + sizeof(double));
+          for (int i = 0; i <= j; ++i)
+            H[(size_t)i * m + j] = cd(hh[i].x, hh[i].y) + cd(hh[m + 1 + i].x, hh[m + 1 + i].y);
           H[(size_t)(j + 1) * m + j] = hn;
           // earlier rotations, then a new one that zeroes H[j+1][j]
           for (int i = 0; i < j; ++i) {
@@ -148,8 +144,6 @@ extern "C" int dfmm_solve(dfmm_plan_t plan, double alpha_re, double alpha_im, do
           k = j + 1;
           rr = std::abs(g[j + 1]) / bnorm;
           if (rr <= tol || hn == 0.0) break;
-          const float invn = (float)(1.0 / hn);
-          check(cublasCsscal(B.h, (int)N, &invn, vj, 1), "scal");
         }
         // y = H[0:k, 0:k]^-1 g[0:k];  x += V[:, 0:k] y
         for (int i = k - 1; i >= 0; --i) {
@@ -157,9 +151,9 @@ extern "C" int dfmm_solve(dfmm_plan_t plan, double alpha_re, double alpha_im, do
           for (int l = i + 1; l < k; ++l) s -= H[(size_t)i * m + l] * y[l];
           y[i] = s / H[(size_t)i * m + i];
         }
-        for (int i = 0; i < k; ++i) yc[i] = c32(y[i]);
-        DFMM_CUDA(cudaMemcpyAsync(hd, yc.data(), (size_t)k * sizeof(cuComplex), cudaMemcpyHostToDevice, stream));
-        check(cublasCgemv(B.h, CUBLAS_OP_N, (int)N, k, &one, V, (int)N, hd, 1, &one, xv, 1), "gemv");
+        for (int i = 0; i < k; ++i) yc[i] = c32(-y[i]);
+        DFMM_CUDA(cudaMemcpyAsync(hd, yc.data(), (size_t)k * sizeof(float2), cudaMemcpyHostToDevice, stream));
+        dfmm::krylov_update(V, k, hd, xv, nd, hb.p, N, stream);
         DFMM_CUDA(cudaStreamSynchronize(stream));
         if (rr <= tol) break;
       }
