@@ -44,13 +44,17 @@
 //    (red.global.add.v4.f32), and one warp instruction covers 8 target rows x
 //    64 contiguous bytes.  Eight warps: 4.35 against 4.54 ms with four on the apply below.
 //
+//  * The MMA warp issues converged, from an elected lane (tcgen05.cuh): from one
+//    diverged thread an MMA took 115 to 140 clocks to issue, more than most take to run.
+//
 // Measured, sphere of 64 wavelengths, eps 1e-5 (N = 1,286,796): all
-// translations 5.27 -> 3.22 ms (228 -> 370 TFLOP/s useful, of 655 at the measured
-// FP16 rate and three products), the apply 6.40 -> 4.31 ms; ellipsoid of 32 with 16
-// right-hand sides, whose rank 144 stages took the real-block form: 6.53 -> 4.02
-// ms.  Role timers: the MMA thread issues or waits for the tensor pipe 90% of a
-// tile (10.2k of 11.3k clocks, 6.1k at the unhindered rate): what bounds it is
-// shared-memory bandwidth, operand reads and copies together.
+// translations 5.27 -> 3.13 ms (228 -> 378 TFLOP/s useful, of 655 at the measured
+// FP16 rate and three products), the apply 6.40 -> 4.22 ms; ellipsoid of 32 with 16
+// right-hand sides, whose rank 144 stages took the real-block form: 6.53 -> 3.73
+// ms.  Of these the warp-wide issue gave 4.31 -> 4.22 and 4.02 -> 3.73 ms.  Role timers: a
+// tile takes 11k clocks, 6.1k of them MMAs at the unhindered rate and 7.4k the
+// epilogue's reductions into L2 (128 KB a tile at 5 TB/s over the chip); copies,
+// operand reads and reductions share the SM's memory pipe, and that is what bounds it.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -127,14 +131,14 @@ __device__ __forceinline__ uint32_t idesc_cx(int n, bool neg_a) {
 }
 
 template <int KIND>
-__device__ __forceinline__ void mma_cx(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_cx(uint32_t lead, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   if (KIND == 2)
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-            d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc));
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n @q tcgen05.mma.cta_group::1.kind::tf32 "
+        "[%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(lead));
   else
-    mma_f16(d_tmem, a, b, idesc, acc);
+    mma_f16_by(lead, d_tmem, a, b, idesc, acc);
 }
 
 // N elements (4 or 8 bytes each) of one tile row as one store
@@ -264,14 +268,6 @@ __device__ __forceinline__ CxStage stage_of(const GemmArgs& a, const TcArgs& t, 
 // component (2 n columns) and two tensor-memory buffers, so that the MMAs
 // of an item overlap the epilogue of the previous one; the cross terms of a
 // chunk then come first, while the accumulators they are truncated to are small.
-struct CxRing {   // position in a ring of shared-memory slots, and the parity of its current use
-  int st = 0;
-  uint32_t ph = 0;
-  __device__ __forceinline__ void next(int n) {
-    if (++st == n) { st = 0; ph ^= 1u; }
-  }
-};
-
 template <int KIND, bool ONE>
 __global__ __launch_bounds__(CX_THREADS, 1) void gemm_cx_kernel(GemmArgs a, TcArgs t, int nblk, unsigned* status) {
   pdl_begin();
@@ -357,7 +353,7 @@ __global__ __launch_bounds__(CX_THREADS, 1) void gemm_cx_kernel(GemmArgs a, TcAr
     const unsigned char *src_n = nullptr, *img_n = nullptr;
     if (it < nitems) load_rows(tile_n, rows_n, src_n, img_n);
     int4 tile_nn = it + G < nitems ? a.tiles[(it + G) / nblk] : none;
-    CxRing ra, rb;
+    Ring ra, rb;
     int ga = 0, gb = 0;   // slots filled so far (ga up to the ring's size: no wait on the first round)
     bool ok = true;
     for (; it < nitems && ok; it += G) {
@@ -419,25 +415,26 @@ __global__ __launch_bounds__(CX_THREADS, 1) void gemm_cx_kernel(GemmArgs a, TcAr
       }
   } else if (warp == CX_MMA_WARP) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      CxRing ra, rb;
+    {
+      const uint32_t lead = elect_one(), tm = __reduce_max_sync(0xffffffffu, tmem);   // uniform
+      Ring ra, rb;
       int last = -1, i = 0;
       uint32_t last_ph = 0;
       // wait_test: a wait that can only end by giving up; the CTA then takes the timeout path
-      bool ok = !(a.wait_test && blockIdx.x == 0) || mbar_wait(smem_u32(never), 0u, status);
+      bool ok = !(a.wait_test && blockIdx.x == 0) || warp_wait(smem_u32(never), 0u, status);
       for (int it = (int)blockIdx.x; it < nitems && ok; it += G, ++i) {
         const int nb = min(n, M - (it % nblk) * n);
         const uint32_t i1 = idesc_cx<KIND>(nb, false), i1n = idesc_cx<KIND>(nb, true), i2 = idesc_cx<KIND>(2 * nb, false);
         // buffer of this item: ONE alternates two buffers of 2 n columns
         const int b = ONE ? (i & 1) : 0;
         const int use = ONE ? (i >> 1) : i;   // earlier items on this buffer
-        const uint32_t YR = tmem + (uint32_t)(b * 256), YI = YR + (uint32_t)nb;
+        const uint32_t YR = tm + (uint32_t)(b * 256), YI = YR + (uint32_t)nb;
         const uint32_t yr = ONE ? YR : YR + 2u * nb, yi = ONE ? YI : YR + 3u * nb;
-        if (use > 0 && !mbar_wait(smem_u32(&acc_empty[b]), (uint32_t)((use - 1) & 1), status)) break;
+        if (use > 0 && !warp_wait(smem_u32(&acc_empty[b]), (uint32_t)((use - 1) & 1), status)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         // next gathered tile: its address in shared memory once it is full
         auto take = [&](uint32_t& xa, uint32_t& bar) {
-          if (!mbar_wait(smem_u32(&fullA[ra.st]), ra.ph, status)) return false;
+          if (!warp_wait(smem_u32(&fullA[ra.st]), ra.ph, status)) return false;
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // cp.async data -> async proxy
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           xa = sA + ra.st * CX_TILE;
@@ -449,7 +446,7 @@ __global__ __launch_bounds__(CX_THREADS, 1) void gemm_cx_kernel(GemmArgs a, TcAr
         };
         for (int c = 0; c < nchunk; ++c) {
           uint32_t xr, xi, br, bi;
-          ok = mbar_wait(smem_u32(&fullB[rb.st]), rb.ph, status) && take(xr, br);
+          ok = warp_wait(smem_u32(&fullB[rb.st]), rb.ph, status) && take(xr, br);
           if (!ok) break;
           const int ksteps = min(BKE, Kh - c * BKE) / KSTEP;
           // operator rows: [Tr hi | Ti hi], [Tr lo | Ti lo]; y = [Re | Im] are adjacent columns, so one
@@ -459,44 +456,44 @@ __global__ __launch_bounds__(CX_THREADS, 1) void gemm_cx_kernel(GemmArgs a, TcAr
           const uint64_t dl = smem_desc_sw128(xr);
           // cross terms: xr lo, xi lo with T hi; xr hi, xi hi with T lo
           for (int k = 0; k < ksteps; ++k)
-            mma_cx<KIND>(yr, dl + 2 * k, rh + 2 * k, i2, (c > 0 || k > 0) ? 1u : 0u);
-          mma_commit(br);
+            mma_cx<KIND>(lead, yr, dl + 2 * k, rh + 2 * k, i2, (c > 0 || k > 0) ? 1u : 0u);
+          mma_commit_by(lead, br);
           ok = take(xi, bi);
           if (!ok) break;
           const uint64_t el = smem_desc_sw128(xi);
           for (int k = 0; k < ksteps; ++k) {
-            mma_cx<KIND>(yr, el + 2 * k, ih + 2 * k, i1n, 1u);
-            mma_cx<KIND>(yi, el + 2 * k, rh + 2 * k, i1, 1u);
+            mma_cx<KIND>(lead, yr, el + 2 * k, ih + 2 * k, i1n, 1u);
+            mma_cx<KIND>(lead, yi, el + 2 * k, rh + 2 * k, i1, 1u);
           }
-          mma_commit(bi);
+          mma_commit_by(lead, bi);
           ok = take(xr, br);
           if (!ok) break;
           const uint64_t dh = smem_desc_sw128(xr);
-          for (int k = 0; k < ksteps; ++k) mma_cx<KIND>(yr, dh + 2 * k, rl + 2 * k, i2, 1u);
+          for (int k = 0; k < ksteps; ++k) mma_cx<KIND>(lead, yr, dh + 2 * k, rl + 2 * k, i2, 1u);
           ok = take(xi, bi);
           if (!ok) break;
           const uint64_t eh = smem_desc_sw128(xi);
           for (int k = 0; k < ksteps; ++k) {
-            mma_cx<KIND>(yr, eh + 2 * k, il + 2 * k, i1n, 1u);
-            mma_cx<KIND>(yi, eh + 2 * k, rl + 2 * k, i1, 1u);
+            mma_cx<KIND>(lead, yr, eh + 2 * k, il + 2 * k, i1n, 1u);
+            mma_cx<KIND>(lead, yi, eh + 2 * k, rl + 2 * k, i1, 1u);
           }
           // the large terms
           for (int k = 0; k < ksteps; ++k)
-            mma_cx<KIND>(YR, dh + 2 * k, rh + 2 * k, i2, (ONE || c > 0 || k > 0) ? 1u : 0u);
-          mma_commit(br);
+            mma_cx<KIND>(lead, YR, dh + 2 * k, rh + 2 * k, i2, (ONE || c > 0 || k > 0) ? 1u : 0u);
+          mma_commit_by(lead, br);
           for (int k = 0; k < ksteps; ++k) {
-            mma_cx<KIND>(YR, eh + 2 * k, ih + 2 * k, i1n, 1u);
-            mma_cx<KIND>(YI, eh + 2 * k, rh + 2 * k, i1, 1u);
+            mma_cx<KIND>(lead, YR, eh + 2 * k, ih + 2 * k, i1n, 1u);
+            mma_cx<KIND>(lead, YI, eh + 2 * k, rh + 2 * k, i1, 1u);
           }
-          mma_commit(bi);
-          mma_commit(smem_u32(&emptyB[rb.st]));
+          mma_commit_by(lead, bi);
+          mma_commit_by(lead, smem_u32(&emptyB[rb.st]));
           rb.next(CX_NB);
         }
         if (!ok) break;
-        mma_commit(smem_u32(&acc_full[b]));
+        mma_commit_by(lead, smem_u32(&acc_full[b]));
       }
       if (last >= 0) {   // every MMA issued so far has completed once one more commit has arrived
-        mma_commit(smem_u32(never));
+        mma_commit_by(lead, smem_u32(never));
         mbar_wait_drain(smem_u32(never), 0u);
       }
     }

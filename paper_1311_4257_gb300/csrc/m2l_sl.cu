@@ -34,11 +34,16 @@
 // shared-memory pass per global line an instruction touches (16-value chunks,
 // 16 lines per instruction: 19 passes instead of 4; 4.16 -> 3.76 ms on the case below).
 //
+// The MMA warp issues converged, from an elected lane (tcgen05.cuh); from one diverged
+// thread the issue of an MMA, 115 to 140 clocks, was the longest part of an item (16.7k
+// clocks, 10k at the MMAs' own rate).
+//
 // Measured against the CUDA-core stages that served these tolerances: sphere of 32
-// wavelengths, eps 1e-6 (N = 321,699, FP32): all translations 19.2 -> 3.3 ms, 22
-// -> 130 TFLOP/s; sphere of 8, eps 1e-8 (FP64): 68 -> 3.1 ms, 0.75 -> 16.5
-// TFLOP/s.  It is bound by shared-memory bandwidth: the MMAs' operand reads and
-// the copies into the tiles.
+// wavelengths, eps 1e-6 (N = 321,699, FP32): all translations 19.2 -> 2.47 ms, 22
+// -> 174 TFLOP/s (of 330 at the MMAs' rate); sphere of 8, eps 1e-8 (FP64): 68 ->
+// 2.43 ms, 0.75 -> 21 TFLOP/s.  The warp-wide issue gave the applies 3.76 -> 2.88 and
+// 3.78 -> 3.03 ms of that.  It is bound by shared-memory bandwidth (operand reads and
+// the copies into the tiles) where tiles are full, by part-filled tiles elsewhere.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -279,14 +284,6 @@ __device__ __forceinline__ double join8(const uint32_t* r) {
   return (double)(hi * (1 << 19) + ((lo + 256) >> 9));
 }
 
-struct Ring {   // position in a ring of shared-memory slots, and the parity of its current use
-  int st = 0;
-  uint32_t ph = 0;
-  __device__ __forceinline__ void next(int n) {
-    if (++st == n) { st = 0; ph ^= 1u; }
-  }
-};
-
 // Persistent, warp-specialised; item = (tile, block of n outputs), CTA x takes
 // items x, x + gridDim.x, ..., so the CTAs that run together share a tile's
 // gathered rows in L2.
@@ -432,7 +429,8 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
       }
   } else if (warp == SL_MMA_WARP) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    {
+      const uint32_t lead = elect_one(), tm = __reduce_max_sync(0xffffffffu, tmem);   // uniform
       Ring ra, rb;
       int last = -1, i = 0;
       uint32_t last_ph = 0;
@@ -440,17 +438,17 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
       bool ok = true;
       for (int it = (int)blockIdx.x; it < nitems && ok; it += G, ++i) {
         const int blk = it % nblk, nb = min(n, Mp - blk * n);
-        if (i > 0 && !mbar_wait(smem_u32(acc_empty), (uint32_t)((i - 1) & 1), status)) break;
+        if (i > 0 && !warp_wait(smem_u32(acc_empty), (uint32_t)((i - 1) & 1), status)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         for (int c = 0; c < nchunk && ok; ++c) {
-          if (!mbar_wait(smem_u32(&fullB[rb.st]), rb.ph, status)) {
+          if (!warp_wait(smem_u32(&fullB[rb.st]), rb.ph, status)) {
             ok = false;
             break;
           }
           const int ksteps = min(SL_K, kp - c * SL_K) / 16;
           const uint32_t tr = sB + rb.st * b_bytes_max<S>(), ti = tr + (uint32_t)(S * SL_ROW * nb);
           for (int h = 0; h < 2 * S; ++h) {
-            if (!mbar_wait(smem_u32(&fullA[ra.st]), ra.ph, status)) {
+            if (!warp_wait(smem_u32(&fullA[ra.st]), ra.ph, status)) {
               ok = false;
               break;
             }
@@ -460,25 +458,25 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
             const bool im = h >= S;
             const int sl = im ? h - S : h;
             const uint32_t xa = sA + ra.st * SL_TILE, b_re = im ? ti : tr, b_im = im ? tr : ti;
-            const uint32_t d_re = tmem + (uint32_t)(sl * nb), d_im = d_re + (uint32_t)(S * nb);
+            const uint32_t d_re = tm + (uint32_t)(sl * nb), d_im = d_re + (uint32_t)(S * nb);
             const uint32_t id_re = idesc_f16((S - sl) * nb, im), id_im = idesc_f16((S - sl) * nb);
             for (int k = 0; k < ksteps; ++k) {
               const uint64_t da = smem_desc_sw128(xa + 32 * k);
               const uint32_t acc = (c > 0 || h > 0 || k > 0) ? 1u : 0u;   // the first covers every group
-              mma_f16(d_re, da, smem_desc_sw128(b_re + 32 * k), id_re, acc);
-              mma_f16(d_im, da, smem_desc_sw128(b_im + 32 * k), id_im, acc);
+              mma_f16_by(lead, d_re, da, smem_desc_sw128(b_re + 32 * k), id_re, acc);
+              mma_f16_by(lead, d_im, da, smem_desc_sw128(b_im + 32 * k), id_im, acc);
             }
-            mma_commit(smem_u32(&emptyA[ra.st]));
+            mma_commit_by(lead, smem_u32(&emptyA[ra.st]));
             last = ra.st;
             last_ph = ra.ph;
             ra.next(NA);
           }
           if (!ok) break;
-          mma_commit(smem_u32(&emptyB[rb.st]));
+          mma_commit_by(lead, smem_u32(&emptyB[rb.st]));
           rb.next(NB);
         }
         if (!ok) break;
-        mma_commit(smem_u32(acc_full));
+        mma_commit_by(lead, smem_u32(acc_full));
       }
       // MMAs complete in order: once the last commit has arrived, all have
       if (last >= 0) mbar_wait_drain(smem_u32(&emptyA[last]), last_ph);

@@ -130,6 +130,46 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
+// ---- issue by a whole warp ----
+// The MMA warp runs its loop converged and one elected lane issues: ring positions and
+// descriptors are then uniform over the warp and stay in uniform registers, which the MMA
+// reads.  Issued from one diverged thread, every descriptor went through a register
+// move of its own and an MMA took 115 to 140 clocks to issue whatever its size.
+
+// 1 on one lane of the (converged) warp
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p;
+}
+// mbar_wait by all lanes together, with one result
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, unsigned* status) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const unsigned long long t0 = globaltimer();
+  for (;;) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const bool late = globaltimer() - t0 > kWaitNs || (*(volatile unsigned*)status & kStatusTimeout);
+    if (__any_sync(0xffffffffu, late)) {
+      atomicOr(status, kStatusTimeout);
+      return false;
+    }
+  }
+}
+__device__ __forceinline__ void mma_f16_by(uint32_t lead, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
+                                           uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n @q tcgen05.mma.cta_group::1.kind::f16 "
+      "[%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(lead));
+}
+__device__ __forceinline__ void mma_commit_by(uint32_t lead, uint32_t bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 "
+      "[%0];\n}\n" ::"r"(bar),
+      "r"(lead)
+      : "memory");
+}
+
 // 16 lanes x 32 columns of one accumulator (.16x256b, 4 repetitions): thread t
 // gets lane t/4 (r[4j], r[4j+1]) and lane t/4 + 8 (r[4j+2], r[4j+3]) at columns
 // 8j + 2 (t % 4) + {0, 1}
@@ -140,6 +180,14 @@ __device__ __forceinline__ void tmem_ld16x256_x4(uint32_t ta, uint32_t* r) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(ta));
 }
+
+struct Ring {   // position in a ring of shared-memory slots, and the parity of its current use
+  int st = 0;
+  uint32_t ph = 0;
+  __device__ __forceinline__ void next(int n) {
+    if (++st == n) { st = 0; ph ^= 1u; }
+  }
+};
 
 // column / nrhs for a tile column below 128 and 1 <= nrhs <= 64 by multiplication:
 // exact, since 127 * 63 < 2^16 (a division per gathered row took 3.5k clocks of a 12k-clock tile)
