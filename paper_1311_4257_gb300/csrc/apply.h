@@ -40,7 +40,9 @@ struct GemmArgs {
 
 void launch_gemm_stage(const GemmArgs& a, LaunchStream s);
 // The same products in the same order for stages whose operators serve a few
-// columns each (gemm_few.cu); Kd a multiple of 8, tiles of up to 128 columns.
+// columns each (gemm_few.cu); Kd a multiple of 8, tiles of up to gemm_few_columns() columns
+// (or one pair's right-hand sides).
+int gemm_few_columns();
 void launch_gemm_stage_few(const GemmArgs& a, LaunchStream s);
 
 // One stage of a multi-stage split-complex launch (the batched form runs the

@@ -85,11 +85,14 @@ enum Fam { F_M2L_HF, F_M2L_LF, F_M2M, F_L2L, F_P2L_PROJ, F_P2M_EVAL, F_P2L_EVAL,
 constexpr int64_t kFusedZero = 160 << 20, kBesideNear = 200000, kEarlyLaunch = 1000000;
 
 // columns (pairs x right-hand sides) per operator up to which a stage takes the few-column
-// form, on average over its operators: where its time crosses the split form's (3 columns: 13
-// against 26 us with the split of its source, sphere of 2 wavelengths, 40 points, eps 1e-5; 7
-// columns: 29 against 26), and the sliced form's and the CUDA-core stage's (8 columns: 43
-// against 89 and 172 us, eps 1e-6; 27 columns: both 80)
-constexpr int kFewColsSplit = 4, kFewCols = 12;
+// form, on average over its operators: where its time crosses the sliced form's and the
+// CUDA-core stage's (8 columns: 43 against 89 and 172 us, eps 1e-6; 27 columns: both 80; a limit
+// of 20: 2.88 against 2.49 ms for the solve of sphere 4), and the split form's.  There 4 columns
+// and, with more operators than SMs, when every SM would compute several nearly empty tiles, 8
+// (applies at eps 1e-5, few against split: sphere of 2 wavelengths, 8 columns, 316 operators: 34
+// against 47 us; of 3, 7 columns, 62 operators: 76 against 70; of 8, 3,000 points, 10 columns: 143
+// against 136).
+constexpr int kFewColsSplit = 4, kFewColsSplitMany = 8, kFewCols = 12, kSMs = 152;
 
 const char* kFamName[F_COUNT] = {"m2l_hf", "m2l_lf", "m2m", "l2l", "p2l_proj", "p2m_eval",
                                  "p2l_eval", "l2p", "m2p", "p2p", "permute", "zero", "split"};
@@ -1310,7 +1313,15 @@ bool sliced_stage(const GemmPlan& g) { return g.sl_img != nullptr; }
 // whether a stage runs in the few-column form (gemm_few.cu): its operators serve so few
 // columns each that reading them bounds it
 bool few_columns(const dfmm_plan_s* P, const GemmPlan& g, int nrhs) {
-  return P->few && g.npairs * nrhs <= (int64_t)(P->opt.m2l_mode == 2 ? kFewColsSplit : kFewCols) * (int64_t)g.groups.size();
+  const int64_t ops = (int64_t)g.groups.size();
+  const int cols = P->opt.m2l_mode != 2 ? kFewCols : ops > kSMs ? kFewColsSplitMany : kFewColsSplit;
+  return P->few && g.npairs * nrhs <= cols * ops;
+}
+
+// columns of a stage's work tiles (slices: whether the workspace holds the slices of its source)
+int tile_columns(const dfmm_plan_s* P, const GemmPlan& g, int nrhs, bool slices) {
+  if (few_columns(P, g, nrhs)) return gemm_few_columns();
+  return on_tensor_cores(P, g) || (slices && sliced_stage(g)) ? gemm_tc_columns() : 64;
 }
 
 // tile_order: 0 = by the 64 MB rule above, 1 = always by target block, 2 = always by operator.
@@ -1430,7 +1441,7 @@ struct Runner {
                                        (first && g.dst_unique) ? 1 : 0});
       return;
     }
-    auto t = tiles_for(P, W, g, nrhs, on_tensor_cores(P, g) || (sliced_stage(g) && W->sl) ? gemm_tc_columns() : 64, s);
+    auto t = tiles_for(P, W, g, nrhs, tile_columns(P, g, nrhs, W->sl != nullptr), s);
     GemmArgs a;
     a.ops = g.ops;
     a.M = g.M;
@@ -1754,7 +1765,7 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
   std::vector<int> tl_cols;
   for (const GemmPlan* g : all_gemms(P)) {
     if (g->npairs == 0) continue;
-    const int cols = on_tensor_cores(P, *g) || (slices && sliced_stage(*g)) ? gemm_tc_columns() : 64;
+    const int cols = tile_columns(P, *g, nrhs, slices);
     tl_cols.push_back(cols);
     tl.push_back({g, make_tiles(*g, nrhs, cols, P->opt.tile_order)});
   }

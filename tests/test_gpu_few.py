@@ -21,10 +21,10 @@ def _lib():
     build.build()
 
 
-@pytest.mark.parametrize("n,K", [(7, 2.0), (40, 2.0), (60, 4.0), (301, 8.0)])
+@pytest.mark.parametrize("n,K", [(7, 2.0), (40, 2.0), (60, 4.0), (301, 8.0), (1256, 2.0)])
 def test_few_column_stages(n, K):
     """Ranks that are no multiple of 64 rows or 16 columns, operators with 1 to more than 8
-    columns (several passes), 1 to 3 right-hand sides.  FP32 against FP64 on the same skeletons:
+    columns (several passes), more than 16 (several tiles), 1 to 3 right-hand sides.  FP32 against FP64 on the same skeletons:
     2e-6 as for the other FP32 forms (rounding of about six stages); the split form of eps 1e-5
     adds up to 2e-6 of its own."""
     import torch
