@@ -17,10 +17,10 @@
 //  * p2p_fast_kernel: the near field (U lists) on FP32 coordinates, with the
 //    exact plan-time corrections of the close pairs (p2p_close_kernel,
 //    p2p_close_apply_kernel); p2p_kernel: the same on double-float coordinates.
+#include <type_traits>
+
 #include "apply.h"
 #include "pdl.h"
-
-#include <type_traits>
 
 namespace dfmm {
 
@@ -304,21 +304,23 @@ __global__ __launch_bounds__(256) void rows_kernel(RowsArgs a) {
 // 0.27 ms at K = 64 against 0.28 ms with four rows and 0.43 ms with eight.
 constexpr int L2P_ROWS = 2;
 
-template <int Q>
-__global__ __launch_bounds__(256) void l2p_kernel(L2PArgs a) {
+template <int Q, bool MANY>
+__global__ __launch_bounds__(256) void l2p_kernel(const __grid_constant__ L2PArgs a) {
   pdl_begin();
-  const int64_t r0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * L2P_ROWS;
+  const L2PArgs::Level& g = a.lv[level_of<MANY>(a, blockIdx.x)];
+  const int64_t r0 = (((int64_t)(blockIdx.x - g.block0) * blockDim.x + threadIdx.x) >> 5) * L2P_ROWS;
   const int lane = threadIdx.x & 31;
-  if (r0 >= a.nrows) return;
-  const int R2 = a.R / 2;
+  const int64_t nrows = g.nrows;
+  if (r0 >= nrows) return;
+  const int R = g.R, R2 = R / 2;
   float4 v[L2P_ROWS][Q];
   int2 m[L2P_ROWS];
 #pragma unroll
   for (int j = 0; j < L2P_ROWS; ++j) {
     const int64_t r = r0 + j;
-    const bool ok = r < a.nrows;
-    m[j] = ok ? a.map[r] : make_int2(-1, 0);
-    const float4* row = (const float4*)(a.rows + (ok ? r : r0) * a.R);
+    const bool ok = r < nrows;
+    m[j] = ok ? g.map[r] : make_int2(-1, 0);
+    const float4* row = (const float4*)(g.rows + (ok ? r : r0) * R);
 #pragma unroll
     for (int t = 0; t < Q; ++t) {
       const int q = lane + 32 * t;
@@ -328,7 +330,7 @@ __global__ __launch_bounds__(256) void l2p_kernel(L2PArgs a) {
 #pragma unroll
   for (int j = 0; j < L2P_ROWS; ++j) {
     if (m[j].x < 0) continue;   // warp-uniform
-    const float4* st = (const float4*)(a.state + (int64_t)m[j].y * a.nrhs * a.R);
+    const float4* st = (const float4*)(g.state + (int64_t)m[j].y * a.nrhs * R);
     for (int k = 0; k < a.nrhs; ++k) {
       float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
@@ -361,16 +363,17 @@ __global__ __launch_bounds__(256) void l2p_kernel(L2PArgs a) {
 // accumulated per pass over the rows: 1 for a single right-hand side, whose
 // accumulators then take a quarter of the registers, so that more warps
 // (more rows in flight) fit on an SM.
-template <int Q, int KB>
-__global__ __launch_bounds__(256) void p2m_rows_kernel(P2MRowsArgs a) {
+template <int Q, int KB, bool MANY>
+__global__ __launch_bounds__(256) void p2m_rows_kernel(const __grid_constant__ P2MRowsArgs a) {
   pdl_begin();
-  const int64_t jw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const P2MRowsArgs::Level& g = a.lv[level_of<MANY>(a, blockIdx.x)];
+  const int64_t jw = ((int64_t)(blockIdx.x - g.block0) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (jw >= a.njobs) return;
-  const int4 job = a.jobs[jw];
-  const int R2 = a.R / 2;
-  const float4* rows = (const float4*)a.rows;
-  float4* st = (float4*)a.state;
+  if (jw >= g.njobs) return;
+  const int4 job = g.jobs[jw];
+  const int R2 = g.R / 2;
+  const float4* rows = (const float4*)g.rows;
+  float4* st = (float4*)g.state;
   for (int k0 = 0; k0 < a.nrhs; k0 += KB) {
     const int nk = min(KB, a.nrhs - k0);
     float4 acc[KB][Q];
@@ -802,25 +805,45 @@ void launch_rows(const RowsArgs& a, LaunchStream s) {
   DFMM_CUDA(cudaGetLastError());
 }
 
+// levels of rank up to 128 and beyond: a lane holds 4 or 8 state entries
+template <class A> bool narrow(const typename A::Level& g) { return g.R <= 128; }
+template <class A, class F>
+void by_levels(const A& a, bool narrow, F&& f) {
+  const auto at = [&](auto q) {
+    if (a.nlv == 1) f(q, std::false_type());
+    else f(q, std::true_type());
+  };
+  if (narrow) at(std::integral_constant<int, 2>());
+  else at(std::integral_constant<int, 4>());
+}
+template <class A> void check_ranks(const A& a) {
+  for (int l = 0; l < a.nlv; ++l)
+    if (a.lv[l].R > 256 || a.lv[l].R % 2) throw Error(-5, "representation rank must be even and at most 256");
+}
+
 void launch_l2p(const L2PArgs& a, LaunchStream s) {
-  if (a.nrows == 0) return;
-  if (a.R > 256 || a.R % 2) throw Error(-5, "representation rank must be even and at most 256");
-  const unsigned grid = (unsigned)((a.nrows + 8 * L2P_ROWS - 1) / (8 * L2P_ROWS));
-  if (a.R <= 128) launch_pdl(l2p_kernel<2>, grid, 256, 0, s, a);
-  else launch_pdl(l2p_kernel<4>, grid, 256, 0, s, a);
+  check_ranks(a);
+  for (const bool nar : {true, false}) {
+    L2PArgs p;
+    const unsigned grid = place_levels(a, p, [&](const L2PArgs::Level& g) { return narrow<L2PArgs>(g) == nar; },
+                                       [](const L2PArgs::Level& g) { return (g.nrows + 8 * L2P_ROWS - 1) / (8 * L2P_ROWS); });
+    if (grid == 0) continue;
+    by_levels(p, nar, [&](auto q, auto many) { launch_pdl(l2p_kernel<q(), many()>, grid, 256, 0, s, p); });
+  }
   DFMM_CUDA(cudaGetLastError());
 }
 
 void launch_p2m_rows(const P2MRowsArgs& a, LaunchStream s) {
-  if (a.njobs == 0) return;
-  if (a.R > 256 || a.R % 2) throw Error(-5, "representation rank must be even and at most 256");
-  const unsigned grid = (unsigned)((a.njobs + 7) / 8);
-  if (a.nrhs == 1) {
-    if (a.R <= 128) launch_pdl(p2m_rows_kernel<2, 1>, grid, 256, 0, s, a);
-    else launch_pdl(p2m_rows_kernel<4, 1>, grid, 256, 0, s, a);
-  } else {
-    if (a.R <= 128) launch_pdl(p2m_rows_kernel<2, 4>, grid, 256, 0, s, a);
-    else launch_pdl(p2m_rows_kernel<4, 4>, grid, 256, 0, s, a);
+  check_ranks(a);
+  for (const bool nar : {true, false}) {
+    P2MRowsArgs p;
+    const unsigned grid = place_levels(a, p, [&](const P2MRowsArgs::Level& g) { return narrow<P2MRowsArgs>(g) == nar; },
+                                       [](const P2MRowsArgs::Level& g) { return (g.njobs + 7) / 8; });
+    if (grid == 0) continue;
+    by_levels(p, nar, [&](auto q, auto many) {
+      if (a.nrhs == 1) launch_pdl(p2m_rows_kernel<q(), 1, many()>, grid, 256, 0, s, p);
+      else launch_pdl(p2m_rows_kernel<q(), 4, many()>, grid, 256, 0, s, p);
+    });
   }
   DFMM_CUDA(cudaGetLastError());
 }

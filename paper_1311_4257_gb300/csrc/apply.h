@@ -30,8 +30,6 @@ struct GemmArgs {
   float2* dst;              // rows of dst_ld complex
   int src_ld, dst_ld;
   int nrhs;
-  int store;                // 1: every target row of the stage has one pair and nothing wrote it
-                            //    earlier in the apply, so results are stored, not added
   int wait_test;            // tensor-core form: 1 = CTA 0 waits on a barrier nothing arrives at
                             //    (exercises the bounded-wait failure path)
   const CxStage* stages;    // split-complex form, several stages in one launch (device array), or
@@ -56,7 +54,6 @@ struct CxStage {
   const float* op_scale;
   float2* dst;              // target states
   int nrhs;
-  int store;
 };
 
 // Tensor-core form (tcgen05, scaled FP16 split) of the same stage; M and Kd
@@ -164,28 +161,66 @@ struct RowsArgs {
 };
 void launch_rows(const RowsArgs& a, LaunchStream s);
 
+// The levels of A (L2PArgs, P2MRowsArgs) that `take` accepts, blocks(level) blocks each: their count.
+template <class A, class Take, class Blocks>
+unsigned place_levels(const A& a, A& out, Take&& take, Blocks&& blocks) {
+  int64_t at = 0;
+  out = a;
+  out.nlv = 0;
+  for (int l = 0; l < a.nlv; ++l)
+    if (take(a.lv[l])) {
+      out.lv[out.nlv] = a.lv[l];
+      out.lv[out.nlv++].block0 = (unsigned)at;
+      at += blocks(a.lv[l]);
+    }
+  if (at > INT32_MAX) throw Error(-5, "too many leaves for one launch");
+  return (unsigned)at;
+}
+#ifdef __CUDACC__
+// the level that block b works on (MANY: there may be several; the lookup costs a short block
+// some 5%, sphere of 64 wavelengths 4.22 -> 4.25 ms, so one level does without)
+template <bool MANY, class A>
+__device__ __forceinline__ int level_of(const A& a, unsigned b) {
+  int l = 0;
+  if (!MANY) return l;
+  while (l + 1 < a.nlv && b >= a.lv[l + 1].block0) ++l;
+  return l;
+}
+#endif
+
 // L2P, one warp per point: us[p_r][rhs] += sum_q rows[r][q] state[s_r][rhs][q]
-// for every row r, with (p_r, s_r) = map[r] (each point has one row).
+// for every row r, with (p_r, s_r) = map[r] (each point has one row).  All levels in one
+// launch: those of an adaptive tree hold a few blocks each.
 struct L2PArgs {
-  const int2* map;           // (point, state row) per row
-  int64_t nrows;
-  const float2* rows;        // [nrows][R]
-  const float2* state;       // [..][nrhs][R]
-  int R, nrhs;               // R even, <= 256
-  float2* us;                // [N][nrhs]
+  static constexpr int kMax = 24;   // LF levels
+  struct Level {
+    const int2* map;           // (point, state row) per row
+    int64_t nrows;
+    const float2* rows;        // [nrows][R]
+    const float2* state;       // [..][nrhs][R]
+    int R;                     // even, <= 256
+    unsigned block0;           // first block of the level (set by the launch)
+  } lv[kMax];
+  int nlv, nrhs;
+  float2* us;                  // [N][nrhs]
 };
 void launch_l2p(const L2PArgs& a, LaunchStream s);
 
 // P2M through per-point rows: for every leaf job (first point, count, first
 // row, box) and right-hand side k, state[box][k][q] = sum_i rows[row + i][q]
-// fs[first + i][k].
+// fs[first + i][k].  All levels in one launch, as L2P.
 struct P2MRowsArgs {
-  const int4* jobs;
-  int64_t njobs;
-  const float2* rows;        // [..][R]
-  const float2* fs;          // [N][nrhs]
-  float2* state;             // [boxes][nrhs][R]
-  int R, nrhs;               // R <= 256
+  static constexpr int kMax = 24;
+  struct Level {
+    const int4* jobs;
+    int64_t njobs;
+    const float2* rows;        // [..][R]
+    float2* state;             // [boxes][nrhs][R]
+    int R;                     // <= 256
+    unsigned block0;
+  } lv[kMax];
+  int nlv, nrhs;
+  const float2* fs;            // [N][nrhs]
 };
 void launch_p2m_rows(const P2MRowsArgs& a, LaunchStream s);
 

@@ -12,6 +12,7 @@
 // wavelengths, eps 1e-8 (N = 20,106): near field 1.75 -> 0.50 ms (35 FP64
 // instructions per interaction: 0.32 ms), P2M 0.217 -> 0.061, L2P 0.097 -> 0.054;
 // cube of 4, 4 right-hand sides: P2L 1.39 -> 0.69, P2M 1.26 -> 0.16 ms.
+#include <algorithm>
 #include <type_traits>
 
 #include "apply.h"
@@ -291,12 +292,14 @@ __global__ __launch_bounds__(256) void rows64_kernel(RowsArgs a) {
 }
 
 template <int NR>
-__global__ __launch_bounds__(256) void l2p64_kernel(L2PArgs a) {
+__global__ __launch_bounds__(256) void l2p64_kernel(const __grid_constant__ L2PArgs a) {
   pdl_begin();
-  const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (r >= a.nrows) return;
-  const int2 m = a.map[r];
-  row_dot<NR>(c128(a.rows) + r * a.R, c128(a.state) + (int64_t)m.y * a.nrhs * a.R, a.R, a.nrhs,
+  const L2PArgs::Level& g = a.lv[level_of<true>(a, blockIdx.x)];
+  const int64_t r = ((int64_t)(blockIdx.x - g.block0) * blockDim.x + threadIdx.x) >> 5;
+  if (r >= g.nrows) return;
+  const int2 m = g.map[r];
+  const int R = g.R;
+  row_dot<NR>(c128(g.rows) + r * R, c128(g.state) + (int64_t)m.y * a.nrhs * R, R, a.nrhs,
               c128(a.us) + (int64_t)m.x * a.nrhs);
 }
 
@@ -305,13 +308,14 @@ __global__ __launch_bounds__(256) void l2p64_kernel(L2PArgs a) {
 // sides per pass over the rows, four rows loaded ahead (one warp per leaf left
 // small bodies two warps per SM).
 template <int NR>
-__global__ __launch_bounds__(C64_T) void p2m64_kernel(P2MRowsArgs a) {
+__global__ __launch_bounds__(C64_T) void p2m64_kernel(const __grid_constant__ P2MRowsArgs a) {
   pdl_begin();
-  const int4 job = a.jobs[blockIdx.x];
-  const int q = blockIdx.y * C64_T + threadIdx.x;
-  if (q >= a.R) return;
-  const double2* row = c128(a.rows) + (int64_t)job.z * a.R + q;
-  double2* st = c128(a.state) + (int64_t)job.w * a.nrhs * a.R + q;
+  const P2MRowsArgs::Level& g = a.lv[level_of<true>(a, blockIdx.x)];
+  const int R = g.R, q = blockIdx.y * C64_T + threadIdx.x;
+  if (q >= R) return;
+  const int4 job = g.jobs[blockIdx.x - g.block0];
+  const double2* row = c128(g.rows) + (int64_t)job.z * R + q;
+  double2* st = c128(g.state) + (int64_t)job.w * a.nrhs * R + q;
   for (int k0 = 0; k0 < a.nrhs; k0 += NR) {
     const double2* f = c128(a.fs) + (int64_t)job.x * a.nrhs;
     double2 acc[NR];
@@ -321,20 +325,20 @@ __global__ __launch_bounds__(C64_T) void p2m64_kernel(P2MRowsArgs a) {
     for (; i + 4 <= job.y; i += 4) {
       double2 v[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = __ldcs(row + (int64_t)(i + j) * a.R);
+      for (int j = 0; j < 4; ++j) v[j] = __ldcs(row + (int64_t)(i + j) * R);
 #pragma unroll
       for (int j = 0; j < 4; ++j)
 #pragma unroll
         for (int k = 0; k < NR; ++k) cfma(acc[k], v[j], f[(int64_t)(i + j) * a.nrhs + min(k0 + k, a.nrhs - 1)]);
     }
     for (; i < job.y; ++i) {
-      const double2 v = __ldcs(row + (int64_t)i * a.R);
+      const double2 v = __ldcs(row + (int64_t)i * R);
 #pragma unroll
       for (int k = 0; k < NR; ++k) cfma(acc[k], v, f[(int64_t)i * a.nrhs + min(k0 + k, a.nrhs - 1)]);
     }
 #pragma unroll
     for (int k = 0; k < NR; ++k)
-      if (k0 + k < a.nrhs) st[(int64_t)(k0 + k) * a.R] = acc[k];
+      if (k0 + k < a.nrhs) st[(int64_t)(k0 + k) * R] = acc[k];
   }
 }
 
@@ -456,17 +460,27 @@ void launch_rows64(const RowsArgs& a, LaunchStream s) {
 }
 
 void launch_l2p64(const L2PArgs& a, LaunchStream s) {
-  if (a.nrows == 0) return;
-  check_rank(a.R);
-  by_rhs(a.nrhs, [&](auto nr) { launch_pdl(l2p64_kernel<nr()>, (unsigned)((a.nrows + 7) / 8), 256, 0, s, a); });
+  for (int l = 0; l < a.nlv; ++l) check_rank(a.lv[l].R);
+  L2PArgs p;
+  const unsigned grid = place_levels(a, p, [](const L2PArgs::Level&) { return true; },
+                                     [](const L2PArgs::Level& g) { return (g.nrows + 7) / 8; });
+  if (grid == 0) return;
+  by_rhs(a.nrhs, [&](auto nr) { launch_pdl(l2p64_kernel<nr()>, grid, 256, 0, s, p); });
   DFMM_CUDA(cudaGetLastError());
 }
 
 void launch_p2m_rows64(const P2MRowsArgs& a, LaunchStream s) {
-  if (a.njobs == 0) return;
-  check_rank(a.R);
-  const dim3 grid((unsigned)a.njobs, (unsigned)((a.R + C64_T - 1) / C64_T));
-  by_rhs(a.nrhs, [&](auto nr) { launch_pdl(p2m64_kernel<nr()>, grid, C64_T, 0, s, a); });
+  int R = 0;
+  for (int l = 0; l < a.nlv; ++l) {
+    check_rank(a.lv[l].R);
+    R = std::max(R, a.lv[l].R);
+  }
+  P2MRowsArgs p;
+  const unsigned n = place_levels(a, p, [](const P2MRowsArgs::Level&) { return true; },
+                                  [](const P2MRowsArgs::Level& g) { return g.njobs; });
+  if (n == 0) return;
+  const dim3 grid(n, (unsigned)((R + C64_T - 1) / C64_T));
+  by_rhs(a.nrhs, [&](auto nr) { launch_pdl(p2m64_kernel<nr()>, grid, C64_T, 0, s, p); });
   DFMM_CUDA(cudaGetLastError());
 }
 

@@ -61,7 +61,6 @@ struct GemmPlan {
   std::vector<int4> groups;        // (op, first pair, count, 0)
   int2* pairs = nullptr;
   std::vector<int32_t> h_dst;      // target row of every pair (host), for tile ordering
-  bool dst_unique = false;         // no two pairs share a target row
   int64_t npairs = 0;
   int fam = 0;                     // profiling family
   __half* img = nullptr;           // tensor-core operator image (tensor form only)
@@ -152,7 +151,9 @@ struct Workspace {
   int nrhs = 0;
   bool external = false;   // buffers carved from caller-provided memory
   DevArena ar;
-  float2 *fs = nullptr, *us = nullptr, *p2l = nullptr;
+  float2 *fs = nullptr, *us = nullptr;
+  std::vector<float2*> p2l;                             // per level: potentials at the P2L check points
+  bool p2l_own = false;                                 // every level has rows of its own (else one array serves all)
   __half *ahi = nullptr, *alo = nullptr;                // split source buffer (tensor form)
   float* ascale = nullptr;                              // its per-row scales
   void *sl = nullptr, *sl_scale = nullptr;              // sliced source buffer and its row scales (sliced form;
@@ -162,7 +163,7 @@ struct Workspace {
   std::vector<std::pair<void*, size_t>> zero_late;      // reset on the side stream, first read by HF M2M
   cudaStream_t side = nullptr;                          // for zero_late, beside P2M and the V list, or the near field
   bool may_fork = false;                                // the workspace lives on, so it may own the side stream
-  cudaEvent_t fork = nullptr, join = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr, ahead = nullptr;   // ahead: P2L potentials
   std::map<std::pair<const void*, int>, std::pair<int4*, int64_t>> tiles;   // key (stage, nrhs * 1024 + columns)
   float2 *f_dev = nullptr, *u_dev = nullptr;            // staging for host applies
   unsigned* status = nullptr;
@@ -174,6 +175,7 @@ struct Workspace {
     for (auto e : pool) cudaEventDestroy(e);
     if (fork) cudaEventDestroy(fork);
     if (join) cudaEventDestroy(join);
+    if (ahead) cudaEventDestroy(ahead);
     if (side) cudaStreamDestroy(side);
   }
   cudaEvent_t ev() {
@@ -374,7 +376,6 @@ void finish_gemm(GemmPlan& g, const std::vector<int32_t>& op, const std::vector<
     for (auto u : used) uops += u;
     g.bytes_fixed = (double)uops * g.M * g.Kd * 8.0;
     g.bytes_rhs = (double)ua * g.Kd * 8.0 + 2.0 * (double)ub * g.M * 8.0;
-    g.dst_unique = ub == n;
   }
   std::vector<int64_t> cnt(g.nops + 1, 0);
   for (int64_t i = 0; i < n; ++i) cnt[op[i] + 1]++;
@@ -1226,6 +1227,28 @@ int64_t max_slice_bytes(const dfmm_plan_s* P) {
   return m;
 }
 
+// Rows (complex elements per right-hand side) that the P2L potentials take: of all levels together
+// (own), so that they can be computed ahead, or of the largest level.
+int64_t p2l_elems(const dfmm_plan_s* P, bool own) {
+  int64_t sum = 0, most = 0;
+  for (const auto& F : P->lf) {
+    const int64_t e = F.n_p2l * 2 * F.R;
+    sum += e;
+    most = std::max(most, e);
+  }
+  return std::max<int64_t>(1, own ? sum : most);
+}
+void set_p2l(const dfmm_plan_s* P, Workspace& W, float2* base, int nrhs, bool own) {
+  W.p2l_own = own || p2l_elems(P, true) == p2l_elems(P, false);
+  W.p2l.assign(P->lf.size(), base);
+  int64_t at = 0;
+  if (W.p2l_own)
+    for (size_t l = 0; l < P->lf.size(); ++l) {
+      W.p2l[l] = base ? base + at * nrhs * P->cw : nullptr;
+      at += P->lf[l].n_p2l * 2 * P->lf[l].R;
+    }
+}
+
 Workspace* get_workspace(dfmm_plan_s* P, cudaStream_t s, int nrhs) {
   std::lock_guard<std::mutex> g(P->ws_mu);
   auto& slot = P->ws[s];
@@ -1242,7 +1265,6 @@ Workspace* get_workspace(dfmm_plan_s* P, cudaStream_t s, int nrhs) {
   W->zero.push_back({W->us, (size_t)N * nrhs * cw * sizeof(float2)});
   W->S.assign(P->nl, nullptr);
   W->T.assign(P->nl, nullptr);
-  int64_t p2l_rows = 1;
   for (int l = 0; l < P->nl; ++l) {
     int64_t rows = 0;
     int R = 0;
@@ -1258,9 +1280,14 @@ Workspace* get_workspace(dfmm_plan_s* P, cudaStream_t s, int nrhs) {
     W->T[l] = ar.alloc<float2>(rows * nrhs * R * cw);
     W->zero.push_back({W->S[l], (size_t)rows * nrhs * R * 8 * cw});
     W->zero.push_back({W->T[l], (size_t)rows * nrhs * R * 8 * cw});
-    p2l_rows = std::max(p2l_rows, P->lf[l].n_p2l * 2 * R);
   }
-  W->p2l = ar.alloc<float2>(p2l_rows * nrhs * cw);
+  try {
+    set_p2l(P, *W, ar.alloc<float2>(p2l_elems(P, true) * nrhs * cw), nrhs, true);
+  } catch (const Error& e) {   // no room for every level's: one array serves them in turn
+    if (e.code != DFMM_ERR_OOM) throw;
+    cudaGetLastError();
+    set_p2l(P, *W, ar.alloc<float2>(p2l_elems(P, false) * nrhs * cw), nrhs, false);
+  }
   if (P->opt.m2l_mode == 2) {
     // split arrays: 2 values per complex element, 2 bytes each (4 for the TF32 split)
     int64_t e = max_source_elems(P) * nrhs * 2 * (P->opt.tc_precision == 2 ? 2 : 1);
@@ -1374,7 +1401,6 @@ struct WaveGemm {
   int dst_ld;
   int nrhs;
   bool split;   // the stage's source buffer must be split first
-  int store;
 };
 
 // Wave filter of the batched form: run_apply acts only on the steps of one wave
@@ -1410,8 +1436,8 @@ struct Runner {
   }
 
   template <class Fn>
-  void launch(int fam, double flops, double bytes, Fn&& fn) {
-    if (count) { ++*count; return; }
+  void launch(int fam, double flops, double bytes, Fn&& fn, int launches = 1) {
+    if (count) { *count += launches; return; }
     if (skip()) return;
     ProfScope ps(W, s, fam, flops, bytes);
     fn();
@@ -1421,10 +1447,8 @@ struct Runner {
 
   // src_key names the source buffer (kSrcS / kSrcT + level, -1 for one used once); a
   // stage whose source is the buffer split for the previous stage reuses that split.
-  // first: no earlier stage of the apply writes dst (it holds zeros), so a stage whose
-  // target rows are all distinct may store its results instead of adding them.
   void gemm(const GemmPlan& g, const float2* src, int src_ld, int64_t src_rows, float2* dst, int dst_ld,
-            int src_key, bool first = false) {
+            int src_key) {
     if (g.npairs == 0) return;
     const bool few = few_columns(P, g, nrhs);
     const bool tc = !few && on_tensor_cores(P, g);
@@ -1437,8 +1461,7 @@ struct Runner {
     if (count) { count[0] += split ? 2 : 1; return; }
     if (skip()) return;
     if (ctl && ctl->collect && cx) {   // the batched form merges this stage with the other plans' same stage
-      ctl->collect->push_back(WaveGemm{P, W, &g, src, src_ld, src_rows, dst, dst_ld, nrhs, split,
-                                       (first && g.dst_unique) ? 1 : 0});
+      ctl->collect->push_back(WaveGemm{P, W, &g, src, src_ld, src_rows, dst, dst_ld, nrhs, split});
       return;
     }
     auto t = tiles_for(P, W, g, nrhs, tile_columns(P, g, nrhs, W->sl != nullptr), s);
@@ -1454,7 +1477,6 @@ struct Runner {
     a.src_ld = src_ld;
     a.dst_ld = dst_ld;
     a.nrhs = nrhs;
-    a.store = (first && g.dst_unique) ? 1 : 0;
     a.wait_test = P->opt.wait_test ? 1 : 0;
     a.stages = nullptr;
     if (tc) {
@@ -1492,13 +1514,13 @@ constexpr int kSrcS = 0, kSrcT = 64;   // source keys: outgoing / incoming state
 constexpr int64_t kWaveStart = 0;
 inline int64_t wave_p2m(int64_t lw) { return 1000 + (lw + 64) * 4; }
 inline int64_t wave_lf_m2m(int64_t lw) { return 1000 + (lw + 64) * 4 + 1; }
+inline int64_t wave_lf_v(int64_t lw) { return 1000 + (lw + 64) * 4 + 2; }
 constexpr int64_t kWaveTopV = 2000;
 inline int64_t wave_hf_m2m(int64_t lw) { return 3000 + (lw + 64) * 4; }
 inline int64_t wave_hf_m2l(int64_t lw) { return 3000 + (lw + 64) * 4 + 1; }
 inline int64_t wave_hf_l2l(int64_t lw) { return 4000 + (64 - lw) * 4; }
 inline int64_t wave_lf_down(int64_t lw, int k) { return 5000 + (64 - lw) * 8 + k; }
-inline int64_t wave_l2p(int64_t lw) { return 6000 + (64 - lw); }
-constexpr int64_t kWaveM2P = 6500, kWaveP2P = 7000, kWaveEnd = 8000;
+constexpr int64_t kWaveL2P = 6000, kWaveM2P = 6500, kWaveP2P = 7000, kWaveEnd = 8000;
 
 void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_t stream, int64_t* count = nullptr,
                Workspace* ext = nullptr, WaveCtl* ctl = nullptr) {
@@ -1531,6 +1553,7 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
       DFMM_CUDA(cudaStreamCreateWithFlags(&W->side, cudaStreamNonBlocking));
       DFMM_CUDA(cudaEventCreateWithFlags(&W->fork, cudaEventDisableTiming));
       DFMM_CUDA(cudaEventCreateWithFlags(&W->join, cudaEventDisableTiming));
+      DFMM_CUDA(cudaEventCreateWithFlags(&W->ahead, cudaEventDisableTiming));
     }
     DFMM_CUDA(cudaEventRecord(W->fork, s));
     DFMM_CUDA(cudaStreamWaitEvent(W->side, W->fork, 0));
@@ -1572,36 +1595,100 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
     else if (P->opt.p2p_mode == 2) launch_p2p_fast(a, N, st);
     else launch_p2p(a, st);
   };
-  // a small apply leaves the device half empty: its near field runs beside the far field
+  auto p2l_eval = [&](int l, LaunchStream st) {
+    LFLevel& F = P->lf[l];
+    P2CArgs a{};
+    a.jobs = F.p2l_jobs;
+    a.njobs = F.n_p2l;
+    a.shifts = F.p2l_shifts;
+    a.chk = F.chk_b2;
+    a.nchk = 2 * F.r;
+    a.ld = 2 * F.R;
+    a.pts = P->pts_local;
+    a.fs = W->fs;
+    a.out = W->p2l[l];
+    a.nrhs = nrhs;
+    a.chk64 = F.chk64;
+    a.halves = F.p2l_halves;
+    a.trig = P->trig;
+    a.pts_lo = P->pts_lo;
+    if (P->fp64) launch_p2c64(a, st);
+    else launch_p2c(a, st);
+  };
+  auto m2p = [&](size_t k, LaunchStream st) {
+    auto& g = P->m2p[k];
+    RowsArgs a;
+    a.jobs = g.jobs;
+    a.njobs = g.njobs;
+    a.rows = g.rows;
+    a.state = W->S[g.src_level];
+    a.R = g.R;
+    a.nrhs = nrhs;
+    a.us = W->us;
+    if (P->fp64) launch_rows64(a, st);
+    else launch_rows(a, st);
+  };
+  // A small apply leaves the device half empty: what needs only the points and the outgoing states
+  // of the LF levels (P2L potentials, near field, M2P) runs beside the far field's chain (adaptive
+  // bodies with P2L and M2P also in line: clustered sphere of 8, 20,000 points in leaves of 16, 776
+  // -> 646 us together with the V lists below; 2 wavelengths, 3,000 points, 180 -> 113; cube of 4, 4
+  // right-hand sides, FP64, 3.48 -> 3.18 ms).
   const bool beside = !count && !ctl && fused && W->may_fork && !W->prof && N * nrhs <= kBesideNear;
+  const bool p2l_ahead = beside && W->p2l_own;
+  bool p2l_wait = false;   // the chain has yet to wait for the P2L potentials
   if (beside) {
     fork_side();
+    if (p2l_ahead) {
+      for (int l = P->l_lf0; l < nl; ++l)
+        if (P->lf[l].n_p2l) {
+          p2l_eval(l, W->side);
+          p2l_wait = true;
+        }
+      if (p2l_wait) DFMM_CUDA(cudaEventRecord(W->ahead, W->side));
+    }
     near_field(W->side);
-    DFMM_CUDA(cudaEventRecord(W->join, W->side));
+    if (P->m2p.empty()) DFMM_CUDA(cudaEventRecord(W->join, W->side));
   }
-  // 1. LF upward: P2M at leaves, LF-M2M from the level below
+  // the point kernels of FP32 take the levels of rank up to 128 and the others in a launch each
+  bool narrow = false, wide = false;
+  for (int l = P->l_lf0; l < nl; ++l)
+    if (P->lf[l].n_l2p) (P->lf[l].R <= 128 ? narrow : wide) = true;
+  const int widths = P->fp64 || !narrow || !wide ? 1 : 2;
+  // 1. LF upward: P2M at the leaves of every level, through their points' rows, then LF-M2M level by level
+  {
+    P2MRowsArgs a;
+    a.nlv = 0;
+    double fl = 0.0, by = 0.0;
+    for (int l = P->l_lf0; l < nl; ++l) {
+      LFLevel& F = P->lf[l];
+      if (!F.n_l2p) continue;
+      if (a.nlv == P2MRowsArgs::kMax) throw Error(DFMM_ERR_UNSUPPORTED, "too many levels");
+      if (!count) a.lv[a.nlv] = {F.l2p_jobs, F.n_l2p, F.p2m_rows, W->S[l], F.R, 0};
+      ++a.nlv;
+      fl += 8.0 * F.r * F.npts * nrhs;
+      by += F.npts * (8.0 * F.R + 8.0 * nrhs) + F.n_l2p * 8.0 * F.R * nrhs;
+    }
+    if (a.nlv)
+      R.at(wave_p2m(lw(nl - 1))).launch(F_P2M_EVAL, fl, by, [&] {
+        a.fs = W->fs;
+        a.nrhs = nrhs;
+        if (P->fp64) launch_p2m_rows64(a, s);
+        else launch_p2m_rows(a, s);
+      }, widths);
+  }
   for (int l = nl - 1; l >= P->l_lf0; --l) {
     LFLevel& F = P->lf[l];
-    if (F.n_l2p) {   // P2M: every leaf of this level, through its points' rows
-      R.at(wave_p2m(lw(l))).launch(F_P2M_EVAL, 8.0 * F.r * F.npts * nrhs, F.npts * (8.0 * F.R + 8.0 * nrhs) + F.n_l2p * 8.0 * F.R * nrhs,
-               [&] {
-                 P2MRowsArgs a;
-                 a.jobs = F.l2p_jobs;
-                 a.njobs = F.n_l2p;
-                 a.rows = F.p2m_rows;
-                 a.fs = W->fs;
-                 a.state = W->S[l];
-                 a.R = F.R;
-                 a.nrhs = nrhs;
-                 if (P->fp64) launch_p2m_rows64(a, s);
-                 else launch_p2m_rows(a, s);
-               });
-    }
     if (l + 1 < nl) R.at(wave_lf_m2m(lw(l))).gemm(F.m2m, S(l + 1), P->lf[l + 1].R, P->lf[l + 1].nbox, S(l), F.R, kSrcS + l + 1);
+    // The V list of each level as soon as its outgoing states are complete, so that the next M2M, which
+    // reads the same states, reuses their split; the L2L into the level then adds to it.
+    if (l > P->l_lf0) R.at(wave_lf_v(lw(l))).gemm(F.v, S(l), F.R, F.nbox, T(l), F.R, kSrcS + l);
   }
-  // M2L of each level as soon as its outgoing states are complete, so that the
-  // next M2M, which reads the same states, reuses their split.  The V list of the
-  // top LF level: its L2L (from HF, summed over directions) adds anyway.
+  if (beside && !P->m2p.empty()) {   // S is complete
+    DFMM_CUDA(cudaEventRecord(W->fork, s));
+    DFMM_CUDA(cudaStreamWaitEvent(W->side, W->fork, 0));
+    for (size_t k = 0; k < P->m2p.size(); ++k) m2p(k, W->side);
+    DFMM_CUDA(cudaEventRecord(W->join, W->side));
+  }
   if (P->l_lf0 < nl)
     R.at(kWaveTopV).gemm(P->lf[P->l_lf0].v, S(P->l_lf0), P->lf[P->l_lf0].R, P->lf[P->l_lf0].nbox, T(P->l_lf0),
            P->lf[P->l_lf0].R, kSrcS + P->l_lf0);
@@ -1628,66 +1715,47 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
       if (P->l_top >= 0)
         R.at(wave_lf_down(lw(l), 0)).gemm(F.l2l, T(P->l1), P->hf[P->l1].R, (int64_t)P->hf[P->l1].in_keys.size(), T(l), F.R, kSrcT + P->l1);
     } else {
-      R.at(wave_lf_down(lw(l), 0)).gemm(F.l2l, T(l - 1), P->lf[l - 1].R, P->lf[l - 1].nbox, T(l), F.R, kSrcT + l - 1,
-                                        true);
-      R.at(wave_lf_down(lw(l), 1)).gemm(F.v, S(l), F.R, F.nbox, T(l), F.R, kSrcS + l);
+      R.at(wave_lf_down(lw(l), 0)).gemm(F.l2l, T(l - 1), P->lf[l - 1].R, P->lf[l - 1].nbox, T(l), F.R, kSrcT + l - 1);
     }
     if (F.n_p2l) {
       double ev = (double)F.npts_x * 2 * F.r;
-      R.at(wave_lf_down(lw(l), 2)).launch(F_P2L_EVAL, ev * (16 + 8.0 * nrhs), F.npts_x * (16.0 + 8.0 * nrhs) + F.n_p2l * 2.0 * F.R * 8 * nrhs, [&] {
-        P2CArgs a{};
-        a.jobs = F.p2l_jobs;
-        a.njobs = F.n_p2l;
-        a.shifts = F.p2l_shifts;
-        a.chk = F.chk_b2;
-        a.nchk = 2 * F.r;
-        a.ld = 2 * F.R;
-        a.pts = P->pts_local;
-        a.fs = W->fs;
-        a.out = W->p2l;
-        a.nrhs = nrhs;
-        a.chk64 = F.chk64;
-        a.halves = F.p2l_halves;
-        a.trig = P->trig;
-        a.pts_lo = P->pts_lo;
-        if (P->fp64) launch_p2c64(a, s);
-        else launch_p2c(a, s);
-      });
-      R.at(wave_lf_down(lw(l), 3)).gemm(F.p2l, count ? nullptr : W->p2l, F.p2l.Kd, F.n_p2l * F.p2l_halves, T(l), F.R, -1);
+      if (p2l_ahead) {
+        if (p2l_wait) DFMM_CUDA(cudaStreamWaitEvent(s, W->ahead, 0));
+        p2l_wait = false;
+      } else {
+        R.at(wave_lf_down(lw(l), 2)).launch(F_P2L_EVAL, ev * (16 + 8.0 * nrhs), F.npts_x * (16.0 + 8.0 * nrhs) + F.n_p2l * 2.0 * F.R * 8 * nrhs,
+                 [&] { p2l_eval(l, s); });
+      }
+      R.at(wave_lf_down(lw(l), 3)).gemm(F.p2l, count ? nullptr : W->p2l[l], F.p2l.Kd, F.n_p2l * F.p2l_halves, T(l), F.R, -1);
     }
   }
   // 5. L2P at every leaf, M2P over the W list
-  for (int l = P->l_lf0; l < nl; ++l) {
-    LFLevel& F = P->lf[l];
-    if (!F.n_l2p) continue;
-    R.at(wave_l2p(lw(l))).launch(F_L2P, 8.0 * F.r * F.npts * nrhs, F.npts * (8.0 * F.R + 16.0 * nrhs) + F.n_l2p * 8.0 * F.R * nrhs, [&] {
-      L2PArgs a;
-      a.map = F.l2p_map;
-      a.nrows = F.n_l2p_rows;
-      a.rows = F.l2p_rows;
-      a.state = W->T[l];
-      a.R = F.R;
-      a.nrhs = nrhs;
-      a.us = W->us;
-      if (P->fp64) launch_l2p64(a, s);
-      else launch_l2p(a, s);
-    });
+  {
+    L2PArgs a;
+    a.nlv = 0;
+    double fl = 0.0, by = 0.0;
+    for (int l = P->l_lf0; l < nl; ++l) {
+      LFLevel& F = P->lf[l];
+      if (!F.n_l2p) continue;
+      if (!count) a.lv[a.nlv] = {F.l2p_map, F.n_l2p_rows, F.l2p_rows, W->T[l], F.R, 0};
+      ++a.nlv;
+      fl += 8.0 * F.r * F.npts * nrhs;
+      by += F.npts * (8.0 * F.R + 16.0 * nrhs) + F.n_l2p * 8.0 * F.R * nrhs;
+    }
+    if (a.nlv)
+      R.at(kWaveL2P).launch(F_L2P, fl, by, [&] {
+        a.us = W->us;
+        a.nrhs = nrhs;
+        if (P->fp64) launch_l2p64(a, s);
+        else launch_l2p(a, s);
+      }, widths);
   }
-  for (size_t k = 0; k < P->m2p.size(); ++k) {
-    auto& g = P->m2p[k];
-    R.at(kWaveM2P + (int64_t)k).launch(F_M2P, 8.0 * P->lf[g.src_level].r * g.nrows * nrhs, g.nrows * (8.0 * g.R + 16.0 * nrhs), [&] {
-      RowsArgs a;
-      a.jobs = g.jobs;
-      a.njobs = g.njobs;
-      a.rows = g.rows;
-      a.state = W->S[g.src_level];
-      a.R = g.R;
-      a.nrhs = nrhs;
-      a.us = W->us;
-      if (P->fp64) launch_rows64(a, s);
-      else launch_rows(a, s);
-    });
-  }
+  if (!beside)
+    for (size_t k = 0; k < P->m2p.size(); ++k) {
+      auto& g = P->m2p[k];
+      R.at(kWaveM2P + (int64_t)k).launch(F_M2P, 8.0 * P->lf[g.src_level].r * g.nrows * nrhs, g.nrows * (8.0 * g.R + 16.0 * nrhs),
+               [&] { m2p(k, s); });
+    }
   // 6. near field
   if (beside) DFMM_CUDA(cudaStreamWaitEvent(s, W->join, 0));
   else
@@ -1711,9 +1779,9 @@ std::vector<const GemmPlan*> all_gemms(dfmm_plan_s* P) {
 // [base, base + bytes): the device status word (at offset 0), state buffers,
 // staging buffers and the work tiles of every stage (copied in on `s`).  No device memory is allocated.  With
 // base == nullptr nothing is laid out or copied: the return value is the
-// number of bytes the layout needs.  slices: with the sliced form's source
-// buffer; without it the plan's sliced stages run on the CUDA cores.
-size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaStream_t s, Workspace& W, bool slices) {
+// number of bytes the layout needs.  full: with the sliced form's source buffer,
+// without which the plan's sliced stages run on the CUDA cores, and P2L rows for every level.
+size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaStream_t s, Workspace& W, bool full) {
   size_t off = 0;
   auto take = [&](size_t n) -> char* {
     off = (off + 255) & ~(size_t)255;
@@ -1733,7 +1801,6 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
   W.zero.push_back({W.us, (size_t)N * nrhs * cb});
   W.S.assign(P->nl, nullptr);
   W.T.assign(P->nl, nullptr);
-  size_t p2l_rows = 1;
   for (int l = 0; l < P->nl; ++l) {
     if (l >= P->l_lf0) {
       size_t b = (size_t)P->lf[l].nbox * nrhs * P->lf[l].R * cb;
@@ -1741,7 +1808,6 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
       W.T[l] = (float2*)take(b);
       W.zero.push_back({W.S[l], b});
       W.zero.push_back({W.T[l], b});
-      p2l_rows = std::max(p2l_rows, (size_t)P->lf[l].n_p2l * 2 * P->lf[l].R);
     } else if (P->l_top >= 0 && l >= P->l_top) {
       size_t so = P->hf[l].out_keys.size(), si = P->hf[l].in_keys.size();
       size_t R = P->hf[l].R;
@@ -1749,14 +1815,14 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
       if (si) { W.T[l] = (float2*)take(si * nrhs * R * cb); W.zero.push_back({W.T[l], si * nrhs * R * cb}); }
     }
   }
-  W.p2l = (float2*)take(p2l_rows * nrhs * cb);
+  set_p2l(P, W, (float2*)take((size_t)p2l_elems(P, full) * nrhs * cb), nrhs, full);
   if (P->opt.m2l_mode == 2) {
     size_t e = (size_t)max_source_elems(P) * nrhs * 2 * (P->opt.tc_precision == 2 ? 2 : 1);
     W.ahi = (__half*)take(e * 4);
     W.alo = W.ahi + e;
     W.ascale = (float*)take((size_t)max_source_rows(P) * nrhs * 4);
   }
-  slices = slices && P->sliced;
+  const bool slices = full && P->sliced;
   if (slices) {
     W.sl = take((size_t)max_slice_bytes(P) * nrhs);
     W.sl_scale = take((size_t)max_source_rows(P) * nrhs * 8);
@@ -1784,27 +1850,27 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
 }
 
 // Device bytes of one apply's workspace with nrhs right-hand sides: the least an
-// apply runs in, or (slices) with room for the sliced form of plans that have it.
-int64_t workspace_bytes(dfmm_plan_s* P, int nrhs, bool slices) {
+// apply runs in, or (full) with room for what makes it faster.
+int64_t workspace_bytes(dfmm_plan_s* P, int nrhs, bool full) {
   Workspace W;
-  return (int64_t)carve_workspace(P, nrhs, nullptr, 0, nullptr, W, slices);
+  return (int64_t)carve_workspace(P, nrhs, nullptr, 0, nullptr, W, full);
 }
 
-// A carved workspace of its own in `ar`: with the slices, or where they do not fit the device, without.
+// A carved workspace of its own in `ar`: the full layout, or where it does not fit the device, the least.
 void own_workspace(dfmm_plan_s* P, int nrhs, DevArena& ar, cudaStream_t s, Workspace& W) {
-  bool slices = P->sliced;
-  size_t bytes = (size_t)workspace_bytes(P, nrhs, slices);
+  bool full = true;
+  size_t bytes = (size_t)workspace_bytes(P, nrhs, full);
   char* base = nullptr;
   try {
     base = ar.alloc<char>((int64_t)bytes);
   } catch (const Error& e) {
-    if (!slices || e.code != DFMM_ERR_OOM) throw;
+    if (e.code != DFMM_ERR_OOM) throw;
     cudaGetLastError();
-    slices = false;
+    full = false;
     bytes = (size_t)workspace_bytes(P, nrhs, false);
     base = ar.alloc<char>((int64_t)bytes);
   }
-  carve_workspace(P, nrhs, base, bytes, s, W, slices);
+  carve_workspace(P, nrhs, base, bytes, s, W, full);
 }
 
 // Operator images of every translation stage for the tensor-core form.
@@ -1984,8 +2050,8 @@ int apply_with_scratch(dfmm_plan_s* P, const void* f, void* u, int nrhs, cudaStr
     if (dev != P->device) return fail(DFMM_ERR_INVALID, "the plan belongs to another device");
     Workspace W;
     // the sliced form where the scratch holds its source slices as well
-    const bool slices = P->sliced && (size_t)workspace_bytes(P, nrhs, true) <= bytes;
-    carve_workspace(P, nrhs, (char*)scratch, bytes, stream, W, slices);
+    const bool full = (size_t)workspace_bytes(P, nrhs, true) <= bytes;
+    carve_workspace(P, nrhs, (char*)scratch, bytes, stream, W, full);
     run_apply(P, (const float2*)f, (float2*)u, nrhs, stream, nullptr, &W);
     return DFMM_OK;
   });
@@ -2108,7 +2174,6 @@ dfmm_batch_s::Merged& merged_for(dfmm_batch_s* B, int64_t wave, int M, int Kd, i
     c.op_scale = w.g->op_scale;
     c.dst = w.dst;
     c.nrhs = w.nrhs;
-    c.store = w.store;
     st.push_back(c);
     for (int v = 0; v < kBatchOrders; ++v) batch_tiles(*w.g, w.nrhs, v, tl[v], (int)i);
   }

@@ -244,7 +244,6 @@ __device__ __forceinline__ CxStage stage_of(const GemmArgs& a, const TcArgs& t, 
   s.op_scale = t.op_scale;
   s.dst = a.dst;
   s.nrhs = a.nrhs;
-  s.store = a.store;
   return s;
 }
 
@@ -563,10 +562,7 @@ __global__ __launch_bounds__(CX_THREADS, 1) void gemm_cx_kernel(GemmArgs a, TcAr
                 const float im0 = (__uint_as_float(vi[r]) + __uint_as_float(wi[r])) * cc;
                 const float re1 = (__uint_as_float(vr[r + 1]) + __uint_as_float(wr[r + 1])) * cc;
                 const float im1 = (__uint_as_float(vi[r + 1]) + __uint_as_float(wi[r + 1])) * cc;
-                if (o) {
-                  if (sg.store) *(float4*)(o + f) = make_float4(re0, im0, re1, im1);
-                  else red_add4(o + f, re0, im0, re1, im1);
-                }
+                if (o) red_add4(o + f, re0, im0, re1, im1);
               }
             }
           }

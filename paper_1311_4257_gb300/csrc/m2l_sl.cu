@@ -559,17 +559,11 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
               if constexpr (S == 3) {
                 const float c = cs[2 * b + h];
                 const float y0 = v[0] * so * c, y1 = v[1] * so * c, y2 = v[2] * so * c, y3 = v[3] * so * c;
-                if (a.store) *(float4*)o = make_float4(y0, y1, y2, y3);
-                else red_add4(o, y0, y1, y2, y3);
+                red_add4(o, y0, y1, y2, y3);
               } else {
                 const double c = so * cs[2 * b + h];
-                if (a.store) {
-                  *(double2*)o = make_double2(v[0] * c, v[1] * c);
-                  *(double2*)(o + 2) = make_double2(v[2] * c, v[3] * c);
-                } else {
 #pragma unroll
-                  for (int e = 0; e < 4; ++e) red_add_f64(o + e, v[e] * c);
-                }
+                for (int e = 0; e < 4; ++e) red_add_f64(o + e, v[e] * c);
               }
             }
           }

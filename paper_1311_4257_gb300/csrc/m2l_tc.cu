@@ -383,13 +383,8 @@ __global__ __launch_bounds__(TC_THREADS, 1) void gemm_tc_kernel(GemmArgs a, TcAr
               const float a1 = (__uint_as_float(v[4 * j + 1]) + __uint_as_float(w[4 * j + 1])) * cA;
               const float b0 = (__uint_as_float(v[4 * j + 2]) + __uint_as_float(w[4 * j + 2])) * cB;
               const float b1 = (__uint_as_float(v[4 * j + 3]) + __uint_as_float(w[4 * j + 3])) * cB;
-              if (a.store) {
-                if (oA) *(float2*)(oA + c) = make_float2(a0, a1);
-                if (oB) *(float2*)(oB + c) = make_float2(b0, b1);
-              } else {
-                if (oA) red_add2(oA + c, a0, a1);
-                if (oB) red_add2(oB + c, b0, b1);
-              }
+              if (oA) red_add2(oA + c, a0, a1);
+              if (oB) red_add2(oB + c, b0, b1);
             }
           }
         }
