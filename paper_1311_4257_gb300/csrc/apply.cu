@@ -17,10 +17,12 @@
 //  * p2p_fast_kernel: the near field (U lists) on FP32 coordinates, with the
 //    exact plan-time corrections of the close pairs (p2p_close_kernel,
 //    p2p_close_apply_kernel); p2p_kernel: the same on double-float coordinates.
+#include <algorithm>
 #include <type_traits>
 
 #include "apply.h"
 #include "pdl.h"
+#include "tcgen05.cuh"
 
 namespace dfmm {
 
@@ -297,7 +299,34 @@ __global__ __launch_bounds__(256) void rows_kernel(RowsArgs a) {
   }
 }
 
-// L2P as a flat stream of rows: warp w evaluates the point rows 2w and 2w+1
+// Sums of N values over the warp: every exchange halves the values a lane holds, so N values take
+// N - 1 + (5 - log2 N) exchanges (N: 5 N).  Returns the sum of value lane / (32 / N), by the same
+// tree as five xor steps per value.
+template <int N>
+__device__ __forceinline__ float warp_sums(float (&v)[N]) {
+  const int lane = threadIdx.x & 31;
+  int o = 16;
+#pragma unroll
+  for (int n = N / 2; n > 0; n >>= 1, o >>= 1)
+#pragma unroll
+    for (int j = 0; j < n; ++j) {
+      const bool up = lane & o;
+      const float mine = up ? v[j + n] : v[j], theirs = up ? v[j] : v[j + n];
+      v[j] = mine + __shfl_xor_sync(0xffffffffu, theirs, o);
+    }
+#pragma unroll
+  for (int p = 16 / N; p > 0; p >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], p);
+  return v[0];
+}
+
+__device__ __forceinline__ void row_dot(float2& c, float4 x, float4 y) {
+  c.x = fmaf(x.x, y.x, fmaf(-x.y, y.y, c.x));
+  c.y = fmaf(x.x, y.y, fmaf(x.y, y.x, c.y));
+  c.x = fmaf(x.z, y.z, fmaf(-x.w, y.w, c.x));
+  c.y = fmaf(x.z, y.w, fmaf(x.w, y.z, c.y));
+}
+
+// L2P of one right-hand side as a flat stream of rows: warp w evaluates the point rows 2w and 2w+1
 // (1 KB each at rank 128, loaded together as float4 before any arithmetic);
 // the state rows they dot with are shared by the points of a leaf and mostly
 // hit in L1.  Two rows per warp keep the registers low and the warps many:
@@ -330,94 +359,177 @@ __global__ __launch_bounds__(256) void l2p_kernel(const __grid_constant__ L2PArg
 #pragma unroll
   for (int j = 0; j < L2P_ROWS; ++j) {
     if (m[j].x < 0) continue;   // warp-uniform
-    const float4* st = (const float4*)(g.state + (int64_t)m[j].y * a.nrhs * R);
-    for (int k = 0; k < a.nrhs; ++k) {
-      float2 acc = make_float2(0.f, 0.f);
+    const float4* st = (const float4*)(g.state + (int64_t)m[j].y * R);
+    float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int t = 0; t < Q; ++t) {
+      const int q = lane + 32 * t;
+      if (q < R2) row_dot(acc, v[j][t], st[q]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+    }
+    if (lane == 0) red_add2((float*)(a.us + m[j].x), acc.x, acc.y);   // beside the near field
+  }
+}
+
+// L2P of several right-hand sides, a block of four warps per leaf.  The leaf's state rows,
+// L2P_KS right-hand sides at a time, go to shared memory while each warp loads its first two
+// point rows, so a leaf waits for memory once; a warp dots two rows with L2P_KB states at a time
+// and its next two rows are in flight meanwhile.  Ellipsoid of 32 wavelengths, 16 right-hand sides:
+// 0.140 -> 0.080 ms (0.04 for the FMAs and shared-memory reads; in the flat form every four
+// right-hand sides waited for their states in L2, 72% of the stalls); torus of 40 with 3: 0.073 ->
+// 0.072; sphere of 16 with 4 (apply): 943 -> 923 us.
+constexpr int L2P_KS = 16, L2P_KB = 4, L2P_LEAF_THREADS = 128;
+
+template <int Q, bool MANY>
+__global__ __launch_bounds__(L2P_LEAF_THREADS) void l2p_leaf_kernel(const __grid_constant__ L2PArgs a) {
+  pdl_begin();
+  extern __shared__ float4 sst[];   // [right-hand side][R / 2]
+  const L2PArgs::Level& g = a.lv[level_of<MANY>(a, blockIdx.x)];
+  const int4 job = g.jobs[blockIdx.x - g.block0];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int R2 = g.R / 2, nrhs = a.nrhs;
+  const float4* rows = (const float4*)g.rows + (int64_t)job.z * R2;
+  const float4* st = (const float4*)g.state + (int64_t)job.w * nrhs * R2;
+  auto load = [&](float4 (&v)[2][Q], int i) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
 #pragma unroll
       for (int t = 0; t < Q; ++t) {
         const int q = lane + 32 * t;
-        if (q < R2) {
-          const float4 sv = st[(int64_t)k * R2 + q];
-          acc.x = fmaf(v[j][t].x, sv.x, fmaf(-v[j][t].y, sv.y, acc.x));
-          acc.y = fmaf(v[j][t].x, sv.y, fmaf(v[j][t].y, sv.x, acc.y));
-          acc.x = fmaf(v[j][t].z, sv.z, fmaf(-v[j][t].w, sv.w, acc.x));
-          acc.y = fmaf(v[j][t].z, sv.w, fmaf(v[j][t].w, sv.z, acc.y));
-        }
+        v[j][t] = i + j < job.y && q < R2 ? rows[(int64_t)(i + j) * R2 + q] : make_float4(0.f, 0.f, 0.f, 0.f);
       }
+  };
+  for (int kc = 0; kc < nrhs; kc += L2P_KS) {
+    const int nk = min(L2P_KS, nrhs - kc);
+    if (kc) __syncthreads();   // the previous states are consumed
+    for (int e = threadIdx.x; e < nk * R2; e += L2P_LEAF_THREADS)
+      tc::cp_async16(tc::smem_u32(sst + e), st + (int64_t)kc * R2 + e);
+    float4 nxt[2][Q];
+    load(nxt, 2 * warp);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    for (int i = 2 * warp; i < job.y; i += L2P_LEAF_THREADS / 16) {
+      float4 v[2][Q];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-      }
-      if (lane == 0) {
-        red_add2((float*)(a.us + (int64_t)m[j].x * a.nrhs + k), acc.x, acc.y);   // beside the near field
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int t = 0; t < Q; ++t) v[j][t] = nxt[j][t];
+      load(nxt, i + L2P_LEAF_THREADS / 16);
+      for (int k0 = 0; k0 < nk; k0 += L2P_KB) {
+        float2 acc[2][L2P_KB];
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+          for (int kk = 0; kk < L2P_KB; ++kk) acc[j][kk] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int t = 0; t < Q; ++t) {
+          const int q = lane + 32 * t;
+          if (q < R2) {
+#pragma unroll
+            for (int kk = 0; kk < L2P_KB; ++kk) {   // a missing right-hand side repeats the last one
+              const float4 sv = sst[min(k0 + kk, nk - 1) * R2 + q];
+              row_dot(acc[0][kk], v[0][t], sv);
+              row_dot(acc[1][kk], v[1][t], sv);
+            }
+          }
+        }
+        __syncwarp();
+        constexpr int N = 4 * L2P_KB;
+        float p[N];
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+          for (int kk = 0; kk < L2P_KB; ++kk) {
+            p[2 * (j * L2P_KB + kk)] = acc[j][kk].x;
+            p[2 * (j * L2P_KB + kk) + 1] = acc[j][kk].y;
+          }
+        const float re = warp_sums<N>(p);
+        const float im = __shfl_down_sync(0xffffffffu, re, 32 / N);
+        const int slot = lane / (32 / N), j = slot / (2 * L2P_KB), kk = (slot / 2) % L2P_KB;
+        if (lane % (64 / N) == 0 && k0 + kk < nk && i + j < job.y)   // beside the near field
+          red_add2((float*)(a.us + (int64_t)(job.x + i + j) * nrhs + kc + k0 + kk), re, im);
       }
     }
   }
 }
 
-// P2M through rows: one warp per leaf, lane l owns the state entries
-// 2 (l + 32 t), 2 (l + 32 t) + 1 (float4 loads); the leaf's point rows are read
-// 4 at a time (4 KB in flight per warp) and weighted by the points' densities
-// (one broadcast load per point and right-hand side).  KB right-hand sides are
-// accumulated per pass over the rows: 1 for a single right-hand side, whose
-// accumulators then take a quarter of the registers, so that more warps
-// (more rows in flight) fit on an SM.
+// P2M through rows: lane l of a warp owns the state entries 2 (l + 32 t), 2 (l + 32 t) + 1
+// (float4 loads) of a leaf for KB right-hand sides; the leaf's point rows are read
+// 4 at a time (4 KB in flight per warp) together with the points' densities (a broadcast
+// load per point and right-hand side).  The warps of a leaf's further right-hand sides are
+// neighbours and find its rows in L1: passes over the rows from one warp, 4 right-hand sides each,
+// read them from memory again and waited for the densities (ellipsoid of 32 wavelengths, 16
+// right-hand sides: 0.207 -> 0.105 ms; two per warp instead of four: 0.155).  A single right-hand side
+// keeps the densities out of the row loads (0.240 against 0.266 ms, sphere of 64, 5.9 TB/s).
+constexpr int P2M_KB = 4;
+
 template <int Q, int KB, bool MANY>
 __global__ __launch_bounds__(256) void p2m_rows_kernel(const __grid_constant__ P2MRowsArgs a) {
   pdl_begin();
   const P2MRowsArgs::Level& g = a.lv[level_of<MANY>(a, blockIdx.x)];
-  const int64_t jw = ((int64_t)(blockIdx.x - g.block0) * blockDim.x + threadIdx.x) >> 5;
+  const int nrhs = a.nrhs, parts = KB == 1 ? 1 : (nrhs + KB - 1) / KB;   // KB = 1: one right-hand side
+  const int64_t w = ((int64_t)(blockIdx.x - g.block0) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
+  const int64_t jw = KB == 1 ? w : (uint32_t)w / (uint32_t)parts;
   if (jw >= g.njobs) return;
+  const int k0 = KB == 1 ? 0 : (int)(w - jw * parts) * KB;
   const int4 job = g.jobs[jw];
   const int R2 = g.R / 2;
-  const float4* rows = (const float4*)g.rows;
-  float4* st = (float4*)g.state;
-  for (int k0 = 0; k0 < a.nrhs; k0 += KB) {
-    const int nk = min(KB, a.nrhs - k0);
-    float4 acc[KB][Q];
+  const float4* rows = (const float4*)g.rows + (int64_t)job.z * R2;
+  const float2* fs = a.fs + (int64_t)job.x * nrhs;
+  float4 acc[KB][Q];
 #pragma unroll
-    for (int kk = 0; kk < KB; ++kk)
+  for (int kk = 0; kk < KB; ++kk)
 #pragma unroll
-      for (int t = 0; t < Q; ++t) acc[kk][t] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int i = 0; i < job.y; i += 4) {
-      float4 r[4][Q];
+    for (int t = 0; t < Q; ++t) acc[kk][t] = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int i = 0; i < job.y; i += 4) {
+    float4 r[4][Q];
+    float2 f[4][KB];
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int t = 0; t < Q; ++t) {
-          const int q = lane + 32 * t;
-          r[j][t] = (i + j < job.y && q < R2) ? __ldcs(rows + (int64_t)(job.z + i + j) * R2 + q)
-                                              : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (i + j >= job.y) break;
-#pragma unroll
-        for (int kk = 0; kk < KB; ++kk) {
-          if (kk >= nk) break;
-          const float2 f = a.fs[(int64_t)(job.x + i + j) * a.nrhs + k0 + kk];
-#pragma unroll
-          for (int t = 0; t < Q; ++t) {
-            float4& c = acc[kk][t];
-            const float4 v = r[j][t];
-            c.x = fmaf(v.x, f.x, fmaf(-v.y, f.y, c.x));
-            c.y = fmaf(v.x, f.y, fmaf(v.y, f.x, c.y));
-            c.z = fmaf(v.z, f.x, fmaf(-v.w, f.y, c.z));
-            c.w = fmaf(v.z, f.y, fmaf(v.w, f.x, c.w));
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int kk = 0; kk < KB; ++kk) {
-      if (kk >= nk) break;
+    for (int j = 0; j < 4; ++j) {
+      const bool in = i + j < job.y;
 #pragma unroll
       for (int t = 0; t < Q; ++t) {
         const int q = lane + 32 * t;
-        if (q < R2) st[((int64_t)job.w * a.nrhs + k0 + kk) * R2 + q] = acc[kk][t];
+        const float4* p = rows + (int64_t)(i + j) * R2 + q;
+        r[j][t] = in && q < R2 ? (KB == 1 ? __ldcs(p) : *p) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
+#pragma unroll
+      for (int kk = 0; kk < KB && KB > 1; ++kk)
+        f[j][kk] = in ? fs[(int64_t)(i + j) * nrhs + min(k0 + kk, nrhs - 1)] : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (KB == 1) {
+        if (i + j >= job.y) break;
+        f[j][0] = fs[i + j];
+      }
+#pragma unroll
+      for (int kk = 0; kk < KB; ++kk)
+#pragma unroll
+        for (int t = 0; t < Q; ++t) {
+          float4& c = acc[kk][t];
+          const float4 v = r[j][t];
+          const float2 x = f[j][kk];
+          c.x = fmaf(v.x, x.x, fmaf(-v.y, x.y, c.x));
+          c.y = fmaf(v.x, x.y, fmaf(v.y, x.x, c.y));
+          c.z = fmaf(v.z, x.x, fmaf(-v.w, x.y, c.z));
+          c.w = fmaf(v.z, x.y, fmaf(v.w, x.x, c.w));
+        }
+    }
+  }
+  float4* st = (float4*)g.state + ((int64_t)job.w * nrhs + k0) * R2;
+#pragma unroll
+  for (int kk = 0; kk < KB; ++kk) {
+    if (k0 + kk >= nrhs) break;
+#pragma unroll
+    for (int t = 0; t < Q; ++t) {
+      const int q = lane + 32 * t;
+      if (q < R2) st[(int64_t)kk * R2 + q] = acc[kk][t];
     }
   }
 }
@@ -825,24 +937,32 @@ void launch_l2p(const L2PArgs& a, LaunchStream s) {
   check_ranks(a);
   for (const bool nar : {true, false}) {
     L2PArgs p;
+    int R = 0;
     const unsigned grid = place_levels(a, p, [&](const L2PArgs::Level& g) { return narrow<L2PArgs>(g) == nar; },
-                                       [](const L2PArgs::Level& g) { return (g.nrows + 8 * L2P_ROWS - 1) / (8 * L2P_ROWS); });
+                                       [&](const L2PArgs::Level& g) {
+                                         R = std::max(R, g.R);
+                                         return a.nrhs > 1 ? g.njobs : (g.nrows + 8 * L2P_ROWS - 1) / (8 * L2P_ROWS);
+                                       });
     if (grid == 0) continue;
-    by_levels(p, nar, [&](auto q, auto many) { launch_pdl(l2p_kernel<q(), many()>, grid, 256, 0, s, p); });
+    by_levels(p, nar, [&](auto q, auto many) {
+      if (a.nrhs == 1) launch_pdl(l2p_kernel<q(), many()>, grid, 256, 0, s, p);
+      else launch_pdl(l2p_leaf_kernel<q(), many()>, grid, L2P_LEAF_THREADS, (size_t)std::min(a.nrhs, L2P_KS) * R * 8, s, p);
+    });
   }
   DFMM_CUDA(cudaGetLastError());
 }
 
 void launch_p2m_rows(const P2MRowsArgs& a, LaunchStream s) {
   check_ranks(a);
+  const int kb = a.nrhs == 1 ? 1 : P2M_KB, parts = (a.nrhs + kb - 1) / kb;
   for (const bool nar : {true, false}) {
     P2MRowsArgs p;
     const unsigned grid = place_levels(a, p, [&](const P2MRowsArgs::Level& g) { return narrow<P2MRowsArgs>(g) == nar; },
-                                       [](const P2MRowsArgs::Level& g) { return (g.njobs + 7) / 8; });
+                                       [&](const P2MRowsArgs::Level& g) { return (g.njobs * parts + 7) / 8; });
     if (grid == 0) continue;
     by_levels(p, nar, [&](auto q, auto many) {
       if (a.nrhs == 1) launch_pdl(p2m_rows_kernel<q(), 1, many()>, grid, 256, 0, s, p);
-      else launch_pdl(p2m_rows_kernel<q(), 4, many()>, grid, 256, 0, s, p);
+      else launch_pdl(p2m_rows_kernel<q(), P2M_KB, many()>, grid, 256, 0, s, p);
     });
   }
   DFMM_CUDA(cudaGetLastError());

@@ -173,7 +173,7 @@ unsigned place_levels(const A& a, A& out, Take&& take, Blocks&& blocks) {
       out.lv[out.nlv++].block0 = (unsigned)at;
       at += blocks(a.lv[l]);
     }
-  if (at > INT32_MAX) throw Error(-5, "too many leaves for one launch");
+  if (at > INT32_MAX / 8) throw Error(-5, "too many leaves for one launch");
   return (unsigned)at;
 }
 #ifdef __CUDACC__
@@ -194,6 +194,8 @@ __device__ __forceinline__ int level_of(const A& a, unsigned b) {
 struct L2PArgs {
   static constexpr int kMax = 24;   // LF levels
   struct Level {
+    const int4* jobs;          // leaves: (first point, count, first row, state row)
+    int64_t njobs;
     const int2* map;           // (point, state row) per row
     int64_t nrows;
     const float2* rows;        // [nrows][R]

@@ -1737,7 +1737,7 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
     for (int l = P->l_lf0; l < nl; ++l) {
       LFLevel& F = P->lf[l];
       if (!F.n_l2p) continue;
-      if (!count) a.lv[a.nlv] = {F.l2p_map, F.n_l2p_rows, F.l2p_rows, W->T[l], F.R, 0};
+      if (!count) a.lv[a.nlv] = {F.l2p_jobs, F.n_l2p, F.l2p_map, F.n_l2p_rows, F.l2p_rows, W->T[l], F.R, 0};
       ++a.nlv;
       fl += 8.0 * F.r * F.npts * nrhs;
       by += F.npts * (8.0 * F.R + 16.0 * nrhs) + F.n_l2p * 8.0 * F.R * nrhs;

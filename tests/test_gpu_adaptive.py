@@ -1,6 +1,7 @@
 """Applies on adaptive octrees: the forms that run P2L, M2P and the near field beside the far field's
 chain (a plain apply and a captured one) against the one that runs every step in turn (a profiled
-apply), and P2M and L2P over several levels of different rank in one launch.
+apply), and P2M and L2P over several levels of different rank in one launch, with up to 17 right-hand sides (L2P
+takes them 16 at a time).
 """
 import numpy as np
 import pytest
@@ -19,7 +20,7 @@ def _lib():
     build.build()
 
 
-@pytest.mark.parametrize("eps,nrhs", [(1e-4, 1), (1e-5, 3), (1e-6, 1), (1e-6, 5), (1e-8, 1), (1e-8, 4)])
+@pytest.mark.parametrize("eps,nrhs", [(1e-4, 1), (1e-5, 3), (1e-5, 17), (1e-6, 1), (1e-6, 5), (1e-8, 1), (1e-8, 4)])
 def test_beside_and_in_line(eps, nrhs):
     """Leaves on many levels, P2L on several (rows of their own per level) and M2P.  The forms differ in
     the order in which FP32 or FP64 terms are added: at most 1e-6 / 1e-13 of the result (about 500
