@@ -707,13 +707,20 @@ __device__ __forceinline__ float4 shifted(float4 v, float4 sh) {
 // One block per target leaf; each thread holds two targets (t and t + nth), so
 // a staged source is read from shared memory once per two interactions; the
 // threads form groups that split the staged sources.  NR right-hand sides per
-// pass.
+// pass.  A leaf of some 20 points meets 260 sources, 22 pairs of interactions per thread, so
+// staging and the groups' sums weigh as much as the interactions: the sums reuse the
+// densities' shared memory (7 blocks per SM instead of 6 at NR = 4: torus of 40 wavelengths, 3
+// right-hand sides, 0.154 -> 0.140 ms), and where there are several passes a thread stages a
+// density, not a source (8 NR bytes apart, NR lanes to a bank: ellipsoid of 32, 16 right-hand
+// sides, 0.306 -> 0.266 ms; one pass: 0.140 against 0.150, the list is read once more).  NR = 8, half
+// the passes: 0.278 ms, five blocks per SM.
 template <int NR>
 __global__ __launch_bounds__(PF_THREADS) void p2p_fast_kernel(P2PArgs a) {
   pdl_begin();
   __shared__ float4 sy[PF_CHUNK];
-  __shared__ float2 sf[PF_CHUNK][NR];
-  __shared__ float2 red[PF_THREADS][2][NR];
+  __shared__ __align__(16) float2 sf[PF_CHUNK][NR];
+  float2 (*red)[2][NR] = (float2 (*)[2][NR])sf;   // [PF_THREADS], once the pass has consumed sf
+  static_assert(2 * PF_THREADS <= PF_CHUNK, "the groups' sums take the place of the densities");
   __shared__ float4 stab[128];   // shift of each entry of the leaf's list
   const int2 lr = a.leaf_range[blockIdx.x];
   const int64_t u0 = a.u_off[blockIdx.x], u1 = a.u_off[blockIdx.x + 1];
@@ -721,6 +728,7 @@ __global__ __launch_bounds__(PF_THREADS) void p2p_fast_kernel(P2PArgs a) {
   const int4 e0 = a.u_src[u0], el = a.u_src[u1 - 1];
   const int total = el.z + el.y - e0.z;
   const int self_end = e0.w ? e0.y : 0;   // staged indices of the own leaf's points
+  const bool many = NR > 1 && a.nrhs > NR;   // several passes
   for (int t = threadIdx.x; t < (int)(u1 - u0); t += PF_THREADS) stab[t] = a.u_shift[u0 + t];
   for (int t0 = 0; t0 < lr.y; t0 += 2 * PF_THREADS) {
     const int nt = min(2 * PF_THREADS, lr.y - t0);
@@ -748,9 +756,17 @@ __global__ __launch_bounds__(PF_THREADS) void p2p_fast_kernel(P2PArgs a) {
           const uint32_t v = a.flat[e0.z + c0 + q];
           const int j = (int)(v & 0x1FFFFFFu);
           sy[q] = shifted(a.pts[j], stab[v >> 25]);
+          if (!many)
 #pragma unroll
-          for (int k = 0; k < NR; ++k)
+            for (int k = 0; k < NR; ++k) sf[q][k] = k < nr ? a.fs[(int64_t)j * a.nrhs + r0 + k] : make_float2(0.f, 0.f);
+        }
+        if (many) {
+#pragma unroll 4
+          for (int e = threadIdx.x; e < fill * NR; e += PF_THREADS) {
+            const int q = e / NR, k = e % NR;
+            const int j = (int)(a.flat[e0.z + c0 + q] & 0x1FFFFFFu);
             sf[q][k] = k < nr ? a.fs[(int64_t)j * a.nrhs + r0 + k] : make_float2(0.f, 0.f);
+          }
         }
         __syncthreads();
         if (active) {
@@ -784,6 +800,7 @@ __global__ __launch_bounds__(PF_THREADS) void p2p_fast_kernel(P2PArgs a) {
           for (; j < jhi; ++j) body(j, std::false_type());
         }
       }
+      __syncthreads();
 #pragma unroll
       for (int k = 0; k < NR; ++k) {
         red[threadIdx.x][0][k] = active ? acc0[k] : make_float2(0.f, 0.f);
