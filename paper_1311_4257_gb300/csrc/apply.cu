@@ -7,12 +7,12 @@
 //    source states (pairs x right-hand sides), and scatter-adds the result
 //    into the target states with vector atomics (targets of one operator are
 //    distinct, different operators meet in L2).  This is the plain CUDA-core
-//    form; the tensor-core forms are in m2l_cx.cu and m2l_tc.cu.
+//    form; the tensor-core forms are in m2l_cx.cu, m2l_sl.cu and m2l_tc.cu.
 //  * p2c_kernel: potentials at check points from points (P2L, X lists), with
 //    the phase 2 pi |x - y| reduced in a compensated form so that far check
 //    points keep full FP32 accuracy.
-//  * p2m_rows_kernel: P2M as a sum of FP64-formed per-point rows.
-//  * l2p_kernel: L2P through precomputed per-point rows (flat row stream).
+//  * p2m_row_kernel, p2m_rows_kernel: P2M as a sum of FP64-formed per-point rows.
+//  * l2p_kernel, l2p_leaf_kernel: L2P through precomputed per-point rows.
 //  * rows_kernel: M2P (W lists) through precomputed rows.
 //  * p2p_fast_kernel: the near field (U lists) on FP32 coordinates, with the
 //    exact plan-time corrections of the close pairs (p2p_close_kernel,
@@ -326,6 +326,14 @@ __device__ __forceinline__ void row_dot(float2& c, float4 x, float4 y) {
   c.y = fmaf(x.z, y.w, fmaf(x.w, y.z, c.y));
 }
 
+// c += v x, two complex entries
+__device__ __forceinline__ void row_axpy(float4& c, float4 v, float2 x) {
+  c.x = fmaf(v.x, x.x, fmaf(-v.y, x.y, c.x));
+  c.y = fmaf(v.x, x.y, fmaf(v.y, x.x, c.y));
+  c.z = fmaf(v.z, x.x, fmaf(-v.w, x.y, c.z));
+  c.w = fmaf(v.z, x.y, fmaf(v.w, x.x, c.w));
+}
+
 // L2P of one right-hand side as a flat stream of rows: warp w evaluates the point rows 2w and 2w+1
 // (1 KB each at rank 128, loaded together as float4 before any arithmetic);
 // the state rows they dot with are shared by the points of a leaf and mostly
@@ -333,10 +341,10 @@ __device__ __forceinline__ void row_dot(float2& c, float4 x, float4 y) {
 // 0.27 ms at K = 64 against 0.28 ms with four rows and 0.43 ms with eight.
 constexpr int L2P_ROWS = 2;
 
-template <int Q, bool MANY>
-__global__ __launch_bounds__(256) void l2p_kernel(const __grid_constant__ L2PArgs a) {
+template <int Q, class A>
+__global__ __launch_bounds__(256) void l2p_kernel(const __grid_constant__ A a) {
   pdl_begin();
-  const L2PArgs::Level& g = a.lv[level_of<MANY>(a, blockIdx.x)];
+  const L2PLevel& g = a.lv[level_of(a, blockIdx.x)];
   const int64_t r0 = (((int64_t)(blockIdx.x - g.block0) * blockDim.x + threadIdx.x) >> 5) * L2P_ROWS;
   const int lane = threadIdx.x & 31;
   const int64_t nrows = g.nrows;
@@ -384,11 +392,11 @@ __global__ __launch_bounds__(256) void l2p_kernel(const __grid_constant__ L2PArg
 // 0.072; sphere of 16 with 4 (apply): 943 -> 923 us.
 constexpr int L2P_KS = 16, L2P_KB = 4, L2P_LEAF_THREADS = 128;
 
-template <int Q, bool MANY>
-__global__ __launch_bounds__(L2P_LEAF_THREADS) void l2p_leaf_kernel(const __grid_constant__ L2PArgs a) {
+template <int Q, class A>
+__global__ __launch_bounds__(L2P_LEAF_THREADS) void l2p_leaf_kernel(const __grid_constant__ A a) {
   pdl_begin();
   extern __shared__ float4 sst[];   // [right-hand side][R / 2]
-  const L2PArgs::Level& g = a.lv[level_of<MANY>(a, blockIdx.x)];
+  const L2PLevel& g = a.lv[level_of(a, blockIdx.x)];
   const int4 job = g.jobs[blockIdx.x - g.block0];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int R2 = g.R / 2, nrhs = a.nrhs;
@@ -458,25 +466,88 @@ __global__ __launch_bounds__(L2P_LEAF_THREADS) void l2p_leaf_kernel(const __grid
 }
 
 // P2M through rows: lane l of a warp owns the state entries 2 (l + 32 t), 2 (l + 32 t) + 1
-// (float4 loads) of a leaf for KB right-hand sides; the leaf's point rows are read
-// 4 at a time (4 KB in flight per warp) together with the points' densities (a broadcast
-// load per point and right-hand side).  The warps of a leaf's further right-hand sides are
+// (float4 loads) of a leaf; the leaf's point rows are read 4 at a time (4 KB in flight per
+// warp).  One right-hand side: a warp per leaf, bound by HBM (sphere of 64: 0.240 ms, 5.9 TB/s);
+// launched with KB = 1, the loops over right-hand sides kept because the compiler schedules the
+// loads better with them (apply of sphere 2: 35 against 37 us without).
+template <int Q, int KB, class A>
+__global__ __launch_bounds__(256) void p2m_row_kernel(const __grid_constant__ A a) {
+  pdl_begin();
+  const P2MLevel& g = a.lv[level_of(a, blockIdx.x)];
+  const int64_t jw = ((int64_t)(blockIdx.x - g.block0) * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (jw >= g.njobs) return;
+  const int4 job = g.jobs[jw];
+  const int R2 = g.R / 2;
+  const float4* rows = (const float4*)g.rows;
+  float4* st = (float4*)g.state;
+  for (int k0 = 0; k0 < a.nrhs; k0 += KB) {
+    const int nk = min(KB, a.nrhs - k0);
+    float4 acc[KB][Q];
+#pragma unroll
+    for (int kk = 0; kk < KB; ++kk)
+#pragma unroll
+      for (int t = 0; t < Q; ++t) acc[kk][t] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < job.y; i += 4) {
+      float4 r[4][Q];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int t = 0; t < Q; ++t) {
+          const int q = lane + 32 * t;
+          r[j][t] = (i + j < job.y && q < R2) ? __ldcs(rows + (int64_t)(job.z + i + j) * R2 + q)
+                                              : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (i + j >= job.y) break;
+#pragma unroll
+        for (int kk = 0; kk < KB; ++kk) {
+          if (kk >= nk) break;
+          const float2 f = a.fs[(int64_t)(job.x + i + j) * a.nrhs + k0 + kk];
+#pragma unroll
+          for (int t = 0; t < Q; ++t) {
+            float4& c = acc[kk][t];
+            const float4 v = r[j][t];
+            c.x = fmaf(v.x, f.x, fmaf(-v.y, f.y, c.x));
+            c.y = fmaf(v.x, f.y, fmaf(v.y, f.x, c.y));
+            c.z = fmaf(v.z, f.x, fmaf(-v.w, f.y, c.z));
+            c.w = fmaf(v.z, f.y, fmaf(v.w, f.x, c.w));
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int kk = 0; kk < KB; ++kk) {
+      if (kk >= nk) break;
+#pragma unroll
+      for (int t = 0; t < Q; ++t) {
+        const int q = lane + 32 * t;
+        if (q < R2) st[((int64_t)job.w * a.nrhs + k0 + kk) * R2 + q] = acc[kk][t];
+      }
+    }
+  }
+}
+
+// Several right-hand sides, KB per warp, their densities loaded with the rows (a broadcast load per
+// point and right-hand side).  The warps of a leaf's further right-hand sides are
 // neighbours and find its rows in L1: passes over the rows from one warp, 4 right-hand sides each,
 // read them from memory again and waited for the densities (ellipsoid of 32 wavelengths, 16
-// right-hand sides: 0.207 -> 0.105 ms; two per warp instead of four: 0.155).  A single right-hand side
-// keeps the densities out of the row loads (0.240 against 0.266 ms, sphere of 64, 5.9 TB/s).
+// right-hand sides: 0.207 -> 0.105 ms; two per warp instead of four: 0.155).  For one right-hand side
+// this form is the slower one (0.266 ms, sphere of 64; the apply of sphere 2: 37 against 35 us).
 constexpr int P2M_KB = 4;
 
-template <int Q, int KB, bool MANY>
-__global__ __launch_bounds__(256) void p2m_rows_kernel(const __grid_constant__ P2MRowsArgs a) {
+template <int Q, class A>
+__global__ __launch_bounds__(256) void p2m_rows_kernel(const __grid_constant__ A a) {
   pdl_begin();
-  const P2MRowsArgs::Level& g = a.lv[level_of<MANY>(a, blockIdx.x)];
-  const int nrhs = a.nrhs, parts = KB == 1 ? 1 : (nrhs + KB - 1) / KB;   // KB = 1: one right-hand side
+  constexpr int KB = P2M_KB;
+  const P2MLevel& g = a.lv[level_of(a, blockIdx.x)];
+  const int nrhs = a.nrhs, parts = (nrhs + KB - 1) / KB;
   const int64_t w = ((int64_t)(blockIdx.x - g.block0) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  const int64_t jw = KB == 1 ? w : (uint32_t)w / (uint32_t)parts;
+  const int64_t jw = (uint32_t)w / (uint32_t)parts;
   if (jw >= g.njobs) return;
-  const int k0 = KB == 1 ? 0 : (int)(w - jw * parts) * KB;
+  const int k0 = (int)(w - jw * parts) * KB;
   const int4 job = g.jobs[jw];
   const int R2 = g.R / 2;
   const float4* rows = (const float4*)g.rows + (int64_t)job.z * R2;
@@ -495,32 +566,18 @@ __global__ __launch_bounds__(256) void p2m_rows_kernel(const __grid_constant__ P
 #pragma unroll
       for (int t = 0; t < Q; ++t) {
         const int q = lane + 32 * t;
-        const float4* p = rows + (int64_t)(i + j) * R2 + q;
-        r[j][t] = in && q < R2 ? (KB == 1 ? __ldcs(p) : *p) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int kk = 0; kk < KB && KB > 1; ++kk)
-        f[j][kk] = in ? fs[(int64_t)(i + j) * nrhs + min(k0 + kk, nrhs - 1)] : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (KB == 1) {
-        if (i + j >= job.y) break;
-        f[j][0] = fs[i + j];
+        r[j][t] = in && q < R2 ? rows[(int64_t)(i + j) * R2 + q] : make_float4(0.f, 0.f, 0.f, 0.f);
       }
 #pragma unroll
       for (int kk = 0; kk < KB; ++kk)
-#pragma unroll
-        for (int t = 0; t < Q; ++t) {
-          float4& c = acc[kk][t];
-          const float4 v = r[j][t];
-          const float2 x = f[j][kk];
-          c.x = fmaf(v.x, x.x, fmaf(-v.y, x.y, c.x));
-          c.y = fmaf(v.x, x.y, fmaf(v.y, x.x, c.y));
-          c.z = fmaf(v.z, x.x, fmaf(-v.w, x.y, c.z));
-          c.w = fmaf(v.z, x.y, fmaf(v.w, x.x, c.w));
-        }
+        f[j][kk] = in ? fs[(int64_t)(i + j) * nrhs + min(k0 + kk, nrhs - 1)] : make_float2(0.f, 0.f);
     }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int kk = 0; kk < KB; ++kk)
+#pragma unroll
+        for (int t = 0; t < Q; ++t) row_axpy(acc[kk][t], r[j][t], f[j][kk]);
   }
   float4* st = (float4*)g.state + ((int64_t)job.w * nrhs + k0) * R2;
 #pragma unroll
@@ -935,12 +992,21 @@ void launch_rows(const RowsArgs& a, LaunchStream s) {
 }
 
 // levels of rank up to 128 and beyond: a lane holds 4 or 8 state entries
-template <class A> bool narrow(const typename A::Level& g) { return g.R <= 128; }
-template <class A, class F>
-void by_levels(const A& a, bool narrow, F&& f) {
+void copy_common(L2PCommon& to, const L2PCommon& from) { to = from; }
+void copy_common(P2MCommon& to, const P2MCommon& from) { to = from; }
+template <class L> bool narrow(const L& g) { return g.R <= 128; }
+// f(entries per lane / 2, arguments), with the arguments of one level where there is one
+template <template <int> class Of, class F>
+void by_levels(const Of<kLFLevels>& a, bool narrow, F&& f) {
   const auto at = [&](auto q) {
-    if (a.nlv == 1) f(q, std::false_type());
-    else f(q, std::true_type());
+    if (a.nlv == 1) {
+      Of<1> one;
+      copy_common(one, a);
+      one.lv[0] = a.lv[0];
+      f(q, one);
+    } else {
+      f(q, a);
+    }
   };
   if (narrow) at(std::integral_constant<int, 2>());
   else at(std::integral_constant<int, 4>());
@@ -955,15 +1021,16 @@ void launch_l2p(const L2PArgs& a, LaunchStream s) {
   for (const bool nar : {true, false}) {
     L2PArgs p;
     int R = 0;
-    const unsigned grid = place_levels(a, p, [&](const L2PArgs::Level& g) { return narrow<L2PArgs>(g) == nar; },
-                                       [&](const L2PArgs::Level& g) {
+    const unsigned grid = place_levels(a, p, [&](const L2PLevel& g) { return narrow(g) == nar; },
+                                       [&](const L2PLevel& g) {
                                          R = std::max(R, g.R);
                                          return a.nrhs > 1 ? g.njobs : (g.nrows + 8 * L2P_ROWS - 1) / (8 * L2P_ROWS);
                                        });
     if (grid == 0) continue;
-    by_levels(p, nar, [&](auto q, auto many) {
-      if (a.nrhs == 1) launch_pdl(l2p_kernel<q(), many()>, grid, 256, 0, s, p);
-      else launch_pdl(l2p_leaf_kernel<q(), many()>, grid, L2P_LEAF_THREADS, (size_t)std::min(a.nrhs, L2P_KS) * R * 8, s, p);
+    by_levels(p, nar, [&](auto q, const auto& v) {
+      using V = std::decay_t<decltype(v)>;
+      if (a.nrhs == 1) launch_pdl(l2p_kernel<q(), V>, grid, 256, 0, s, v);
+      else launch_pdl(l2p_leaf_kernel<q(), V>, grid, L2P_LEAF_THREADS, (size_t)std::min(a.nrhs, L2P_KS) * R * 8, s, v);
     });
   }
   DFMM_CUDA(cudaGetLastError());
@@ -974,12 +1041,13 @@ void launch_p2m_rows(const P2MRowsArgs& a, LaunchStream s) {
   const int kb = a.nrhs == 1 ? 1 : P2M_KB, parts = (a.nrhs + kb - 1) / kb;
   for (const bool nar : {true, false}) {
     P2MRowsArgs p;
-    const unsigned grid = place_levels(a, p, [&](const P2MRowsArgs::Level& g) { return narrow<P2MRowsArgs>(g) == nar; },
-                                       [&](const P2MRowsArgs::Level& g) { return (g.njobs * parts + 7) / 8; });
+    const unsigned grid = place_levels(a, p, [&](const P2MLevel& g) { return narrow(g) == nar; },
+                                       [&](const P2MLevel& g) { return (g.njobs * parts + 7) / 8; });
     if (grid == 0) continue;
-    by_levels(p, nar, [&](auto q, auto many) {
-      if (a.nrhs == 1) launch_pdl(p2m_rows_kernel<q(), 1, many()>, grid, 256, 0, s, p);
-      else launch_pdl(p2m_rows_kernel<q(), P2M_KB, many()>, grid, 256, 0, s, p);
+    by_levels(p, nar, [&](auto q, const auto& v) {
+      using V = std::decay_t<decltype(v)>;
+      if (a.nrhs == 1) launch_pdl(p2m_row_kernel<q(), 1, V>, grid, 256, 0, s, v);
+      else launch_pdl(p2m_rows_kernel<q(), V>, grid, 256, 0, s, v);
     });
   }
   DFMM_CUDA(cudaGetLastError());

@@ -161,6 +161,8 @@ struct RowsArgs {
 };
 void launch_rows(const RowsArgs& a, LaunchStream s);
 
+constexpr int kLFLevels = 24;   // levels of the octree at most
+
 // The levels of A (L2PArgs, P2MRowsArgs) that `take` accepts, blocks(level) blocks each: their count.
 template <class A, class Take, class Blocks>
 unsigned place_levels(const A& a, A& out, Take&& take, Blocks&& blocks) {
@@ -177,12 +179,12 @@ unsigned place_levels(const A& a, A& out, Take&& take, Blocks&& blocks) {
   return (unsigned)at;
 }
 #ifdef __CUDACC__
-// the level that block b works on (MANY: there may be several; the lookup costs a short block
-// some 5%, sphere of 64 wavelengths 4.22 -> 4.25 ms, so one level does without)
-template <bool MANY, class A>
+// The level that block b works on.  A launch of one level takes arguments of one, since the lookup costs
+// a short block some 5% (sphere of 64 wavelengths 4.22 -> 4.25 ms).
+template <class A>
 __device__ __forceinline__ int level_of(const A& a, unsigned b) {
   int l = 0;
-  if (!MANY) return l;
+  if (A::kMax == 1) return l;
   while (l + 1 < a.nlv && b >= a.lv[l + 1].block0) ++l;
   return l;
 }
@@ -191,39 +193,49 @@ __device__ __forceinline__ int level_of(const A& a, unsigned b) {
 // L2P, one warp per point: us[p_r][rhs] += sum_q rows[r][q] state[s_r][rhs][q]
 // for every row r, with (p_r, s_r) = map[r] (each point has one row).  All levels in one
 // launch: those of an adaptive tree hold a few blocks each.
-struct L2PArgs {
-  static constexpr int kMax = 24;   // LF levels
-  struct Level {
-    const int4* jobs;          // leaves: (first point, count, first row, state row)
-    int64_t njobs;
-    const int2* map;           // (point, state row) per row
-    int64_t nrows;
-    const float2* rows;        // [nrows][R]
-    const float2* state;       // [..][nrhs][R]
-    int R;                     // even, <= 256
-    unsigned block0;           // first block of the level (set by the launch)
-  } lv[kMax];
-  int nlv, nrhs;
-  float2* us;                  // [N][nrhs]
+struct L2PLevel {
+  const int4* jobs;          // leaves: (first point, count, first row, state row)
+  int64_t njobs;
+  const int2* map;           // (point, state row) per row
+  int64_t nrows;
+  const float2* rows;        // [nrows][R]
+  const float2* state;       // [..][nrhs][R]
+  int R;                     // even, <= 256
+  unsigned block0;           // first block of the level (set by the launch)
 };
+struct L2PCommon {
+  int nlv, nrhs;
+  float2* us;                // [N][nrhs]
+};
+template <int LEVELS>
+struct L2PArgsOf : L2PCommon {
+  static constexpr int kMax = LEVELS;
+  L2PLevel lv[LEVELS];
+};
+using L2PArgs = L2PArgsOf<kLFLevels>;
 void launch_l2p(const L2PArgs& a, LaunchStream s);
 
 // P2M through per-point rows: for every leaf job (first point, count, first
 // row, box) and right-hand side k, state[box][k][q] = sum_i rows[row + i][q]
 // fs[first + i][k].  All levels in one launch, as L2P.
-struct P2MRowsArgs {
-  static constexpr int kMax = 24;
-  struct Level {
-    const int4* jobs;
-    int64_t njobs;
-    const float2* rows;        // [..][R]
-    float2* state;             // [boxes][nrhs][R]
-    int R;                     // <= 256
-    unsigned block0;
-  } lv[kMax];
-  int nlv, nrhs;
-  const float2* fs;            // [N][nrhs]
+struct P2MLevel {
+  const int4* jobs;
+  int64_t njobs;
+  const float2* rows;        // [..][R]
+  float2* state;             // [boxes][nrhs][R]
+  int R;                     // <= 256
+  unsigned block0;
 };
+struct P2MCommon {
+  int nlv, nrhs;
+  const float2* fs;          // [N][nrhs]
+};
+template <int LEVELS>
+struct P2MRowsArgsOf : P2MCommon {
+  static constexpr int kMax = LEVELS;
+  P2MLevel lv[LEVELS];
+};
+using P2MRowsArgs = P2MRowsArgsOf<kLFLevels>;
 void launch_p2m_rows(const P2MRowsArgs& a, LaunchStream s);
 
 // Near field: us[i] += sum over U-list source leaves of G(p_i, p_j) f_j,

@@ -294,7 +294,7 @@ __global__ __launch_bounds__(256) void rows64_kernel(RowsArgs a) {
 template <int NR>
 __global__ __launch_bounds__(256) void l2p64_kernel(const __grid_constant__ L2PArgs a) {
   pdl_begin();
-  const L2PArgs::Level& g = a.lv[level_of<true>(a, blockIdx.x)];
+  const L2PLevel& g = a.lv[level_of(a, blockIdx.x)];
   const int64_t r = ((int64_t)(blockIdx.x - g.block0) * blockDim.x + threadIdx.x) >> 5;
   if (r >= g.nrows) return;
   const int2 m = g.map[r];
@@ -310,7 +310,7 @@ __global__ __launch_bounds__(256) void l2p64_kernel(const __grid_constant__ L2PA
 template <int NR>
 __global__ __launch_bounds__(C64_T) void p2m64_kernel(const __grid_constant__ P2MRowsArgs a) {
   pdl_begin();
-  const P2MRowsArgs::Level& g = a.lv[level_of<true>(a, blockIdx.x)];
+  const P2MLevel& g = a.lv[level_of(a, blockIdx.x)];
   const int R = g.R, q = blockIdx.y * C64_T + threadIdx.x;
   if (q >= R) return;
   const int4 job = g.jobs[blockIdx.x - g.block0];
@@ -462,8 +462,8 @@ void launch_rows64(const RowsArgs& a, LaunchStream s) {
 void launch_l2p64(const L2PArgs& a, LaunchStream s) {
   for (int l = 0; l < a.nlv; ++l) check_rank(a.lv[l].R);
   L2PArgs p;
-  const unsigned grid = place_levels(a, p, [](const L2PArgs::Level&) { return true; },
-                                     [](const L2PArgs::Level& g) { return (g.nrows + 7) / 8; });
+  const unsigned grid = place_levels(a, p, [](const L2PLevel&) { return true; },
+                                     [](const L2PLevel& g) { return (g.nrows + 7) / 8; });
   if (grid == 0) return;
   by_rhs(a.nrhs, [&](auto nr) { launch_pdl(l2p64_kernel<nr()>, grid, 256, 0, s, p); });
   DFMM_CUDA(cudaGetLastError());
@@ -476,8 +476,8 @@ void launch_p2m_rows64(const P2MRowsArgs& a, LaunchStream s) {
     R = std::max(R, a.lv[l].R);
   }
   P2MRowsArgs p;
-  const unsigned n = place_levels(a, p, [](const P2MRowsArgs::Level&) { return true; },
-                                  [](const P2MRowsArgs::Level& g) { return g.njobs; });
+  const unsigned n = place_levels(a, p, [](const P2MLevel&) { return true; },
+                                  [](const P2MLevel& g) { return g.njobs; });
   if (n == 0) return;
   const dim3 grid(n, (unsigned)((R + C64_T - 1) / C64_T));
   by_rhs(a.nrhs, [&](auto nr) { launch_pdl(p2m64_kernel<nr()>, grid, C64_T, 0, s, p); });

@@ -150,6 +150,7 @@ struct M2PGroup {
 struct Workspace {
   int nrhs = 0;
   bool external = false;   // buffers carved from caller-provided memory
+  bool full = true;        // not the least layout: with work tiles for the few-column form
   DevArena ar;
   float2 *fs = nullptr, *us = nullptr;
   std::vector<float2*> p2l;                             // per level: potentials at the P2L check points
@@ -1311,14 +1312,6 @@ Workspace* get_workspace(dfmm_plan_s* P, cudaStream_t s, int nrhs) {
   return W;
 }
 
-// Work tiles of a stage: runs of up to cols / nrhs pairs of one operator.
-// Pairs of an operator are sorted by target, so an operator's tiles sweep the
-// whole target array.  When the stage's operators are small enough to stay in
-// L2 (<= 64 MB), tiles are ordered by block of target rows first and operator
-// second, so that the tiles in flight together touch one block of targets
-// (and the sources near them) and keep those rows in L2; blocks hold about
-// 8 MB of target rows.  Otherwise tiles stay in operator order, so that an
-// operator is read from DRAM once for all its tiles.
 // whether a translation stage runs on the tensor cores (m2l_mode 2, ranks padded
 // for the MMA, its family selected by options.tc_stages)
 bool on_tensor_cores(const dfmm_plan_s* P, const GemmPlan& g) {
@@ -1327,8 +1320,8 @@ bool on_tensor_cores(const dfmm_plan_s* P, const GemmPlan& g) {
          (P->opt.tc_precision == 0 || gemm_cx_supported(g.M, g.Kd, P->opt.tc_precision));
 }
 
-// whether a tensor-core stage takes the split-complex form (m2l_cx.cu): target
-// rank at most 128 and ranks that are multiples of 16; else the real-block form
+// whether a tensor-core stage takes the split-complex form (m2l_cx.cu): ranks that are multiples
+// of 16, the target's at most 256 (128 for the BF16 and TF32 splits); else the real-block form
 bool split_complex(const dfmm_plan_s* P, const GemmPlan& g) {
   return on_tensor_cores(P, g) && P->opt.tc_layout != 1 && gemm_cx_supported(g.M, g.Kd, P->opt.tc_precision);
 }
@@ -1345,12 +1338,20 @@ bool few_columns(const dfmm_plan_s* P, const GemmPlan& g, int nrhs) {
   return P->few && g.npairs * nrhs <= cols * ops;
 }
 
-// columns of a stage's work tiles (slices: whether the workspace holds the slices of its source)
-int tile_columns(const dfmm_plan_s* P, const GemmPlan& g, int nrhs, bool slices) {
-  if (few_columns(P, g, nrhs)) return gemm_few_columns();
+// columns of a stage's work tiles (full: in a full layout; slices: the workspace holds its source's slices)
+int tile_columns(const dfmm_plan_s* P, const GemmPlan& g, int nrhs, bool full, bool slices) {
+  if (full && few_columns(P, g, nrhs)) return gemm_few_columns();
   return on_tensor_cores(P, g) || (slices && sliced_stage(g)) ? gemm_tc_columns() : 64;
 }
 
+// Work tiles of a stage: runs of up to cols / nrhs pairs of one operator.
+// Pairs of an operator are sorted by target, so an operator's tiles sweep the
+// whole target array.  When the stage's operators are small enough to stay in
+// L2 (<= 64 MB), tiles are ordered by block of target rows first and operator
+// second, so that the tiles in flight together touch one block of targets
+// (and the sources near them) and keep those rows in L2; blocks hold about
+// 8 MB of target rows.  Otherwise tiles stay in operator order, so that an
+// operator is read from DRAM once for all its tiles.
 // tile_order: 0 = by the 64 MB rule above, 1 = always by target block, 2 = always by operator.
 // block_bytes: target rows per block in the blocked order (8 MB unless the
 // batched form's autotuner tries another size).
@@ -1450,7 +1451,7 @@ struct Runner {
   void gemm(const GemmPlan& g, const float2* src, int src_ld, int64_t src_rows, float2* dst, int dst_ld,
             int src_key) {
     if (g.npairs == 0) return;
-    const bool few = few_columns(P, g, nrhs);
+    const bool few = (count || W->full) && few_columns(P, g, nrhs);
     const bool tc = !few && on_tensor_cores(P, g);
     const bool cx = tc && split_complex(P, g);
     const bool sl = !few && sliced_stage(g) && (count || W->sl);
@@ -1464,7 +1465,7 @@ struct Runner {
       ctl->collect->push_back(WaveGemm{P, W, &g, src, src_ld, src_rows, dst, dst_ld, nrhs, split});
       return;
     }
-    auto t = tiles_for(P, W, g, nrhs, tile_columns(P, g, nrhs, W->sl != nullptr), s);
+    auto t = tiles_for(P, W, g, nrhs, tile_columns(P, g, nrhs, W->full, W->sl != nullptr), s);
     GemmArgs a;
     a.ops = g.ops;
     a.M = g.M;
@@ -1662,7 +1663,7 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
     for (int l = P->l_lf0; l < nl; ++l) {
       LFLevel& F = P->lf[l];
       if (!F.n_l2p) continue;
-      if (a.nlv == P2MRowsArgs::kMax) throw Error(DFMM_ERR_UNSUPPORTED, "too many levels");
+      if (a.nlv == kLFLevels) throw Error(DFMM_ERR_UNSUPPORTED, "too many levels");
       if (!count) a.lv[a.nlv] = {F.l2p_jobs, F.n_l2p, F.p2m_rows, W->S[l], F.R, 0};
       ++a.nlv;
       fl += 8.0 * F.r * F.npts * nrhs;
@@ -1780,7 +1781,8 @@ std::vector<const GemmPlan*> all_gemms(dfmm_plan_s* P) {
 // staging buffers and the work tiles of every stage (copied in on `s`).  No device memory is allocated.  With
 // base == nullptr nothing is laid out or copied: the return value is the
 // number of bytes the layout needs.  full: with the sliced form's source buffer,
-// without which the plan's sliced stages run on the CUDA cores, and P2L rows for every level.
+// without which the plan's sliced stages run on the CUDA cores, P2L rows for every
+// level and the few-column form's work tiles; without them an apply runs in no more than it always did.
 size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaStream_t s, Workspace& W, bool full) {
   size_t off = 0;
   auto take = [&](size_t n) -> char* {
@@ -1792,6 +1794,7 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
   const int64_t N = P->N;
   const size_t cb = 8 * (size_t)P->cw;   // bytes per complex element
   W.external = true;
+  W.full = full;
   W.nrhs = nrhs;
   // the device status word first, at offset 0 of the region (reset by every apply)
   W.status = (unsigned*)take(4);
@@ -1831,7 +1834,7 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
   std::vector<int> tl_cols;
   for (const GemmPlan* g : all_gemms(P)) {
     if (g->npairs == 0) continue;
-    const int cols = tile_columns(P, *g, nrhs, slices);
+    const int cols = tile_columns(P, *g, nrhs, full, slices);
     tl_cols.push_back(cols);
     tl.push_back({g, make_tiles(*g, nrhs, cols, P->opt.tile_order)});
   }

@@ -253,7 +253,7 @@ __device__ __forceinline__ CxStage stage_of(const GemmArgs& a, const TcArgs& t, 
 //              xr lo, xi lo, xr hi or xi hi) with 16-byte cp.async, counted on the
 //              slot's full barrier, up to CX_NA tiles ahead; thread 0 also
 //              bulk-copies the operator chunk, up to CX_NB chunks ahead.
-//   last warp  one thread issues the MMAs, commits each tile and each operator
+//   last warp  an elected lane issues the MMAs, commits each tile and each operator
 //              chunk to their slots' empty barriers and each item to acc_full; it
 //              waits for acc_empty before it overwrites the accumulators.
 //   warps 4 .. epilogue: warp 4 + q reads tensor-memory lanes 32 (q % 4) ..

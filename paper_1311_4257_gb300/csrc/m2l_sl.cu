@@ -290,7 +290,7 @@ __device__ __forceinline__ double join8(const uint32_t* r) {
 //   warps 0-3  producers: 8 lanes copy one row of a tile (a slice of the real or
 //              imaginary parts, one 128-byte line) with 16-byte cp.async into the
 //              swizzled tile; thread 0 also bulk-copies the operator chunk.
-//   warp 12    one thread issues the two stacked MMAs of every K step of a tile.
+//   warp 12    an elected lane issues the two stacked MMAs of every K step of a tile.
 //   warps 4-11 epilogue: join the groups of an output into registers, hand the
 //              accumulators back, scale, add to the target row.
 // Every wait is time-limited; on a timeout the CTA reports it, stops issuing,
