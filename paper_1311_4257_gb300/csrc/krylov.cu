@@ -156,6 +156,13 @@ __global__ __launch_bounds__(KV_T) void update_kernel(const float2* V, int ncols
     n2 = fmaf(wv[r].x, wv[r].x, fmaf(wv[r].y, wv[r].y, n2));
   }
   double t = n2;
+  // Where the entries are far from one (about 1e-15, 1e18) their squares leave FP32's range or its full
+  // precision; FP64 holds the square of any FP32 number.  Zeros, infinities and NaN come out as themselves.
+  if (!(n2 > 1e-30f && n2 < 1e37f)) {
+    t = 0.0;
+#pragma unroll
+    for (int r = 0; r < KV_ROWS; ++r) t += (double)wv[r].x * wv[r].x + (double)wv[r].y * wv[r].y;
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   if (lane == 0) sums[warp] = t;
@@ -180,8 +187,14 @@ __global__ __launch_bounds__(KV_T) void scale_kernel(float2* w, const double* no
   const int64_t i = (int64_t)blockIdx.x * KV_T + threadIdx.x;
   const double n = *norm;
   if (i >= N || !(n > 0.0)) return;
-  const float f = (float)(1.0 / n);
-  w[i] = make_float2(w[i].x * f, w[i].y * f);
+  const float2 x = w[i];
+  if (n > 1e-37 && n < 1e37) {
+    const float f = (float)(1.0 / n);
+    w[i] = make_float2(x.x * f, x.y * f);
+  } else {   // 1 / n is no normal FP32 number
+    const double f = 1.0 / n;
+    w[i] = make_float2((float)(x.x * f), (float)(x.y * f));
+  }
 }
 
 int64_t blocks_of(int64_t N) { return (N + KV_BLOCK - 1) / KV_BLOCK; }
