@@ -359,7 +359,8 @@ int dfmm_graph_destroy(dfmm_graph_t graph);
  * 32; else DFMM_ERR_UNSUPPORTED).  Allocates (restart + 2) N complex64 of
  * device workspace per call; synchronises `stream` at every iteration (the
  * small least-squares problem is solved on the host).  Returns DFMM_OK
- * whether or not tol was reached (compare *relres), or an error status. */
+ * whether or not tol was reached (compare *relres), or an error status:
+ * DFMM_ERR_TIMEOUT as soon as a device wait of one of its matvecs gave up. */
 int dfmm_solve(dfmm_plan_t plan, double alpha_re, double alpha_im, double beta_re, double beta_im, const void* b,
                void* x, int restart, int maxit, double tol, cudaStream_t stream, int* iters, double* relres);
 

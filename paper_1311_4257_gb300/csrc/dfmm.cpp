@@ -2042,6 +2042,18 @@ void plan_release(const dfmm_plan_s* plan) {
   if (it != g_plans.end() && it->second > 0) --it->second;
 }
 
+const unsigned* apply_status_word(dfmm_plan_s* P, cudaStream_t stream) {
+  std::lock_guard<std::mutex> g(P->ws_mu);
+  auto it = P->ws.find(stream);
+  return it == P->ws.end() ? nullptr : it->second->status;
+}
+
+int status_error(unsigned st) {
+  if (st & kStatusTimeout) return fail(DFMM_ERR_TIMEOUT, "a device wait gave up");
+  if (st) return fail(DFMM_ERR_DEVICE, "a device-side check failed");
+  return DFMM_OK;
+}
+
 int apply_with_scratch(dfmm_plan_s* P, const void* f, void* u, int nrhs, cudaStream_t stream, void* scratch,
                        size_t bytes) {
   return guarded([&]() -> int {
@@ -2423,9 +2435,7 @@ int dfmm_sync_status(dfmm_plan_t plan, cudaStream_t stream) {
       DFMM_CUDA(cudaMemcpy(&sn, na, 4, cudaMemcpyDeviceToHost));
       st |= sn;
     }
-    if (st & kStatusTimeout) return fail(DFMM_ERR_TIMEOUT, "a device wait gave up");
-    if (st) return fail(DFMM_ERR_DEVICE, "a device-side check failed");
-    return DFMM_OK;
+    return status_error(st);
   });
 }
 

@@ -27,4 +27,11 @@ int apply_with_scratch(dfmm_plan_s* plan, const void* f, void* u, int nrhs, cuda
 // `stream`, else nullptr.
 const unsigned* noalloc_status_word(cudaStream_t stream);
 
+// Device address of the status word of the plan's applies on `stream` (set by the last
+// dfmm_apply there, cleared by the next), nullptr before the first.
+const unsigned* apply_status_word(dfmm_plan_s* plan, cudaStream_t stream);
+
+// The code (and message) of a status word that a host has read: DFMM_OK if it is 0.
+int status_error(unsigned status);
+
 }  // namespace dfmm

@@ -41,9 +41,14 @@ __device__ __forceinline__ bool last_block(unsigned* counter) {
   return last;
 }
 
+__device__ __forceinline__ void gather(StatusGather st) {
+  if (blockIdx.x == 0 && threadIdx.x == 0 && st.word) *st.sum |= *st.word;
+}
+
 __global__ __launch_bounds__(KV_T) void combine_kernel(float2 a, const float2* x, float2 b, const float2* y, float2 c,
-                                                       const float2* z, float2* out, int64_t N) {
+                                                       const float2* z, float2* out, StatusGather st, int64_t N) {
   pdl_begin();
+  gather(st);
   const int64_t i = (int64_t)blockIdx.x * KV_T + threadIdx.x;
   if (i >= N) return;
   float2 r = cmul(a, x[i]);
@@ -54,9 +59,10 @@ __global__ __launch_bounds__(KV_T) void combine_kernel(float2 a, const float2* x
 
 __global__ __launch_bounds__(KV_T) void dots_kernel(const float2* V, int ncols, float2* w, const float2* u, float2 b,
                                                     const float2* v, float2 a, float2* h, double2* part,
-                                                    unsigned* counter, int64_t N) {
+                                                    unsigned* counter, StatusGather st, int64_t N) {
   __shared__ float2 sums[KV_GROUP][KV_T / 32];
   pdl_begin();
+  gather(st);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t i0 = (int64_t)blockIdx.x * KV_BLOCK + threadIdx.x;
   float2 wv[KV_ROWS];
@@ -207,14 +213,15 @@ double2* partials(void* scratch) { return (double2*)((char*)scratch + 256); }
 int64_t krylov_scratch_bytes(int64_t N, int ncols) { return 256 + blocks_of(N) * (ncols > 0 ? ncols : 1) * (int64_t)sizeof(double2); }
 
 void krylov_combine(float2 a, const float2* x, float2 b, const float2* y, float2 c, const float2* z, float2* out,
-                    int64_t N, cudaStream_t s) {
-  launch_pdl(combine_kernel, (unsigned)((N + KV_T - 1) / KV_T), KV_T, 0, LaunchStream(s, true), a, x, b, y, c, z, out, N);
+                    StatusGather st, int64_t N, cudaStream_t s) {
+  launch_pdl(combine_kernel, (unsigned)((N + KV_T - 1) / KV_T), KV_T, 0, LaunchStream(s, true), a, x, b, y, c, z, out,
+             st, N);
 }
 
 void krylov_dots(const float2* V, int ncols, float2* w, const float2* u, float2 b, const float2* v, float2 a,
-                 float2* h, void* scratch, int64_t N, cudaStream_t s) {
+                 float2* h, void* scratch, StatusGather st, int64_t N, cudaStream_t s) {
   launch_pdl(dots_kernel, (unsigned)blocks_of(N), KV_T, 0, LaunchStream(s, true), V, ncols, w, u, b, v, a, h,
-             partials(scratch), (unsigned*)scratch, N);
+             partials(scratch), (unsigned*)scratch, st, N);
 }
 
 void krylov_update(const float2* V, int ncols, const float2* h, float2* w, double* norm, void* scratch, int64_t N,

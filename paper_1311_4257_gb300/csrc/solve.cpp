@@ -9,7 +9,8 @@
 // device (complex64); each new vector is orthogonalised by classical
 // Gram-Schmidt done twice (two kernels per pass, krylov.cu), the small
 // Hessenberg least-squares problem is solved on the host in double precision
-// with Givens rotations; the host waits once per iteration.
+// with Givens rotations; the host waits once per iteration, and then also sees
+// whether a device wait of an apply gave up.
 #include <cmath>
 #include <complex>
 #include <cstring>
@@ -52,10 +53,12 @@ extern "C" int dfmm_solve(dfmm_plan_t plan, double alpha_re, double alpha_im, do
     const int m = restart;
     const cd alpha(alpha_re, alpha_im), beta(beta_re, beta_im);
     // basis, one vector, and beside the kernels' scratch what the host reads back in one copy: the
-    // norm of the new vector and its products with the basis in the two passes
+    // norm of the new vector, the applies' status words so far and the vector's products with the basis
+    // in the two passes
     DevBuf Vb, wb, hb;
     const int64_t scratch = (dfmm::krylov_scratch_bytes(N, m + 1) + 255) & ~(int64_t)255;
-    const size_t back = sizeof(double) + 2 * (size_t)(m + 1) * sizeof(float2);
+    constexpr size_t head = 2 * sizeof(double);   // the norm and the status
+    const size_t back = head + 2 * (size_t)(m + 1) * sizeof(float2);
     if (cudaMalloc(&Vb.p, (size_t)(m + 1) * N * sizeof(float2)) != cudaSuccess ||
         cudaMalloc(&wb.p, (size_t)N * sizeof(float2)) != cudaSuccess ||
         cudaMalloc(&hb.p, scratch + back) != cudaSuccess) {
@@ -63,10 +66,12 @@ extern "C" int dfmm_solve(dfmm_plan_t plan, double alpha_re, double alpha_im, do
       return dfmm::set_error(DFMM_ERR_OOM, "GMRES workspace allocation failed");
     }
     DFMM_CUDA(cudaMemsetAsync(hb.p, 0, 256, stream));
+    DFMM_CUDA(cudaMemsetAsync((char*)hb.p + scratch, 0, head, stream));
     float2* V = (float2*)Vb.p;
     float2* w = (float2*)wb.p;
     double* nd = (double*)((char*)hb.p + scratch);
-    float2* hd = (float2*)(nd + 1);
+    float2* hd = (float2*)((char*)nd + head);
+    dfmm::StatusGather gather{nullptr, (unsigned*)(nd + 1)};
     float2* xv = (float2*)x;
     const float2* bv = (const float2*)b;
     const float2 ca = c32(alpha), cb = c32(beta);
@@ -74,6 +79,9 @@ extern "C" int dfmm_solve(dfmm_plan_t plan, double alpha_re, double alpha_im, do
     auto read_back = [&](size_t bytes) {
       DFMM_CUDA(cudaMemcpyAsync(hback.data(), nd, bytes, cudaMemcpyDeviceToHost, stream));
       DFMM_CUDA(cudaStreamSynchronize(stream));
+      unsigned st;
+      std::memcpy(&st, hback.data() + sizeof(double), sizeof st);
+      if (const int rc = dfmm::status_error(st)) throw dfmm::Error(rc, dfmm_last_error());
       double r;
       std::memcpy(&r, hback.data(), sizeof r);
       return r;
@@ -82,15 +90,17 @@ extern "C" int dfmm_solve(dfmm_plan_t plan, double alpha_re, double alpha_im, do
     auto apply = [&](const float2* v, float2* out) {
       const int rc = dfmm_apply(plan, v, out, 1, stream);
       if (rc != DFMM_OK) throw dfmm::Error(rc, dfmm_last_error());
+      gather.word = dfmm::apply_status_word(plan, stream);
     };
     auto nrm = [&](float2* v) {
       dfmm::krylov_update(V, 0, nullptr, v, nd, hb.p, N, stream);
-      return read_back(sizeof(double));
+      return read_back(head);
     };
     // r = b - A x into dst
     auto residual = [&](float2* dst) {
       apply(xv, w);
-      dfmm::krylov_combine(c32(-alpha), xv, c32(-beta), w, make_float2(1.f, 0.f), bv, dst, N, stream);
+      dfmm::krylov_combine(c32(-alpha), xv, c32(-beta), w, make_float2(1.f, 0.f), bv, dst, gather, N,
+                           stream);
     };
 
     const double bnorm = nrm((float2*)bv);   // no columns: only read
@@ -116,13 +126,13 @@ extern "C" int dfmm_solve(dfmm_plan_t plan, double alpha_re, double alpha_im, do
           float2* vj = V + (size_t)(j + 1) * N;
           // vj = (alpha I + beta G) v, orthogonalised by classical Gram-Schmidt, twice
           apply(v, w);
-          dfmm::krylov_dots(V, j + 1, vj, w, cb, v, ca, hd, hb.p, N, stream);
+          dfmm::krylov_dots(V, j + 1, vj, w, cb, v, ca, hd, hb.p, gather, N, stream);
           dfmm::krylov_update(V, j + 1, hd, vj, nd, hb.p, N, stream);
-          dfmm::krylov_dots(V, j + 1, vj, nullptr, cb, nullptr, ca, hd + m + 1, hb.p, N, stream);
+          dfmm::krylov_dots(V, j + 1, vj, nullptr, cb, nullptr, ca, hd + m + 1, hb.p, dfmm::StatusGather{}, N, stream);
           dfmm::krylov_update(V, j + 1, hd + m + 1, vj, nd, hb.p, N, stream);
           dfmm::krylov_scale(vj, nd, N, stream);
           const double hn = read_back(back);
-          const float2* hh = (const float2*)(hback.data() + sizeof(double));
+          const float2* hh = (const float2*)(hback.data() + head);
           for (int i = 0; i <= j; ++i)
             H[(size_t)i * m + j] = cd(hh[i].x, hh[i].y) + cd(hh[m + 1 + i].x, hh[m + 1 + i].y);
           H[(size_t)(j + 1) * m + j] = hn;
