@@ -96,24 +96,31 @@ void launch_split_cx(const float2* x, int64_t rows, int r, void* out, float* sca
 void launch_gemm_stage_cx(const GemmArgs& a, const TcArgs& t, unsigned* status, bool one_acc, int kind,
                           LaunchStream s);
 
-// Sliced tensor-core form (m2l_sl.cu): FP32 or FP64 products without loss of
-// precision on the FP16 tensor cores, for M, Kd multiples of 8 up to 512 and
+// Sliced tensor-core form (m2l_sl.cu): products of FP32 or FP64 accuracy on the
+// FP16 tensor cores, for M, Kd multiples of 8 up to 512 and
 // dense source rows.  src / src_scale: the source buffer's slices
-// (launch_split_sl, sl_row_bytes per row) and per-row scales; img / op_scale:
-// the operator images (build_sl_image, from the operators in FP64).  Scales are float, or double with fp64,
+// (launch_split_sl, sl_row_bytes per row) and per-row scales; img / row_scale:
+// the operator images and their scales, sl_padded_rows(M) values per operator.  Scales are float, or double with fp64,
 // where every complex array holds complex128.  Tiles hold up to
 // gemm_tc_columns() columns.
 struct SlArgs {
   const void* src;
   const void* src_scale;
   const void* img;
-  const void* op_scale;
+  const void* row_scale;
 };
 bool gemm_sl_supported(int M, int Kd);
+int sl_padded_rows(int M);
 int64_t sl_row_bytes(int r, bool fp64);
 int64_t sl_image_bytes(int M, int Kd, int nops, bool fp64);
-void build_sl_image(const double2* ops, int M, int Kd, int nops, void* img, void* scale, bool fp64, cudaStream_t s);
-void launch_split_sl(const float2* x, int64_t rows, int r, void* out, void* scale, bool fp64, LaunchStream s);
+// The scales of a source buffer's entries, Kd values, from all the operators that read it: the maxima
+// of their columns gathered into bits (cleared before), then the scales.
+void sl_column_max(const void* ops, int M, int Kd, int nops, uint32_t* bits, bool fp64, cudaStream_t s);
+void sl_column_scales(const uint32_t* bits, int Kd, void* col, bool fp64, cudaStream_t s);
+void build_sl_image(const void* ops, const void* col, int M, int Kd, int nops, void* img, void* row, bool fp64,
+                    cudaStream_t s);
+void launch_split_sl(const float2* x, const void* col, int64_t rows, int r, void* out, void* scale, bool fp64,
+                     LaunchStream s);
 void launch_gemm_stage_sl(const GemmArgs& a, const SlArgs& t, unsigned* status, bool fp64, LaunchStream s);
 
 // Permutes: fs[k][rhs] = f[rhs][perm[k]];  u[rhs][perm[k]] = us[k][rhs].  The first also

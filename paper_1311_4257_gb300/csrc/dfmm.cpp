@@ -66,7 +66,8 @@ struct GemmPlan {
   __half* img = nullptr;           // tensor-core operator image (tensor form only)
   float* op_scale = nullptr;       // its per-operator power-of-two scales
   void* sl_img = nullptr;          // sliced operator image (m2l_sl.cu; automatic form below eps 1e-5)
-  void* sl_scale = nullptr;        // its per-operator scales (float, double in the FP64 form)
+  void* sl_row = nullptr;          // its scales per operator and output (float, double in the FP64 form)
+  const void* sl_col = nullptr;    // scales of the source buffer's entries, one array per buffer
   double flops_rhs = 0;            // algorithmic flops per right-hand side
   double bytes_fixed = 0;          // operators (bytes once per launch)
   double bytes_rhs = 0;            // unique source rows + target rows (read and write), per rhs
@@ -418,20 +419,6 @@ float2* upload_projection(const std::vector<cd>& Q, int r, int halves, int R, bo
   return upload(f, ar, s);
 }
 
-// Room for the sliced operator images of a stage (m2l_sl.cu), if the plan takes the form
-// and the device has it; a stage without stays on the CUDA cores.
-bool alloc_slices(dfmm_plan_s* P, GemmPlan& g, DevArena& ar) {
-  if (!P->sliced || g.nops == 0 || !gemm_sl_supported(g.M, g.Kd)) return false;
-  try {
-    void* scale = ar.alloc<double>(g.nops);
-    g.sl_img = ar.alloc<char>(sl_image_bytes(g.M, g.Kd, g.nops, P->fp64));
-    g.sl_scale = scale;
-  } catch (const Error& e) {
-    if (e.code != DFMM_ERR_OOM) throw;
-  }
-  return g.sl_img != nullptr;
-}
-
 ChkPt* upload_chk(const std::vector<double>& pts, int n, DevArena& ar, cudaStream_t s) {
   std::vector<ChkPt> h(n);
   for (int p = 0; p < n; ++p) {
@@ -638,14 +625,7 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
   // apart within phase 3
   auto timed_form = [&](OpKind kind, const std::vector<OpSpec>& sp, const std::vector<DevRep>& dr, GemmPlan& g) {
     const double t = now();
-    OpSink sink;
-    if (alloc_slices(P, g, ar)) {
-      const int64_t per = sl_image_bytes(g.M, g.Kd, 1, P->fp64), sc = P->fp64 ? 8 : 4;
-      sink = [=, &g](const double2* ops, int first, int n) {
-        build_sl_image(ops, g.M, g.Kd, n, (char*)g.sl_img + first * per, (char*)g.sl_scale + first * sc, P->fp64, s);
-      };
-    }
-    form_ops(kind, sp, dr, g.M, g.Kd, g.ops, P->fp64, ar, s, sink);
+    form_ops(kind, sp, dr, g.M, g.Kd, g.ops, P->fp64, ar, s);
     ph[7] += now() - t;
   };
   double m2l_flops = 0, other_flops = 0;
@@ -706,12 +686,6 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
       F.p2l.src_rows = F.n_p2l * F.p2l_halves;
       F.p2l.dst_rows = LV[l].n;
       finish_gemm(F.p2l, op, pr, ar, s);
-      if (F.p2l.npairs > 0 && alloc_slices(P, F.p2l, ar)) {
-        ArenaMark mk(ar);
-        const float2* p64 = upload_projection(rp.Qi, rp.r, F.p2l_halves, R, true, ar, s);
-        build_sl_image((const double2*)p64, F.p2l.M, F.p2l.Kd, F.p2l.nops, F.p2l.sl_img, F.p2l.sl_scale, P->fp64, s);
-        DFMM_CUDA(cudaStreamSynchronize(s));
-      }
     }
     // LF-M2L over the V list: one operator per offset
     {
@@ -1493,10 +1467,10 @@ struct Runner {
     } else if (sl) {
       if (split) {
         ProfScope ps(W, s, F_SPLIT, 0.0, (double)src_rows * nrhs * (src_ld * 8.0 * P->cw + sl_row_bytes(src_ld, P->fp64)));
-        launch_split_sl(src, src_rows * nrhs, src_ld, W->sl, W->sl_scale, P->fp64, s);
+        launch_split_sl(src, g.sl_col, src_rows * nrhs, src_ld, W->sl, W->sl_scale, P->fp64, s);
       }
       ProfScope ps(W, s, g.fam, g.flops_rhs * nrhs, g.bytes_fixed + g.bytes_rhs * nrhs);
-      launch_gemm_stage_sl(a, SlArgs{W->sl, W->sl_scale, g.sl_img, g.sl_scale}, W->status, P->fp64, s);
+      launch_gemm_stage_sl(a, SlArgs{W->sl, W->sl_scale, g.sl_img, g.sl_row}, W->status, P->fp64, s);
     } else {
       ProfScope ps(W, s, g.fam, g.flops_rhs * nrhs, g.bytes_fixed + g.bytes_rhs * nrhs);
       if (few) launch_gemm_stage_few(a, s);
@@ -1888,6 +1862,65 @@ void build_images(dfmm_plan_s* P, cudaStream_t s) {
     } else {
       g->img = P->ar.alloc<__half>(tc_image_elems(g->M, g->Kd, g->nops));
       build_tc_image(g->ops, g->M, g->Kd, g->nops, g->img, g->op_scale, s);
+    }
+  }
+  DFMM_CUDA(cudaStreamSynchronize(s));
+  P->stats.plan_bytes = (int64_t)P->ar.bytes() + (P->close_keep ? (int64_t)P->close_keep->bytes() : 0);
+}
+
+// The translation stages by the source buffer that they read (as run_apply numbers them: outgoing
+// states, incoming states and check-point potentials of every level).
+std::vector<std::vector<GemmPlan*>> stages_by_source(dfmm_plan_s* P) {
+  std::vector<std::vector<GemmPlan*>> v;
+  const bool has_hf = P->l_top >= 0;
+  for (int l = has_hf ? P->l_top : P->l_lf0; l < P->nl; ++l) {
+    std::vector<GemmPlan*> out, in;
+    if (l >= P->l_lf0) {
+      out.push_back(&P->lf[l].v);
+      if (l > P->l_lf0) out.push_back(&P->lf[l - 1].m2m);
+      else if (has_hf) out.push_back(&P->hf[P->l1].m2m);
+      if (l + 1 < P->nl) in.push_back(&P->lf[l + 1].l2l);
+      v.push_back({&P->lf[l].p2l});
+    } else {
+      out.push_back(&P->hf[l].m2l);
+      if (l > P->l_top) out.push_back(&P->hf[l - 1].m2m);
+      in.push_back(l < P->l1 ? &P->hf[l + 1].l2l : &P->lf[P->l_lf0].l2l);
+    }
+    v.push_back(out);
+    v.push_back(in);
+  }
+  return v;
+}
+
+// Sliced images of every translation stage that has the form and that the device has room for (a stage
+// without one stays on the CUDA cores).  They come last, from the operators as the apply's other forms
+// hold them: the entries' scales need all the operators that read a buffer, and nothing that the plan cannot
+// do without is allocated after them.
+void build_slices(dfmm_plan_s* P, cudaStream_t s) {
+  const int64_t sc = P->fp64 ? 8 : 4;
+  DevArena& ar = P->ar;
+  uint32_t* bits = ar.alloc<uint32_t>(512);
+  for (auto& list : stages_by_source(P)) {
+    char* col = nullptr;
+    for (GemmPlan* g : list) {
+      if (g->npairs == 0 || g->nops == 0 || !gemm_sl_supported(g->M, g->Kd)) continue;
+      try {
+        if (!col) {
+          col = ar.alloc<char>(g->Kd * sc);
+          DFMM_CUDA(cudaMemsetAsync(bits, 0, 512 * sizeof(uint32_t), s));
+          for (const GemmPlan* o : list)
+            if (o->npairs > 0) sl_column_max(o->ops, o->M, o->Kd, o->nops, bits, P->fp64, s);
+          sl_column_scales(bits, g->Kd, col, P->fp64, s);
+        }
+        void* img = ar.alloc<char>(sl_image_bytes(g->M, g->Kd, g->nops, P->fp64));
+        void* row = ar.alloc<char>((int64_t)g->nops * sl_padded_rows(g->M) * sc);
+        build_sl_image(g->ops, col, g->M, g->Kd, g->nops, img, row, P->fp64, s);
+        g->sl_img = img;
+        g->sl_row = row;
+        g->sl_col = col;
+      } catch (const Error& e) {
+        if (e.code != DFMM_ERR_OOM) throw;
+      }
     }
   }
   DFMM_CUDA(cudaStreamSynchronize(s));
@@ -2353,8 +2386,8 @@ int dfmm_plan(const double* points, int64_t N, double K, double eps, const dfmm_
     P->eps = eps;
     P->opt = o;
     P->fp64 = o.arith == 64;
-    // automatic translations below eps 1e-5: the sliced tensor-core form, at least
-    // as precise as the CUDA cores and faster from the smallest stages on (apply,
+    // automatic translations below eps 1e-5: the sliced tensor-core form, with products
+    // of FP32 or FP64 accuracy (m2l_sl.cu) and faster from the smallest stages on (apply,
     // sphere of 4 wavelengths, eps 1e-6: 0.21 against 0.49 ms; of 32: 3.7 against
     // 19.5); m2l_mode 1 asks for the CUDA cores, which also serve what the form
     // does not take
@@ -2373,9 +2406,10 @@ int dfmm_plan(const double* points, int64_t N, double K, double eps, const dfmm_
     DFMM_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     struct SG { cudaStream_t s; ~SG() { cudaStreamDestroy(s); } } sg{s};
     build_plan(P.get(), points, s);
-    if (P->opt.m2l_mode == 2) {
+    if (P->opt.m2l_mode == 2 || P->sliced) {
       const double ti = now();
-      build_images(P.get(), s);
+      if (P->sliced) build_slices(P.get(), s);
+      else build_images(P.get(), s);
       DFMM_CUDA(cudaStreamSynchronize(s));
       P->stats.plan_phase_seconds[6] = now() - ti;
       P->stats.plan_seconds += P->stats.plan_phase_seconds[6];

@@ -1,9 +1,14 @@
 // Sliced tensor-core form of the translation stage y[dst] += T_op x[src] for the
 // tolerances below 1e-5, where the two-term split of m2l_cx.cu is too coarse:
-// FP32 and FP64 products on the FP16 tensor cores without loss of precision.
+// products of FP32 or FP64 accuracy on the FP16 tensor cores.
 //
-// Source rows and operators are scaled by a power of two (|v| <= 1) and cut
-// into S FP16 slices v = sum_i v_i B^-i.  The product keeps the slice pairs
+// A state's entries span many decades, and so do an operator's columns and rows: what its
+// representation resolves least is what a touching-shell operator amplifies most (eps
+// 1e-8, boxes of half a wavelength: states 2.6e2 to 1e-6, columns 0.6 to 80).  Powers of two
+// even them out first, exactly: c_q per entry of a state, the largest |T[p][q]| of all the
+// operators that read it, at most 1; d_p per row of an operator, above its |T[p][q]| / c_q; and
+// s per gathered row, above its c_q |x_q|.  The scaled values (|v| <= 1) are
+// cut into S FP16 slices v = sum_i v_i B^-i.  The product keeps the slice pairs
 // i + j < S; the pairs of one sum g = i + j share the weight B^-g and accumulate
 // in one tensor-memory accumulator ("group" g) of the FP32-accumulating MMA.
 //
@@ -11,14 +16,20 @@
 //    v_2 are FP16 numbers that hold the rest to 2^-20 and 2^-31 of the row's
 //    largest entry.  Group 0 sums integers below 2 K 2^14 <= 2^24 (K <= 512): it is
 //    exact.  The accumulators of groups 1 and 2 truncate at 2^-24 of terms that
-//    weigh 2^-8 and 2^-16, and the dropped pairs weigh 2^-27: the stage's error
-//    is the FP32 rounding of its result, below that of an FP32 FMA chain.
+//    weigh 2^-8 and 2^-16, and the dropped pairs weigh 2^-27.
 //  * FP64 rows, S = 8, B = 2^7: v = sum_i d_i 2^-(6 + 7 i) with balanced 7-bit
-//    integers |d_i| <= 64, exact to 2^-56 of the row's largest entry.  Group g
+//    integers |d_i| <= 64, to 2^-56 of the row's largest entry.  Group g
 //    sums (g + 1) 2 K products of at most 2^12, below 2^24 and so exact for
 //    (g + 1) K <= 2048; K <= 512 covers groups 0 to 3, and a truncation in group 4
 //    or later weighs 2^-24 2^-28 at most.  The epilogue joins the eight integers in
-//    64-bit arithmetic and rounds once to FP64.
+//    64-bit arithmetic, to 2^-52, and rounds to FP64.
+//
+// So the error is fixed against the largest possible product, not against each: what one stage
+// loses depends on how even the scaled values are.  Emulated on operators and states of the
+// representations (boxes of 1/2 and 1/4, offsets from touching to far and M2M; relative 2-norm
+// against 80-bit products): FP32 4e-8 to 1e-7, where an FP32 FMA chain makes 3e-7 to
+// 1e-6; FP64 4e-16 to 3e-15, where an FP64 chain makes 4e-16 to 2e-15.  With one power of two per
+// operator and per row it was 8e-8 to 8e-7 and 5e-15 to 6e-13.
 //
 // One CTA computes 128 gathered columns (pairs x right-hand sides) against a
 // block of n outputs (n <= 80, 32): operator slices of the block are stacked as
@@ -115,16 +126,6 @@ __device__ __forceinline__ void slice(float v, __half (&d)[3]) {
   d[1] = h1;
   d[2] = __float2half_rn((r - __half2float(h1)) * 256.f);
 }
-// an operator's value as formed in FP64, to the same 2^-31: no rounding to FP32 in between
-__device__ __forceinline__ void slice(double v, __half (&d)[3]) {
-  const double t = v * 128.0;
-  const double d0 = rint(t);
-  const double r = (t - d0) * 256.0;
-  const __half h1 = __float2half_rn((float)r);
-  d[0] = __float2half_rn((float)d0);
-  d[1] = h1;
-  d[2] = __float2half_rn((float)((r - (double)__half2float(h1)) * 256.0));
-}
 __device__ __forceinline__ void slice(double v, __half (&d)[8]) {
   constexpr long long kBias = 64ll * (1ll + (1ll << 7) + (1ll << 14) + (1ll << 21) + (1ll << 28) + (1ll << 35) + (1ll << 42));
   const unsigned long long I = (unsigned long long)(__double2ll_rn(v * 36028797018963968.0) + kBias);   // 2^55 v
@@ -147,39 +148,68 @@ __device__ __forceinline__ void store_pieces(unsigned char* out, const __half (*
   }
 }
 
-// Source rows (r complex values each) -> slices [row][chunk][re, im][slice][64] (r to a
-// multiple of 16 with zeros; what is left of the last chunk is not read), one scale per row.  One warp per row; a lane takes 8
-// complex values, i.e. one 16-byte piece of every slice.
+// the largest of the magnitudes of a value's parts, as bits that compare like it (of a double its high word)
+__device__ __forceinline__ uint32_t mag_bits(float2 v) {
+  return max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu);
+}
+__device__ __forceinline__ uint32_t mag_bits(double2 v) {
+  return max((uint32_t)__double2hiint(v.x) & 0x7fffffffu, (uint32_t)__double2hiint(v.y) & 0x7fffffffu);
+}
+template <class T2, class T> __device__ __forceinline__ T2 scaled(T2 v, T f) { return T2{v.x * f, v.y * f}; }
+
+// 8 consecutive values of a row, times their scales
+__device__ __forceinline__ void load_piece(const float2* x, const float* col, float2 (&v)[8]) {
+  const float4 c0 = ((const float4*)col)[0], c1 = ((const float4*)col)[1];
+  const float c[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float4 w = ((const float4*)x)[k];
+    v[2 * k] = make_float2(w.x * c[2 * k], w.y * c[2 * k]);
+    v[2 * k + 1] = make_float2(w.z * c[2 * k + 1], w.w * c[2 * k + 1]);
+  }
+}
+__device__ __forceinline__ void load_piece(const double2* x, const double* col, double2 (&v)[8]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const double2 c = ((const double2*)col)[k];
+    v[2 * k] = scaled(x[2 * k], c.x);
+    v[2 * k + 1] = scaled(x[2 * k + 1], c.y);
+  }
+}
+
+// Source rows (r complex values each, r a multiple of 8), times col[q] -> slices [row][chunk][re, im][slice][64]
+// (r to a multiple of 16 with zeros; what is left of the last chunk is not read), one scale per row.  One warp per row;
+// a lane takes 8 complex values, i.e. one 16-byte piece of every slice, and holds those of its first
+// piece (all of them up to rank 256) while the row's largest entry is found.
 template <int S, class T2, class T>
-__global__ __launch_bounds__(256) void split_sl_kernel(const T2* x, int64_t rows, int r, unsigned char* out, T* scale) {
+__global__ __launch_bounds__(256) void split_sl_kernel(const T2* x, const T* col, int64_t rows, int r, unsigned char* out,
+                                                       T* scale) {
   pdl_begin();
   const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
   const T2* xr = x + row * r;
+  const int nx = r / 8, np = round16(r) / 8;   // pieces with values, pieces
+  T2 v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = T2{T(0), T(0)};
   uint32_t m = 0;
-  for (int q = lane; q < r; q += 32) {
-    const T2 v = xr[q];
-    uint32_t a, b;
-    if constexpr (S == 3) { a = __float_as_uint(v.x); b = __float_as_uint(v.y); }
-    else { a = (uint32_t)__double2hiint(v.x); b = (uint32_t)__double2hiint(v.y); }
-    m = max(m, max(a & 0x7fffffffu, b & 0x7fffffffu));
-  }
+  if (lane < nx) load_piece(xr + 8 * lane, col + 8 * lane, v);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) m = max(m, mag_bits(v[k]));
+  for (int q = lane + 256; q < r; q += 32) m = max(m, mag_bits(scaled(xr[q], col[q])));
   m = __reduce_max_sync(0xffffffffu, m);
   T s, inv;
   if constexpr (S == 3) scale32(m, s, inv);
   else scale64(m, s, inv);
   if (lane == 0) scale[row] = s;
   const bool fin = s == s;
-  const int np = round16(r) / 8;
   unsigned char* o = out + row * (int64_t)((r + SL_K - 1) / SL_K * 2 * S * SL_ROW);
   for (int p = lane; p < np; p += 32) {
-    T2 v[8];
+    if (p >= 32 && p < nx) load_piece(xr + 8 * p, col + 8 * p, v);
+    if (!fin || p >= nx)
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      v[k] = T2{T(0), T(0)};
-      if (fin && 8 * p + k < r) v[k] = xr[8 * p + k];
-    }
+      for (int k = 0; k < 8; ++k) v[k] = T2{T(0), T(0)};
     __half d[8][S];
     unsigned char* oc = o + (p >> 3) * (2 * S * SL_ROW) + (p & 7) * 16;
 #pragma unroll
@@ -191,56 +221,79 @@ __global__ __launch_bounds__(256) void split_sl_kernel(const T2* x, int64_t rows
   }
 }
 
-// scale[op]: a power of two above the largest magnitude of an operator formed in FP64
-template <class T>
-__global__ __launch_bounds__(256) void op_scale_sl_kernel(const double2* __restrict__ ops, int64_t per_op,
-                                                          T* __restrict__ scale) {
-  __shared__ uint32_t sm;
-  if (threadIdx.x == 0) sm = 0;
+// bits[q] = max of mag_bits over the entries of column q of all operators; one block per operator
+template <class T2>
+__global__ __launch_bounds__(256) void op_col_max_kernel(const T2* __restrict__ ops, int M, int Kd, uint32_t* bits) {
+  const T2* a = ops + (int64_t)blockIdx.x * M * Kd;
+  for (int q = threadIdx.x; q < Kd; q += 256) {
+    uint32_t m = 0;
+    for (int p = 0; p < M; ++p) m = max(m, mag_bits(a[(int64_t)p * Kd + q]));
+    atomicMax(bits + q, m);
+  }
+}
+
+// col[q] = the power of two of column q over that of the largest column, at least 2^-100, and 1 where
+// nothing reads the entry (padding); one block
+template <class T, int MANT>
+__global__ __launch_bounds__(512) void op_col_scale_kernel(const uint32_t* __restrict__ bits, int Kd, T* __restrict__ col) {
+  __shared__ int top;
+  if (threadIdx.x == 0) top = 0;
   __syncthreads();
-  const double2* a = ops + (int64_t)blockIdx.x * per_op;
+  const int q = threadIdx.x, e = q < Kd ? (int)(bits[q] >> MANT) : 0;
+  atomicMax(&top, e);
+  __syncthreads();
+  if (q < Kd) col[q] = bits[q] == 0 ? T(1) : (T)__uint_as_float((uint32_t)(127 + max(e - top, -100)) << 23);
+}
+
+// row[op][p] (rows of Mp values): a power of two above |T[p][q]| / col[q] for every q, times the unit
+// that the groups are joined in; a warp per row
+template <class T> __host__ __device__ constexpr T sl_unit() { return sizeof(T) == 4 ? T(6.103515625e-05) : T(2.220446049250313e-16); }   // 2^-14, 2^-52
+
+template <class T2, class T>
+__global__ __launch_bounds__(256) void op_row_scale_kernel(const T2* __restrict__ ops, const T* __restrict__ col, int M,
+                                                           int Kd, int Mp, int64_t rows, T* __restrict__ row) {
+  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (i >= rows) return;
+  const T2* a = ops + i * Kd;
   uint32_t m = 0;
-  for (int64_t q = threadIdx.x; q < per_op; q += blockDim.x) {
-    const double2 v = a[q];
-    m = max(m, max((uint32_t)__double2hiint(v.x) & 0x7fffffffu, (uint32_t)__double2hiint(v.y) & 0x7fffffffu));
-  }
-  atomicMax(&sm, m);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s, inv;
-    scale64(sm, s, inv);
-    scale[blockIdx.x] = (T)s;
-  }
+  for (int q = lane; q < Kd; q += 32) m = max(m, mag_bits(scaled(a[q], T(1) / col[q])));
+  m = __reduce_max_sync(0xffffffffu, m);
+  T s, inv;
+  if constexpr (sizeof(T) == 4) scale32(m, s, inv);
+  else scale64(m, s, inv);
+  if (lane == 0) row[i / M * Mp + i % M] = s * sl_unit<T>();
 }
 
 // Operator image [op][block][chunk][Tr, Ti][slice][row of the block][64], zero beyond M
 // and Kd, each row of 128 bytes swizzled as the MMA reads it: a chunk is one
 // bulk copy and the slices of Tr (or Ti) are one stacked operand.  One block per (op, chunk).
-template <int S, class T>
-__global__ __launch_bounds__(256) void op_image_sl_kernel(const double2* __restrict__ ops, const T* __restrict__ scale,
-                                                          int M, int Kd, unsigned char* __restrict__ img) {
+template <int S, class T2, class T>
+__global__ __launch_bounds__(256) void op_image_sl_kernel(const T2* __restrict__ ops, const T* __restrict__ col,
+                                                          const T* __restrict__ rows, int M, int Kd,
+                                                          unsigned char* __restrict__ img) {
   const int nchunk = (Kd + SL_K - 1) / SL_K, Mp = round16(M), n = block_rows<S>(M);
   const int64_t op = blockIdx.x / nchunk;
   const int c = (int)(blockIdx.x % nchunk);
-  const double2* top = ops + op * (int64_t)M * Kd;
+  const T2* top = ops + op * (int64_t)M * Kd;
   unsigned char* base = img + op * (int64_t)nchunk * 2 * S * SL_ROW * Mp;
-  const double inv = 1.0 / (double)scale[op];
   for (int e = threadIdx.x; e < Mp * 8; e += blockDim.x) {
     const int p = e >> 3, pc = e & 7;
     const int blk = p / n, row = p - blk * n, nb = min(n, Mp - blk * n);
     unsigned char* o = base + (int64_t)blk * n * (nchunk * 2 * S * SL_ROW) + (int64_t)c * (2 * S * SL_ROW * nb);
-    double2 v[8];
+    const T inv = p < M ? sl_unit<T>() / rows[op * Mp + p] : T(0);
+    T2 v[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int q = c * SL_K + 8 * pc + k;
-      v[k] = make_double2(0.0, 0.0);
-      if (p < M && q < Kd) v[k] = top[(int64_t)p * Kd + q];
+      v[k] = T2{T(0), T(0)};
+      if (p < M && q < Kd) v[k] = scaled(scaled(top[(int64_t)p * Kd + q], T(1) / col[q]), inv);
     }
 #pragma unroll
     for (int part = 0; part < 2; ++part) {
       __half d[8][S];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) slice((part ? v[k].y : v[k].x) * inv, d[k]);
+      for (int k = 0; k < 8; ++k) slice(part ? v[k].y : v[k].x, d[k]);
 #pragma unroll
       for (int i = 0; i < S; ++i) {
         __half2 w[4];
@@ -266,11 +319,11 @@ __device__ __forceinline__ void red_add_f64(double* p, double v) {
   asm volatile("red.relaxed.gpu.global.add.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
 }
 
-// The groups of one output, r[4 g] the group's accumulator, as the stage's value / (column scale).
+// The groups of one output, r[4 g] the group's accumulator, as the stage's value / (row scale x column scale).
 __device__ __forceinline__ float join3(const uint32_t* r) {
   return __uint_as_float(r[0]) + (__uint_as_float(r[4]) + __uint_as_float(r[8]) * 0.00390625f) * 0.00390625f;
 }
-// unit 2^-52: |sum| <= 2 K <= 2^10, so the 64-bit integer does not overflow
+// |sum| <= 2 K <= 2^10, in units of 2^-52, so the 64-bit integer does not overflow
 __device__ __forceinline__ double join8(const uint32_t* r) {
   int s[8];
 #pragma unroll
@@ -508,9 +561,9 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
           out[h] = (T*)((T2*)a.dst + ((int64_t)pr.y * a.nrhs + k) * a.dst_ld) + 2 * blk * n + 4 * (lane & 3);
         }
       }
-      // the slices' units: 2^-14 (S = 3), 2^-52 (S = 8)
-      const T so = ((const T*)t.op_scale)[tile.x] * (S == 3 ? T(6.103515625e-05) : T(2.220446049250313e-16));
       const int nout = min(nb, M - blk * n);   // outputs of the block; the rest pads it
+      // row scales of this thread's outputs, 8 (2 j + par) + 2 (lane % 4) + {0, 1}
+      const T2* rs = (const T2*)((const T*)t.row_scale + (int64_t)tile.x * Mp + blk * n + 8 * par + 2 * (lane & 3));
       int okw = 0;
       if (lane == 0) okw = mbar_wait(smem_u32(acc_full), (uint32_t)(i & 1), status) ? 1 : 0;
       okw = __shfl_sync(0xffffffffu, okw, 0);
@@ -545,6 +598,9 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(acc_empty)) : "memory");
+      T2 so[STEPS];   // loaded here: the registers were the accumulators' until now
+#pragma unroll
+      for (int j = 0; j < STEPS; ++j) so[j] = 8 * (2 * j + par) < nout ? rs[8 * j] : T2{T(0), T(0)};
 #pragma unroll
       for (int b = 0; b < 2; ++b)
 #pragma unroll
@@ -558,12 +614,11 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
             if (out[2 * b + h]) {
               if constexpr (S == 3) {
                 const float c = cs[2 * b + h];
-                const float y0 = v[0] * so * c, y1 = v[1] * so * c, y2 = v[2] * so * c, y3 = v[3] * so * c;
-                red_add4(o, y0, y1, y2, y3);
+                red_add4(o, v[0] * so[j].x * c, v[1] * so[j].x * c, v[2] * so[j].y * c, v[3] * so[j].y * c);
               } else {
-                const double c = so * cs[2 * b + h];
+                const double c0 = so[j].x * cs[2 * b + h], c1 = so[j].y * cs[2 * b + h];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) red_add_f64(o + e, v[e] * c);
+                for (int e = 0; e < 4; ++e) red_add_f64(o + e, v[e] * (e < 2 ? c0 : c1));
               }
             }
           }
@@ -604,28 +659,49 @@ int64_t sl_row_bytes(int r, bool fp64) { return (int64_t)((r + SL_K - 1) / SL_K)
 
 int64_t sl_image_bytes(int M, int Kd, int nops, bool fp64) { return (int64_t)nops * round16(M) * sl_row_bytes(Kd, fp64); }
 
-void build_sl_image(const double2* ops, int M, int Kd, int nops, void* img, void* scale, bool fp64, cudaStream_t s) {
+int sl_padded_rows(int M) { return round16(M); }
+
+void sl_column_max(const void* ops, int M, int Kd, int nops, uint32_t* bits, bool fp64, cudaStream_t s) {
   if (nops == 0) return;
-  if (!gemm_sl_supported(M, Kd)) throw Error(-5, "sliced stage needs ranks that are multiples of 8, <= 512");
-  const unsigned blocks = (unsigned)((int64_t)nops * ((Kd + SL_K - 1) / SL_K));
-  unsigned char* p = (unsigned char*)img;
-  if (fp64) {
-    op_scale_sl_kernel<<<nops, 256, 0, s>>>(ops, (int64_t)M * Kd, (double*)scale);
-    op_image_sl_kernel<8><<<blocks, 256, 0, s>>>(ops, (const double*)scale, M, Kd, p);
-  } else {
-    op_scale_sl_kernel<<<nops, 256, 0, s>>>(ops, (int64_t)M * Kd, (float*)scale);
-    op_image_sl_kernel<3><<<blocks, 256, 0, s>>>(ops, (const float*)scale, M, Kd, p);
-  }
+  if (fp64) op_col_max_kernel<<<nops, 256, 0, s>>>((const double2*)ops, M, Kd, bits);
+  else op_col_max_kernel<<<nops, 256, 0, s>>>((const float2*)ops, M, Kd, bits);
   DFMM_CUDA(cudaGetLastError());
 }
 
-void launch_split_sl(const float2* x, int64_t rows, int r, void* out, void* scale, bool fp64, LaunchStream s) {
+void sl_column_scales(const uint32_t* bits, int Kd, void* col, bool fp64, cudaStream_t s) {
+  if (Kd > SL_KMAX) throw Error(-5, "sliced stage needs ranks up to 512");
+  if (fp64) op_col_scale_kernel<double, 20><<<1, SL_KMAX, 0, s>>>(bits, Kd, (double*)col);
+  else op_col_scale_kernel<float, 23><<<1, SL_KMAX, 0, s>>>(bits, Kd, (float*)col);
+  DFMM_CUDA(cudaGetLastError());
+}
+
+template <int S, class T2, class T>
+void build_sl(const T2* ops, const T* col, int M, int Kd, int nops, unsigned char* img, T* row, cudaStream_t s) {
+  const int64_t rows = (int64_t)nops * M;
+  op_row_scale_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(ops, col, M, Kd, round16(M), rows, row);
+  op_image_sl_kernel<S><<<(unsigned)((int64_t)nops * ((Kd + SL_K - 1) / SL_K)), 256, 0, s>>>(ops, col, row, M, Kd, img);
+  DFMM_CUDA(cudaGetLastError());
+}
+
+void build_sl_image(const void* ops, const void* col, int M, int Kd, int nops, void* img, void* row, bool fp64,
+                    cudaStream_t s) {
+  if (nops == 0) return;
+  if (!gemm_sl_supported(M, Kd)) throw Error(-5, "sliced stage needs ranks that are multiples of 8, <= 512");
+  unsigned char* p = (unsigned char*)img;
+  if (fp64) build_sl<8>((const double2*)ops, (const double*)col, M, Kd, nops, p, (double*)row, s);
+  else build_sl<3>((const float2*)ops, (const float*)col, M, Kd, nops, p, (float*)row, s);
+}
+
+void launch_split_sl(const float2* x, const void* col, int64_t rows, int r, void* out, void* scale, bool fp64,
+                     LaunchStream s) {
   if (rows == 0) return;
   const unsigned grid = (unsigned)((rows * 32 + 255) / 256);
   if (fp64)
-    launch_pdl(split_sl_kernel<8, double2, double>, grid, 256, 0, s, (const double2*)x, rows, r, (unsigned char*)out, (double*)scale);
+    launch_pdl(split_sl_kernel<8, double2, double>, grid, 256, 0, s, (const double2*)x, (const double*)col, rows, r,
+               (unsigned char*)out, (double*)scale);
   else
-    launch_pdl(split_sl_kernel<3, float2, float>, grid, 256, 0, s, x, rows, r, (unsigned char*)out, (float*)scale);
+    launch_pdl(split_sl_kernel<3, float2, float>, grid, 256, 0, s, x, (const float*)col, rows, r, (unsigned char*)out,
+               (float*)scale);
   DFMM_CUDA(cudaGetLastError());
 }
 

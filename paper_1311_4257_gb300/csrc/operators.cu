@@ -208,7 +208,7 @@ DevRep upload_rep(const Rep& rep, int R, DevArena& ar, cudaStream_t s) {
 }
 
 void form_ops(OpKind kind, const std::vector<OpSpec>& ops, const std::vector<DevRep>& reps, int Rt, int Rs,
-              void* out, bool fp64, DevArena& ar, cudaStream_t s, const OpSink& sink) {
+              void* out, bool fp64, DevArena& ar, cudaStream_t s) {
   if (ops.empty()) return;
   ArenaMark mark(ar);
   DevRep* d_reps = ar.alloc<DevRep>(reps.size());
@@ -260,7 +260,6 @@ void form_ops(OpKind kind, const std::vector<OpSpec>& ops, const std::vector<Dev
     DFMM_CUDA(cudaMemcpyAsync(pC, hC.data(), nb * sizeof(void*), cudaMemcpyHostToDevice, s));
     zgemm(pA, pB, pC, nb, Rt, Rs, Rs, Rs, Rs, Rs, false, s);
     store_out(T2, out, (int64_t)start * Rt * Rs, (int64_t)nb * Rt * Rs, fp64, s);
-    if (sink) sink(T2, start, nb);
     DFMM_CUDA(cudaStreamSynchronize(s));
   }
 }

@@ -1,6 +1,5 @@
 // Plan-time formation of the translation operators in FP64 (see operators.cu).
 #pragma once
-#include <functional>
 #include <vector>
 
 #include "common.h"
@@ -37,12 +36,9 @@ struct OpSpec {
 
 // Forms ops (all of one kind, one pair of width classes R_t, R_s) and writes
 // them as complex64 [n][R_t][R_s] into out (device), or as complex128 when
-// fp64 is set (the FP64 form of the apply).  sink, if set, is also given every
-// batch in FP64 on the device, as (operators, index of the first, how many),
-// before the batch's memory is used again on `s`.
-using OpSink = std::function<void(const double2*, int, int)>;
+// fp64 is set (the FP64 form of the apply).
 void form_ops(OpKind kind, const std::vector<OpSpec>& ops, const std::vector<DevRep>& reps, int Rt, int Rs,
-              void* out, bool fp64, DevArena& ar, cudaStream_t s, const OpSink& sink = OpSink());
+              void* out, bool fp64, DevArena& ar, cudaStream_t s);
 
 // Rows for evaluating a representation at points:
 //   L2P (incoming): row_i = G(y_i - c, a_in) W Ri^{-1}
