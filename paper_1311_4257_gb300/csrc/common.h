@@ -20,6 +20,10 @@ struct Error : std::runtime_error {
                           std::string(#call) + ": " + cudaGetErrorString(e_));             \
   } while (0)
 
+// cudaMalloc that, before it reports that the device is full, has plans give up memory that only makes them
+// faster (operator images, dfmm.cpp).
+cudaError_t device_malloc(void** p, size_t bytes);
+
 constexpr int kLevelBits = 21;   // Morton bits per axis; deepest level
 constexpr int kMaxLevels = 22;
 

@@ -148,10 +148,77 @@ struct M2PGroup {
   int64_t nrows = 0;
 };
 
+// The sliced operator images of a plan (m2l_sl.cu): memory that makes its applies faster and that they can do
+// without.  When the device is full (device_malloc) it is given back, unless somebody uses it: an apply
+// being queued, a workspace laid out for it that lives on, a captured apply.
+struct SliceImages {
+  DevArena ar;
+  int device = 0;
+  std::mutex mu;
+  int users = 0;
+  bool gone = false;
+  bool acquire() {
+    std::lock_guard<std::mutex> g(mu);
+    if (gone) return false;
+    ++users;
+    return true;
+  }
+  void release() {
+    std::lock_guard<std::mutex> g(mu);
+    --users;
+  }
+  bool there() {
+    std::lock_guard<std::mutex> g(mu);
+    return !gone;
+  }
+};
+std::mutex g_images_mu;
+std::vector<std::weak_ptr<SliceImages>> g_images;   // of every live plan that has some
+
+// Frees the largest unused set of images on the current device; false if there is none.
+bool reclaim_images() {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::shared_ptr<SliceImages> most;
+  {
+    std::lock_guard<std::mutex> g(g_images_mu);
+    for (auto& w : g_images)
+      if (auto im = w.lock()) {
+        std::lock_guard<std::mutex> gi(im->mu);
+        if (im->device == dev && im->users == 0 && !im->gone && (!most || im->ar.bytes() > most->ar.bytes())) most = im;
+      }
+    if (!most) return false;
+    std::lock_guard<std::mutex> gi(most->mu);
+    if (most->users) return false;
+    most->gone = true;   // no apply queued from now on reads them
+  }
+  if (cudaDeviceSynchronize() != cudaSuccess) {   // not allowed while this thread captures a stream
+    cudaGetLastError();
+    std::lock_guard<std::mutex> gi(most->mu);
+    most->gone = false;
+    return false;
+  }
+  most->ar.release(0);
+  return true;
+}
+
+// Holds a plan's images for as long as it lives.
+struct SliceUse {
+  std::shared_ptr<SliceImages> im;
+  explicit SliceUse(std::shared_ptr<SliceImages> p) {
+    if (p && p->acquire()) im = std::move(p);
+  }
+  SliceUse(const SliceUse&) = delete;
+  ~SliceUse() {
+    if (im) im->release();
+  }
+};
+
 struct Workspace {
   int nrhs = 0;
   bool external = false;   // buffers carved from caller-provided memory
   bool full = true;        // not the least layout: with work tiles for the few-column form
+  std::unique_ptr<SliceUse> slices;   // a carved workspace with a sliced source buffer holds its plan's images
   DevArena ar;
   float2 *fs = nullptr, *us = nullptr;
   std::vector<float2*> p2l;                             // per level: potentials at the P2L check points
@@ -220,6 +287,7 @@ struct dfmm_plan_s {
   bool fp64 = false;   // FP64 form (options.arith 64): complex128 densities, states and operators
   bool few = false;    // stages of few columns per operator may run in their own form (gemm_few.cu)
   bool sliced = false; // translations in the sliced tensor-core form (automatic form below eps 1e-5)
+  std::shared_ptr<SliceImages> images;   // its operator images, if it has any
   int cw = 1;          // complex element width in float2 units (2 in the FP64 form)
   DevArena ar;
   TreeBuilder tree;
@@ -1256,13 +1324,9 @@ Workspace* get_workspace(dfmm_plan_s* P, cudaStream_t s, int nrhs) {
     W->zero.push_back({W->S[l], (size_t)rows * nrhs * R * 8 * cw});
     W->zero.push_back({W->T[l], (size_t)rows * nrhs * R * 8 * cw});
   }
-  try {
-    set_p2l(P, *W, ar.alloc<float2>(p2l_elems(P, true) * nrhs * cw), nrhs, true);
-  } catch (const Error& e) {   // no room for every level's: one array serves them in turn
-    if (e.code != DFMM_ERR_OOM) throw;
-    cudaGetLastError();
+  if (float2* all = ar.try_alloc<float2>(p2l_elems(P, true) * nrhs * cw)) set_p2l(P, *W, all, nrhs, true);
+  else   // no room for every level's: one array serves them in turn
     set_p2l(P, *W, ar.alloc<float2>(p2l_elems(P, false) * nrhs * cw), nrhs, false);
-  }
   if (P->opt.m2l_mode == 2) {
     // split arrays: 2 values per complex element, 2 bytes each (4 for the TF32 split)
     int64_t e = max_source_elems(P) * nrhs * 2 * (P->opt.tc_precision == 2 ? 2 : 1);
@@ -1270,19 +1334,18 @@ Workspace* get_workspace(dfmm_plan_s* P, cudaStream_t s, int nrhs) {
     W->alo = W->ahi + e;
     W->ascale = ar.alloc<float>(max_source_rows(P) * nrhs);
   }
-  if (P->sliced) {
-    try {
-      W->sl = ar.alloc<char>(max_slice_bytes(P) * nrhs);
-      W->sl_scale = ar.alloc<double>(max_source_rows(P) * nrhs);
-    } catch (const Error& e) {   // no room for the slices: the stages run on the CUDA cores
-      if (e.code != DFMM_ERR_OOM) throw;
-      cudaGetLastError();
-      W->sl = W->sl_scale = nullptr;
-    }
-  }
   W->status = ar.alloc<unsigned>(1);
   W->zero.push_back({W->status, 4});   // reset by every apply; read by dfmm_sync_status
   DFMM_CUDA(cudaMemsetAsync(W->status, 0, 4, s));
+  if (P->images && P->images->there()) {   // last: without room for the slices the stages run on the CUDA cores
+    const size_t m = ar.mark();
+    W->sl = ar.try_alloc<char>(max_slice_bytes(P) * nrhs);
+    W->sl_scale = W->sl ? ar.try_alloc<double>(max_source_rows(P) * nrhs) : nullptr;
+    if (!W->sl_scale) {
+      ar.release(m);
+      W->sl = nullptr;
+    }
+  }
   return W;
 }
 
@@ -1301,7 +1364,7 @@ bool split_complex(const dfmm_plan_s* P, const GemmPlan& g) {
 }
 
 // whether a stage has the sliced form (m2l_sl.cu): operators sliced at plan time; it runs so
-// where the workspace holds the slices of its source
+// while the plan has the images and where the workspace holds the slices of its source
 bool sliced_stage(const GemmPlan& g) { return g.sl_img != nullptr; }
 
 // whether a stage runs in the few-column form (gemm_few.cu): its operators serve so few
@@ -1312,7 +1375,7 @@ bool few_columns(const dfmm_plan_s* P, const GemmPlan& g, int nrhs) {
   return P->few && g.npairs * nrhs <= cols * ops;
 }
 
-// columns of a stage's work tiles (full: in a full layout; slices: the workspace holds its source's slices)
+// columns of a stage's work tiles (full: in a full layout; slices: images and source slices are there)
 int tile_columns(const dfmm_plan_s* P, const GemmPlan& g, int nrhs, bool full, bool slices) {
   if (full && few_columns(P, g, nrhs)) return gemm_few_columns();
   return on_tensor_cores(P, g) || (slices && sliced_stage(g)) ? gemm_tc_columns() : 64;
@@ -1393,6 +1456,7 @@ struct Runner {
   LaunchStream s;
   int nrhs;
   int64_t* count;   // dry run: count launches only
+  bool slices = true;   // sliced stages run as such
   WaveCtl* ctl = nullptr;
   int64_t cur = 0;  // wave key of the next step
 
@@ -1428,7 +1492,7 @@ struct Runner {
     const bool few = (count || W->full) && few_columns(P, g, nrhs);
     const bool tc = !few && on_tensor_cores(P, g);
     const bool cx = tc && split_complex(P, g);
-    const bool sl = !few && sliced_stage(g) && (count || W->sl);
+    const bool sl = !few && sliced_stage(g) && (count || slices);
     // the split arrays hold one source buffer in one layout (interleaved or split-complex)
     const int key = src_key < 0 ? -1 : 2 * src_key + (cx ? 1 : 0);
     const bool split = (tc || sl) && (key < 0 || key != split_key);
@@ -1439,7 +1503,7 @@ struct Runner {
       ctl->collect->push_back(WaveGemm{P, W, &g, src, src_ld, src_rows, dst, dst_ld, nrhs, split});
       return;
     }
-    auto t = tiles_for(P, W, g, nrhs, tile_columns(P, g, nrhs, W->full, W->sl != nullptr), s);
+    auto t = tiles_for(P, W, g, nrhs, tile_columns(P, g, nrhs, W->full, slices), s);
     GemmArgs a;
     a.ops = g.ops;
     a.M = g.M;
@@ -1503,6 +1567,13 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
   const LaunchStream s(stream, P->N * nrhs <= kEarlyLaunch);
   Runner R{P, W, s, nrhs, count};
   R.ctl = ctl;
+  SliceUse use(!count && W->sl ? P->images : nullptr);
+  R.slices = use.im != nullptr;
+  if (use.im && !W->slices) {   // a capture of the caller's reads the images whenever it is replayed
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) cudaGetLastError();
+    else if (cap != cudaStreamCaptureStatusNone) use.im->acquire();
+  }
   const int64_t lW = (int64_t)std::llround(std::log2(P->W));
   auto lw = [&](int l) -> int64_t { return lW - l; };   // log2 of the width of level l
   const int64_t N = P->N;
@@ -1754,10 +1825,11 @@ std::vector<const GemmPlan*> all_gemms(dfmm_plan_s* P) {
 // [base, base + bytes): the device status word (at offset 0), state buffers,
 // staging buffers and the work tiles of every stage (copied in on `s`).  No device memory is allocated.  With
 // base == nullptr nothing is laid out or copied: the return value is the
-// number of bytes the layout needs.  full: with the sliced form's source buffer,
-// without which the plan's sliced stages run on the CUDA cores, P2L rows for every
-// level and the few-column form's work tiles; without them an apply runs in no more than it always did.
-size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaStream_t s, Workspace& W, bool full) {
+// number of bytes the layout needs.  full: with P2L rows for every
+// level and the few-column form's work tiles, and, if slices is set, the sliced form's source buffer,
+// without which the plan's sliced stages run on the CUDA cores; without them an apply runs in no more than it always did.
+size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaStream_t s, Workspace& W, bool full,
+                       bool slices) {
   size_t off = 0;
   auto take = [&](size_t n) -> char* {
     off = (off + 255) & ~(size_t)255;
@@ -1799,7 +1871,7 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
     W.alo = W.ahi + e;
     W.ascale = (float*)take((size_t)max_source_rows(P) * nrhs * 4);
   }
-  const bool slices = full && P->sliced;
+  slices = slices && full;
   if (slices) {
     W.sl = take((size_t)max_slice_bytes(P) * nrhs);
     W.sl_scale = take((size_t)max_source_rows(P) * nrhs * 8);
@@ -1828,26 +1900,24 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
 
 // Device bytes of one apply's workspace with nrhs right-hand sides: the least an
 // apply runs in, or (full) with room for what makes it faster.
-int64_t workspace_bytes(dfmm_plan_s* P, int nrhs, bool full) {
+int64_t workspace_bytes(dfmm_plan_s* P, int nrhs, bool full, bool slices = false) {
   Workspace W;
-  return (int64_t)carve_workspace(P, nrhs, nullptr, 0, nullptr, W, full);
+  return (int64_t)carve_workspace(P, nrhs, nullptr, 0, nullptr, W, full, slices);
 }
 
-// A carved workspace of its own in `ar`: the full layout, or where it does not fit the device, the least.
+// A carved workspace of its own in `ar`, for applies that live on: the full layout, or where it does not fit
+// the device, the least.
 void own_workspace(dfmm_plan_s* P, int nrhs, DevArena& ar, cudaStream_t s, Workspace& W) {
-  bool full = true;
-  size_t bytes = (size_t)workspace_bytes(P, nrhs, full);
-  char* base = nullptr;
-  try {
-    base = ar.alloc<char>((int64_t)bytes);
-  } catch (const Error& e) {
-    if (e.code != DFMM_ERR_OOM) throw;
-    cudaGetLastError();
-    full = false;
+  W.slices.reset(new SliceUse(P->images));
+  size_t bytes = (size_t)workspace_bytes(P, nrhs, true, W.slices->im != nullptr);
+  char* base = ar.try_alloc<char>((int64_t)bytes);
+  const bool full = base != nullptr;
+  if (!full) {
+    W.slices.reset();
     bytes = (size_t)workspace_bytes(P, nrhs, false);
     base = ar.alloc<char>((int64_t)bytes);
   }
-  carve_workspace(P, nrhs, base, bytes, s, W, full);
+  carve_workspace(P, nrhs, base, bytes, s, W, full, full && W.slices->im);
 }
 
 // Operator images of every translation stage for the tensor-core form.
@@ -1894,37 +1964,57 @@ std::vector<std::vector<GemmPlan*>> stages_by_source(dfmm_plan_s* P) {
 
 // Sliced images of every translation stage that has the form and that the device has room for (a stage
 // without one stays on the CUDA cores).  They come last, from the operators as the apply's other forms
-// hold them: the entries' scales need all the operators that read a buffer, and nothing that the plan cannot
-// do without is allocated after them.
+// hold them: the entries' scales need all the operators that read a buffer, and what the plan cannot
+// do without is there by then.  An eighth of the device stays free for workspaces, further plans and other
+// users of it.
 void build_slices(dfmm_plan_s* P, cudaStream_t s) {
   const int64_t sc = P->fp64 ? 8 : 4;
-  DevArena& ar = P->ar;
-  uint32_t* bits = ar.alloc<uint32_t>(512);
+  auto images = std::make_shared<SliceImages>();
+  DFMM_CUDA(cudaGetDevice(&images->device));
+  DevArena& ar = images->ar;
+  size_t free = 0, total = 0;
+  DFMM_CUDA(cudaMemGetInfo(&free, &total));
+  const size_t spare = free > total / 8 ? free - total / 8 : 0;
+  uint32_t* bits = ar.try_alloc<uint32_t>(512);
+  if (!bits) return;
   for (auto& list : stages_by_source(P)) {
     char* col = nullptr;
     for (GemmPlan* g : list) {
       if (g->npairs == 0 || g->nops == 0 || !gemm_sl_supported(g->M, g->Kd)) continue;
-      try {
-        if (!col) {
-          col = ar.alloc<char>(g->Kd * sc);
-          DFMM_CUDA(cudaMemsetAsync(bits, 0, 512 * sizeof(uint32_t), s));
-          for (const GemmPlan* o : list)
-            if (o->npairs > 0) sl_column_max(o->ops, o->M, o->Kd, o->nops, bits, P->fp64, s);
-          sl_column_scales(bits, g->Kd, col, P->fp64, s);
-        }
-        void* img = ar.alloc<char>(sl_image_bytes(g->M, g->Kd, g->nops, P->fp64));
-        void* row = ar.alloc<char>((int64_t)g->nops * sl_padded_rows(g->M) * sc);
-        build_sl_image(g->ops, col, g->M, g->Kd, g->nops, img, row, P->fp64, s);
-        g->sl_img = img;
-        g->sl_row = row;
-        g->sl_col = col;
-      } catch (const Error& e) {
-        if (e.code != DFMM_ERR_OOM) throw;
+      if (!col) {
+        col = ar.try_alloc<char>(g->Kd * sc);
+        if (!col) continue;
+        DFMM_CUDA(cudaMemsetAsync(bits, 0, 512 * sizeof(uint32_t), s));
+        for (const GemmPlan* o : list)
+          if (o->npairs > 0) sl_column_max(o->ops, o->M, o->Kd, o->nops, bits, P->fp64, s);
+        sl_column_scales(bits, g->Kd, col, P->fp64, s);
       }
+      const size_t m = ar.mark();
+      const int64_t bytes = sl_image_bytes(g->M, g->Kd, g->nops, P->fp64);
+      void* img = ar.bytes() + bytes <= spare ? ar.try_alloc<char>(bytes) : nullptr;
+      void* row = img ? ar.try_alloc<char>((int64_t)g->nops * sl_padded_rows(g->M) * sc) : nullptr;
+      if (!row) {
+        ar.release(m);
+        continue;
+      }
+      build_sl_image(g->ops, col, g->M, g->Kd, g->nops, img, row, P->fp64, s);
+      g->sl_img = img;
+      g->sl_row = row;
+      g->sl_col = col;
+      P->images = images;
     }
   }
   DFMM_CUDA(cudaStreamSynchronize(s));
-  P->stats.plan_bytes = (int64_t)P->ar.bytes() + (P->close_keep ? (int64_t)P->close_keep->bytes() : 0);
+  if (P->images) {
+    std::lock_guard<std::mutex> g(g_images_mu);
+    g_images.erase(std::remove_if(g_images.begin(), g_images.end(), [](auto& w) { return w.expired(); }), g_images.end());
+    g_images.push_back(images);
+  }
+}
+
+// Device bytes that the plan holds now.
+int64_t plan_bytes(const dfmm_plan_s* P) {
+  return P->stats.plan_bytes + (P->images && P->images->there() ? (int64_t)P->images->ar.bytes() : 0);
 }
 
 // Bounds checks of every index table of the plan and of the work tiles of
@@ -2061,6 +2151,15 @@ namespace dfmm {
 
 int set_error(int code, const char* msg) { return fail(code, msg); }
 
+cudaError_t device_malloc(void** p, size_t bytes) {
+  cudaError_t e;
+  while ((e = cudaMalloc(p, bytes)) == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    if (!reclaim_images()) break;
+  }
+  return e;
+}
+
 bool plan_acquire(const dfmm_plan_s* plan) {
   std::lock_guard<std::mutex> g(g_plans_mu);
   auto it = g_plans.find(plan);
@@ -2098,8 +2197,9 @@ int apply_with_scratch(dfmm_plan_s* P, const void* f, void* u, int nrhs, cudaStr
     if (dev != P->device) return fail(DFMM_ERR_INVALID, "the plan belongs to another device");
     Workspace W;
     // the sliced form where the scratch holds its source slices as well
-    const bool full = (size_t)workspace_bytes(P, nrhs, true) <= bytes;
-    carve_workspace(P, nrhs, (char*)scratch, bytes, stream, W, full);
+    SliceUse use(P->images);
+    const bool slices = use.im != nullptr, full = (size_t)workspace_bytes(P, nrhs, true, slices) <= bytes;
+    carve_workspace(P, nrhs, (char*)scratch, bytes, stream, W, full, slices);
     run_apply(P, (const float2*)f, (float2*)u, nrhs, stream, nullptr, &W);
     return DFMM_OK;
   });
@@ -2501,6 +2601,7 @@ int dfmm_destroy(dfmm_plan_t plan) {
 int dfmm_plan_stats(dfmm_plan_t plan, dfmm_stats* out) {
   if (!plan || !out) return fail(DFMM_ERR_INVALID, "null argument");
   *out = plan->stats;
+  out->plan_bytes = plan_bytes(plan);
   return DFMM_OK;
 }
 
@@ -2513,7 +2614,7 @@ int64_t dfmm_apply_workspace_bytes(dfmm_plan_t plan, int nrhs) {
   }
 }
 
-int64_t dfmm_plan_bytes(dfmm_plan_t plan) { return plan ? plan->stats.plan_bytes : -1; }
+int64_t dfmm_plan_bytes(dfmm_plan_t plan) { return plan ? plan_bytes(plan) : -1; }
 
 int dfmm_graph_create(dfmm_plan_t plan, const void* f, void* u, int nrhs, cudaStream_t stream, dfmm_graph_t* out) {
   return guarded([&]() -> int {

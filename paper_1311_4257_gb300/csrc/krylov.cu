@@ -62,7 +62,6 @@ __global__ __launch_bounds__(KV_T) void dots_kernel(const float2* V, int ncols, 
                                                     unsigned* counter, StatusGather st, int64_t N) {
   __shared__ float2 sums[KV_GROUP][KV_T / 32];
   pdl_begin();
-  gather(st);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t i0 = (int64_t)blockIdx.x * KV_BLOCK + threadIdx.x;
   float2 wv[KV_ROWS];
@@ -112,6 +111,7 @@ __global__ __launch_bounds__(KV_T) void dots_kernel(const float2* V, int ncols, 
       part[(int64_t)(c0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
     }
   }
+  gather(st);
   if (!last_block(counter)) return;
   for (int c = warp; c < ncols; c += KV_T / 32) {
     double2 t = make_double2(0.0, 0.0);

@@ -562,8 +562,11 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
         }
       }
       const int nout = min(nb, M - blk * n);   // outputs of the block; the rest pads it
-      // row scales of this thread's outputs, 8 (2 j + par) + 2 (lane % 4) + {0, 1}
-      const T2* rs = (const T2*)((const T*)t.row_scale + (int64_t)tile.x * Mp + blk * n + 8 * par + 2 * (lane & 3));
+      // row scales: of this thread's outputs, 8 (2 j + par) + 2 (lane % 4) + {0, 1}, at rs[8 j]; the block's are on
+      // their way to L1 while the MMAs run
+      const T* rs0 = (const T*)t.row_scale + (int64_t)tile.x * Mp + blk * n;
+      const T2* rs = (const T2*)(rs0 + 8 * par + 2 * (lane & 3));
+      if (lane * 32 < nb * (int)sizeof(T)) asm volatile("prefetch.global.L1 [%0];" ::"l"((const char*)rs0 + lane * 32));
       int okw = 0;
       if (lane == 0) okw = mbar_wait(smem_u32(acc_full), (uint32_t)(i & 1), status) ? 1 : 0;
       okw = __shfl_sync(0xffffffffu, okw, 0);

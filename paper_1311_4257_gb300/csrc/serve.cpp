@@ -290,7 +290,7 @@ int dfmm_server_create(int streams, int64_t budget_bytes, int max_rhs, dfmm_serv
   if (cudaGetDevice(&S->device) != cudaSuccess) return serr(DFMM_ERR_CUDA, "no current device");
   S->budget = (size_t)budget_bytes;
   S->max_rhs = max_rhs;
-  if (cudaMalloc(&S->base, S->budget) != cudaSuccess) {
+  if (dfmm::device_malloc((void**)&S->base, S->budget) != cudaSuccess) {
     cudaGetLastError();
     return serr(DFMM_ERR_OOM, "the server's memory arena could not be allocated");
   }

@@ -59,9 +59,9 @@ extern "C" int dfmm_solve(dfmm_plan_t plan, double alpha_re, double alpha_im, do
     const int64_t scratch = (dfmm::krylov_scratch_bytes(N, m + 1) + 255) & ~(int64_t)255;
     constexpr size_t head = 2 * sizeof(double);   // the norm and the status
     const size_t back = head + 2 * (size_t)(m + 1) * sizeof(float2);
-    if (cudaMalloc(&Vb.p, (size_t)(m + 1) * N * sizeof(float2)) != cudaSuccess ||
-        cudaMalloc(&wb.p, (size_t)N * sizeof(float2)) != cudaSuccess ||
-        cudaMalloc(&hb.p, scratch + back) != cudaSuccess) {
+    if (dfmm::device_malloc(&Vb.p, (size_t)(m + 1) * N * sizeof(float2)) != cudaSuccess ||
+        dfmm::device_malloc(&wb.p, (size_t)N * sizeof(float2)) != cudaSuccess ||
+        dfmm::device_malloc(&hb.p, scratch + back) != cudaSuccess) {
       cudaGetLastError();
       return dfmm::set_error(DFMM_ERR_OOM, "GMRES workspace allocation failed");
     }

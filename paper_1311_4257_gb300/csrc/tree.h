@@ -18,15 +18,23 @@ class DevArena {
   T* alloc(int64_t n) {
     void* p = nullptr;
     size_t bytes = (size_t)(n > 0 ? n : 1) * sizeof(T);
-    cudaError_t e = cudaMalloc(&p, bytes);
+    cudaError_t e = device_malloc(&p, bytes);
     if (e != cudaSuccess) {
       cudaGetLastError();
       throw Error(-3, std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
     }
-    ptrs_.push_back(p);
-    bytes_ += bytes;
-    sizes_.push_back(bytes);
-    return (T*)p;
+    return (T*)keep(p, bytes);
+  }
+  // memory that the caller can do without: nullptr where the device has none
+  template <class T>
+  T* try_alloc(int64_t n) {
+    void* p = nullptr;
+    size_t bytes = (size_t)(n > 0 ? n : 1) * sizeof(T);
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    return (T*)keep(p, bytes);
   }
   size_t mark() const { return ptrs_.size(); }
   void release(size_t m) {
@@ -40,6 +48,12 @@ class DevArena {
   size_t bytes() const { return bytes_; }
 
  private:
+  void* keep(void* p, size_t bytes) {
+    ptrs_.push_back(p);
+    bytes_ += bytes;
+    sizes_.push_back(bytes);
+    return p;
+  }
   std::vector<void*> ptrs_;
   std::vector<size_t> sizes_;
   size_t bytes_ = 0;

@@ -1,0 +1,88 @@
+"""Plans and applies that fit the device without the sliced operator images fit with them: the images are the
+last thing a plan takes, and they are given back when something else needs the memory.
+"""
+import gc
+
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+MB = 1 << 20
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1311_4257_gb300 import build
+    build.build()
+
+
+def _rel(a, b):
+    return float((a - b).norm() / b.norm())
+
+
+@pytest.fixture
+def nearly_full():
+    """fill(room): takes the device's free memory but for `room` bytes."""
+    import torch
+    held = []
+
+    def fill(room):
+        gc.collect()
+        torch.cuda.empty_cache()
+        torch.cuda.synchronize()
+        free, _ = torch.cuda.mem_get_info()
+        if free > room:
+            held.append(torch.empty(free - room, dtype=torch.uint8, device="cuda"))
+
+    yield fill
+    held.clear()
+    torch.cuda.empty_cache()
+
+
+def test_images_leave_room_for_what_fitted_without_them(nearly_full):
+    """Room for the plan, the batches its operators are formed in (768 MB) and half a gigabyte more: less
+    than the images would take beside them."""
+    import torch
+    from paper_1311_4257_gb300 import Plan
+    p = workloads.sphere(4.0, 5)
+    plain = Plan(p, 4.0, 1e-8, m2l_mode=1)
+    need = plain.plan_bytes()
+    f = torch.as_tensor(workloads.densities(p.shape[0], 64, 1), device="cuda").to(plain.dtype)
+    want = plain.apply(f)
+    plain.close()
+    u = torch.empty_like(f)
+    nearly_full(need + 768 * MB + 512 * MB)
+    g = Plan(p, 4.0, 1e-8)
+    assert _rel(g.apply(f[:1], u[:1]), want[:1]) < 1e-12
+    assert _rel(g.apply(f, u), want) < 1e-12   # the largest workspace
+    g.validate()
+
+
+def test_images_are_given_back_and_graphs_keep_theirs(nearly_full):
+    """An allocation that the device has room for only without a plan's images takes their place, and the
+    plan's applies run on; the images of a plan with a captured apply stay."""
+    import torch
+    from paper_1311_4257_gb300 import Plan, Server
+    p = workloads.sphere(4.0, 5)
+    a, b = Plan(p, 4.0, 1e-8), Plan(p, 4.0, 1e-8)
+    f = torch.as_tensor(workloads.densities(p.shape[0], 1, 1), device="cuda").to(a.dtype)
+    u, w, t = torch.empty_like(f), torch.empty_like(f), torch.empty_like(f)
+    gr = b.graph(f, w)
+    gr.launch()
+    want = a.apply(f, u).clone()
+    assert _rel(w, want) < 1e-13
+    with_images, kept = a.plan_bytes(), b.plan_bytes()
+    torch.cuda.synchronize()
+    nearly_full(128 * MB)
+    srv = Server(streams=1, budget_bytes=512 * MB)
+    assert a.plan_bytes() < with_images - 256 * MB and b.plan_bytes() == kept
+    assert _rel(a.apply(f, t), want) < 1e-12
+    w.zero_()
+    gr.launch()
+    assert _rel(w, want) < 1e-13
+    torch.cuda.synchronize()
+    srv.close()
