@@ -1294,10 +1294,13 @@ void set_p2l(const dfmm_plan_s* P, Workspace& W, float2* base, int nrhs, bool ow
 
 Workspace* get_workspace(dfmm_plan_s* P, cudaStream_t s, int nrhs) {
   std::lock_guard<std::mutex> g(P->ws_mu);
-  auto& slot = P->ws[s];
-  if (slot && slot->nrhs >= nrhs) return slot.get();
-  slot.reset(new Workspace());
-  Workspace* W = slot.get();
+  auto it = P->ws.find(s);
+  if (it != P->ws.end()) {
+    if (it->second->nrhs >= nrhs) return it->second.get();
+    P->ws.erase(it);
+  }
+  std::unique_ptr<Workspace> own(new Workspace());   // the stream's once it is complete
+  Workspace* W = own.get();
   W->nrhs = nrhs;
   W->may_fork = true;
   DevArena& ar = W->ar;
@@ -1346,6 +1349,7 @@ Workspace* get_workspace(dfmm_plan_s* P, cudaStream_t s, int nrhs) {
       W->sl = nullptr;
     }
   }
+  P->ws[s] = std::move(own);
   return W;
 }
 

@@ -86,3 +86,28 @@ def test_images_are_given_back_and_graphs_keep_theirs(nearly_full):
     assert _rel(w, want) < 1e-13
     torch.cuda.synchronize()
     srv.close()
+
+
+def test_apply_fails_again_after_a_workspace_that_did_not_fit(nearly_full):
+    """A workspace that the device has no room for is not there for the next call either: every such call
+    reports it, and smaller ones and later ones run."""
+    import torch
+    from paper_1311_4257_gb300 import Plan, dfmm
+    p = workloads.sphere(4.0, 5)
+    g = Plan(p, 4.0, 1e-5)
+    f = torch.as_tensor(workloads.densities(p.shape[0], 64, 1), device="cuda").to(g.dtype)
+    u = torch.empty_like(f)
+    want = g.apply(f).clone()
+    assert _rel(g.apply(f[:1], u[:1]), want[:1]) < 1e-6   # and everything the comparison needs is loaded
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    nearly_full(g.workspace_bytes(64) // 2)
+    for _ in range(3):
+        with pytest.raises(dfmm.DfmmError) as e:
+            g.apply(f, u, stream=s)
+        assert e.value.code == dfmm.ERR_OOM
+    assert g.sync_status(s) == dfmm.OK
+    g.validate()
+    g.apply(f[:1], u[:1], stream=s)
+    s.synchronize()
+    assert _rel(u[:1], want[:1]) < 1e-6
