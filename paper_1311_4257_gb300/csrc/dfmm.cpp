@@ -2548,10 +2548,8 @@ int dfmm_apply_host(dfmm_plan_t plan, const void* f_host, void* u_host, int nrhs
     if (nrhs < 1 || nrhs > 64) return fail(DFMM_ERR_INVALID, "nrhs must be in [1, 64]");
     Workspace* W = get_workspace(plan, stream, nrhs);
     size_t bytes = (size_t)plan->N * nrhs * sizeof(float2) * plan->cw;
-    if (!W->f_dev) {
-      W->f_dev = W->ar.alloc<float2>(plan->N * W->nrhs * plan->cw);
-      W->u_dev = W->ar.alloc<float2>(plan->N * W->nrhs * plan->cw);
-    }
+    if (!W->f_dev) W->f_dev = W->ar.alloc<float2>(plan->N * W->nrhs * plan->cw);
+    if (!W->u_dev) W->u_dev = W->ar.alloc<float2>(plan->N * W->nrhs * plan->cw);
     DFMM_CUDA(cudaMemcpyAsync(W->f_dev, f_host, bytes, cudaMemcpyHostToDevice, stream));
     run_apply(plan, W->f_dev, W->u_dev, nrhs, stream);
     DFMM_CUDA(cudaMemcpyAsync(u_host, W->u_dev, bytes, cudaMemcpyDeviceToHost, stream));

@@ -38,6 +38,7 @@ def nearly_full():
         if free > room:
             held.append(torch.empty(free - room, dtype=torch.uint8, device="cuda"))
 
+    fill.held = held
     yield fill
     held.clear()
     torch.cuda.empty_cache()
@@ -111,3 +112,27 @@ def test_apply_fails_again_after_a_workspace_that_did_not_fit(nearly_full):
     g.apply(f[:1], u[:1], stream=s)
     s.synchronize()
     assert _rel(u[:1], want[:1]) < 1e-6
+
+
+def test_host_apply_fails_again_without_room_for_its_staging(nearly_full):
+    """Room for the workspace and one of the two staging buffers of a host apply: it reports that every time,
+    and runs once there is more."""
+    import numpy as np
+    import torch
+    from paper_1311_4257_gb300 import Plan, dfmm
+    p = workloads.sphere(16.0, 5)   # 64 right-hand sides: 41 MB a staging buffer
+    g = Plan(p, 16.0, 1e-4)
+    f = np.ascontiguousarray(workloads.densities(p.shape[0], 64, 1), dtype=np.complex64)
+    fd = torch.as_tensor(f, device="cuda")
+    want = g.apply(fd)
+    assert _rel(g.apply(fd), want) < 1e-6
+    torch.cuda.synchronize()
+    one = f.nbytes
+    nearly_full(one + one // 2)
+    for _ in range(3):
+        with pytest.raises(dfmm.DfmmError) as e:
+            g.apply_host(f)
+        assert e.value.code == dfmm.ERR_OOM
+    nearly_full.held.clear()
+    torch.cuda.empty_cache()
+    assert _rel(torch.as_tensor(g.apply_host(f), device="cuda"), want) < 1e-6
