@@ -1598,6 +1598,17 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
       }
   const bool fused = zbytes <= kFusedZero && z.n <= ZeroRanges::kMax;
   const bool late = !count && !ctl && !fused && !W->zero_late.empty();
+  // an apply that ends in an error leaves nothing on the side stream that its stream, and with it the next apply
+  // on the workspace, does not wait for
+  struct Rejoin {
+    cudaStream_t s;
+    Workspace* W = nullptr;
+    ~Rejoin() {
+      if (!W) return;
+      cudaEventRecord(W->join, W->side);
+      cudaStreamWaitEvent(s, W->join, 0);
+    }
+  } rejoin{stream};
   auto fork_side = [&] {
     if (!W->side) {
       DFMM_CUDA(cudaStreamCreateWithFlags(&W->side, cudaStreamNonBlocking));
@@ -1607,6 +1618,7 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
     }
     DFMM_CUDA(cudaEventRecord(W->fork, s));
     DFMM_CUDA(cudaStreamWaitEvent(W->side, W->fork, 0));
+    rejoin.W = W;
   };
   if (late) {
     fork_side();
@@ -1742,7 +1754,10 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
   if (P->l_lf0 < nl)
     R.at(kWaveTopV).gemm(P->lf[P->l_lf0].v, S(P->l_lf0), P->lf[P->l_lf0].R, P->lf[P->l_lf0].nbox, T(P->l_lf0),
            P->lf[P->l_lf0].R, kSrcS + P->l_lf0);
-  if (late) DFMM_CUDA(cudaStreamWaitEvent(s, W->join, 0));   // the HF states are reset
+  if (late) {
+    DFMM_CUDA(cudaStreamWaitEvent(s, W->join, 0));   // the HF states are reset
+    rejoin.W = nullptr;
+  }
   // 2. HF upward: M2M, then that level's M2L
   if (P->l_top >= 0) {
     for (int l = P->l1; l >= P->l_top; --l) {
@@ -1807,8 +1822,10 @@ void run_apply(dfmm_plan_s* P, const float2* f, float2* u, int nrhs, cudaStream_
                [&] { m2p(k, s); });
     }
   // 6. near field
-  if (beside) DFMM_CUDA(cudaStreamWaitEvent(s, W->join, 0));
-  else
+  if (beside) {
+    DFMM_CUDA(cudaStreamWaitEvent(s, W->join, 0));
+    rejoin.W = nullptr;
+  } else
     R.at(kWaveP2P).launch(F_P2P, (double)P->stats.p2p_interactions * (16.0 + 8.0 * nrhs),
                           (double)N * (32.0 + 24.0 * nrhs), [&] { near_field(s); });
   R.at(kWaveEnd).launch(F_PERMUTE, 0.0, 20.0 * N * nrhs, [&] {
