@@ -1927,11 +1927,11 @@ int64_t workspace_bytes(dfmm_plan_s* P, int nrhs, bool full, bool slices = false
 }
 
 // A carved workspace of its own in `ar`, for applies that live on: the full layout, or where it does not fit
-// the device, the least.
-void own_workspace(dfmm_plan_s* P, int nrhs, DevArena& ar, cudaStream_t s, Workspace& W) {
-  W.slices.reset(new SliceUse(P->images));
-  size_t bytes = (size_t)workspace_bytes(P, nrhs, true, W.slices->im != nullptr);
-  char* base = ar.try_alloc<char>((int64_t)bytes);
+// the device (or `least` is set), the least.
+void own_workspace(dfmm_plan_s* P, int nrhs, DevArena& ar, cudaStream_t s, Workspace& W, bool least = false) {
+  W.slices.reset(new SliceUse(least ? nullptr : P->images));
+  size_t bytes = least ? 0 : (size_t)workspace_bytes(P, nrhs, true, W.slices->im != nullptr);
+  char* base = least ? nullptr : ar.try_alloc<char>((int64_t)bytes);
   const bool full = base != nullptr;
   if (!full) {
     W.slices.reset();
@@ -2742,13 +2742,24 @@ int dfmm_batch_create(const dfmm_plan_t* plans, const void* const* f, void* cons
       B->f.push_back((const float2*)f[k]);
       B->u.push_back((float2*)u[k]);
     }
-    // one carved workspace per plan (work tables copied in here, before any capture)
-    for (int k = 0; k < count; ++k) {
-      std::unique_ptr<Workspace> W(new Workspace());
-      own_workspace(B->plans[k], B->nrhs[k], B->ar, stream, *W);
-      B->ws.push_back(std::move(W));
+    // one carved workspace per plan (work tables copied in here, before any capture); if the full layouts of
+    // some leave no room for the others, the least for all
+    for (bool least = false;;) {
+      try {
+        B->status = B->ar.alloc<unsigned>(1);
+        for (int k = 0; k < count; ++k) {
+          std::unique_ptr<Workspace> W(new Workspace());
+          own_workspace(B->plans[k], B->nrhs[k], B->ar, stream, *W, least);
+          B->ws.push_back(std::move(W));
+        }
+        break;
+      } catch (const Error& e) {
+        if (e.code != DFMM_ERR_OOM || least) throw;
+        least = true;
+        B->ws.clear();
+        B->ar.release(0);
+      }
     }
-    B->status = B->ar.alloc<unsigned>(1);
     DFMM_CUDA(cudaMemsetAsync(B->status, 0, 4, stream));
     for (int j = 0; j < dfmm_batch_s::kSide; ++j) {
       DFMM_CUDA(cudaStreamCreateWithFlags(&B->side[j], cudaStreamNonBlocking));

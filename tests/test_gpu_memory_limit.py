@@ -136,3 +136,27 @@ def test_host_apply_fails_again_without_room_for_its_staging(nearly_full):
     nearly_full.held.clear()
     torch.cuda.empty_cache()
     assert _rel(torch.as_tensor(g.apply_host(f), device="cuda"), want) < 1e-6
+
+
+def test_batch_fits_where_its_least_workspaces_do(nearly_full):
+    """Room for the least workspace of every plan of a batch, with the first ones' full layouts taken first."""
+    import torch
+    from paper_1311_4257_gb300 import Batch, Plan
+    p, nrhs = workloads.sphere(8.0, 5), 32
+    plans = [Plan(p, 8.0, 1e-6) for _ in range(2)]
+    fs = [torch.as_tensor(workloads.densities(p.shape[0], nrhs, k), device="cuda").to(torch.complex64) for k in range(2)]
+    want = [g.apply(f) for g, f in zip(plans, fs)]
+    us = [torch.empty_like(f) for f in fs]
+    for w, f in zip(want, fs):
+        assert _rel(w, w) == 0.0 and f.shape == w.shape
+    least = plans[0].workspace_bytes(nrhs)
+    torch.cuda.synchronize()
+    nearly_full(2 * least + 8 * MB)
+    b = Batch(plans, fs, us, graph=False, tune=False)
+    b.launch()
+    torch.cuda.synchronize()
+    nearly_full.held.clear()
+    torch.cuda.empty_cache()
+    for u, w in zip(us, want):
+        assert _rel(u, w) < 1e-6
+    b.close()
