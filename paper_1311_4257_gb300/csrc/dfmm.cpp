@@ -1418,6 +1418,14 @@ std::vector<int4> make_tiles(const GemmPlan& g, int nrhs, int cols, int tile_ord
   return out;
 }
 
+// how many that are
+int64_t tile_count(const GemmPlan& g, int nrhs, int cols) {
+  const int per = std::max(1, cols / nrhs);
+  int64_t n = 0;
+  for (const int4& grp : g.groups) n += (grp.z + per - 1) / per;
+  return n;
+}
+
 std::pair<int4*, int64_t> tiles_for(const dfmm_plan_s* P, Workspace* W, const GemmPlan& g, int nrhs, int cols,
                                     cudaStream_t s) {
   auto key = std::make_pair((const void*)&g, nrhs * 1024 + cols);
@@ -1897,24 +1905,28 @@ size_t carve_workspace(dfmm_plan_s* P, int nrhs, char* base, size_t bytes, cudaS
     W.sl = take((size_t)max_slice_bytes(P) * nrhs);
     W.sl_scale = take((size_t)max_source_rows(P) * nrhs * 8);
   }
-  std::vector<std::pair<const GemmPlan*, std::vector<int4>>> tl;
-  std::vector<int> tl_cols;
+  struct Tiles {
+    const GemmPlan* g;
+    int cols;
+    int64_t n;
+    int4* dst;
+  };
+  std::vector<Tiles> tl;
   for (const GemmPlan* g : all_gemms(P)) {
     if (g->npairs == 0) continue;
     const int cols = tile_columns(P, *g, nrhs, full, slices);
-    tl_cols.push_back(cols);
-    tl.push_back({g, make_tiles(*g, nrhs, cols, P->opt.tile_order)});
+    tl.push_back({g, cols, tile_count(*g, nrhs, cols), nullptr});
   }
-  std::vector<int4*> dst(tl.size());
-  for (size_t k = 0; k < tl.size(); ++k) dst[k] = (int4*)take(tl[k].second.size() * sizeof(int4));
+  for (Tiles& t : tl) t.dst = (int4*)take(t.n * sizeof(int4));
   if (!base) return off;
   if (off > bytes)
     throw Error(DFMM_ERR_UNSUPPORTED, "apply needs " + std::to_string(off) + " bytes of scratch, more than the " +
                                           std::to_string(bytes) + " bytes of the static scratch array");
-  for (size_t k = 0; k < tl.size(); ++k) {
-    DFMM_CUDA(cudaMemcpyAsync(dst[k], tl[k].second.data(), tl[k].second.size() * sizeof(int4),
-                              cudaMemcpyHostToDevice, s));
-    W.tiles[std::make_pair((const void*)tl[k].first, nrhs * 1024 + tl_cols[k])] = {dst[k], (int64_t)tl[k].second.size()};
+  // (copies from pageable memory return once the source has been read)
+  for (const Tiles& t : tl) {
+    const std::vector<int4> h = make_tiles(*t.g, nrhs, t.cols, P->opt.tile_order);
+    DFMM_CUDA(cudaMemcpyAsync(t.dst, h.data(), h.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+    W.tiles[std::make_pair((const void*)t.g, nrhs * 1024 + t.cols)] = {t.dst, t.n};
   }
   return off;
 }
