@@ -62,6 +62,8 @@ struct GemmPlan {
   int2* pairs = nullptr;
   std::vector<int32_t> h_dst;      // target row of every pair (host), for tile ordering
   int64_t npairs = 0;
+  int parts = 1;                   // operators that one product's columns are divided over (P2L of the FP64 form),
+                                   // as many pairs each; the CUDA cores take them in turn with the first one's tiles
   int fam = 0;                     // profiling family
   __half* img = nullptr;           // tensor-core operator image (tensor form only)
   float* op_scale = nullptr;       // its per-operator power-of-two scales
@@ -123,7 +125,7 @@ struct LFLevel {
   int R = 0, r = 0;
   int64_t nbox = 0;
   GemmPlan m2m, l2l, v, p2l;   // m2m from l+1, l2l from l-1 (LF or HF)
-  int p2l_halves = 1;          // operators the P2L projection's columns are divided over
+  int p2l_halves = 1;          // p2l.parts: rows that the check points of an X pair take
   ChkPt* chk_b2 = nullptr;
   double* chk64 = nullptr;         // FP64 form: the check points b2, [2r][3]
   int4* p2l_jobs = nullptr;
@@ -718,7 +720,7 @@ void build_plan(dfmm_plan_s* P, const double* d_points, cudaStream_t s) {
     // the P2L projection, R x 2R; the sliced FP64 form takes it as two operators of R
     // columns on the two halves of a check-point row, whose integer sums stay exact
     F.p2l_halves = P->sliced && P->fp64 ? 2 : 1;
-    F.p2l.M = R; F.p2l.Kd = 2 * R / F.p2l_halves; F.p2l.nops = F.p2l_halves;
+    F.p2l.M = R; F.p2l.Kd = 2 * R / F.p2l_halves; F.p2l.nops = F.p2l.parts = F.p2l_halves;
     F.p2l.ops = upload_projection(rp.Qi, rp.r, F.p2l_halves, R, P->fp64, ar, s);
     std::vector<int4> jobs;
     std::vector<int32_t> op;
@@ -1379,10 +1381,17 @@ bool few_columns(const dfmm_plan_s* P, const GemmPlan& g, int nrhs) {
   return P->few && g.npairs * nrhs <= cols * ops;
 }
 
+constexpr int kCoreColumns = 64;   // of the CUDA-core forms' work tiles
+
 // columns of a stage's work tiles (full: in a full layout; slices: images and source slices are there)
 int tile_columns(const dfmm_plan_s* P, const GemmPlan& g, int nrhs, bool full, bool slices) {
   if (full && few_columns(P, g, nrhs)) return gemm_few_columns();
-  return on_tensor_cores(P, g) || (slices && sliced_stage(g)) ? gemm_tc_columns() : 64;
+  return on_tensor_cores(P, g) || (slices && sliced_stage(g)) ? gemm_tc_columns() : kCoreColumns;
+}
+
+// Groups of pairs that a stage has work tiles for.
+size_t tile_groups(const GemmPlan& g, int cols) {
+  return g.parts > 1 && cols == kCoreColumns ? std::min<size_t>(1, g.groups.size()) : g.groups.size();
 }
 
 // Work tiles of a stage: runs of up to cols / nrhs pairs of one operator.
@@ -1404,12 +1413,14 @@ std::vector<int4> make_tiles(const GemmPlan& g, int nrhs, int cols, int tile_ord
   const bool blocked = tile_order == 1 || (tile_order == 0 && (double)g.nops * g.M * g.Kd * 8.0 <= 64.0 * (1 << 20));
   const int64_t block_rows = blocked ? std::max<int64_t>(1, block_bytes / std::max<int64_t>(1, row_bytes))
                                      : ((int64_t)1 << 40);
-  for (const int4& grp : g.groups)
+  for (size_t k = 0, n = tile_groups(g, cols); k < n; ++k) {
+    const int4 grp = g.groups[k];
     for (int p = 0; p < grp.z; p += per) {
       t.push_back(make_int4(grp.x, grp.y + p, std::min(per, grp.z - p), 0));
       const int64_t blk = g.h_dst.empty() ? 0 : g.h_dst[grp.y + p] / block_rows;
       key.push_back(blk * (int64_t)(g.nops + 1) + grp.x);
     }
+  }
   std::vector<int64_t> order(t.size());
   for (size_t i = 0; i < order.size(); ++i) order[i] = (int64_t)i;
   std::stable_sort(order.begin(), order.end(), [&](int64_t a, int64_t b) { return key[a] < key[b]; });
@@ -1422,7 +1433,7 @@ std::vector<int4> make_tiles(const GemmPlan& g, int nrhs, int cols, int tile_ord
 int64_t tile_count(const GemmPlan& g, int nrhs, int cols) {
   const int per = std::max(1, cols / nrhs);
   int64_t n = 0;
-  for (const int4& grp : g.groups) n += (grp.z + per - 1) / per;
+  for (size_t k = 0; k < tile_groups(g, cols); ++k) n += (g.groups[k].z + per - 1) / per;
   return n;
 }
 
@@ -1550,8 +1561,13 @@ struct Runner {
     } else {
       ProfScope ps(W, s, g.fam, g.flops_rhs * nrhs, g.bytes_fixed + g.bytes_rhs * nrhs);
       if (few) launch_gemm_stage_few(a, s);
-      else if (P->fp64) launch_gemm_stage64(a, s);
-      else launch_gemm_stage(a, s);
+      else if (!P->fp64) launch_gemm_stage(a, s);
+      else
+        for (int h = 0; h < g.parts; ++h) {
+          a.ops = g.ops + (size_t)h * g.M * g.Kd * P->cw;
+          a.pairs = g.pairs + h * (g.npairs / g.parts);
+          launch_gemm_stage64(a, s);
+        }
     }
   }
 };
