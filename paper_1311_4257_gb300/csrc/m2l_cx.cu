@@ -62,6 +62,7 @@
 
 #include "apply.h"
 #include "pdl.h"
+#include "per_device.h"
 #include "tcgen05.cuh"
 
 namespace dfmm {
@@ -622,16 +623,20 @@ void launch_split_cx(const float2* x, int64_t rows, int r, void* out, float* sca
 }
 
 template <int KIND, bool ONE>
-void launch_cx(const GemmArgs& a, const TcArgs& t, int nblk, unsigned* status, unsigned grid, LaunchStream s) {
-  static bool attr[64] = {false};
+void launch_cx(const GemmArgs& a, const TcArgs& t, unsigned* status, LaunchStream s) {
+  static PerDevice<int> sms;   // set up with the kernel's launch attribute
   int dev = 0;
   DFMM_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) throw Error(-1, "device ordinal out of range");
-  if (!attr[dev]) {
+  const int nsm = sms.get(dev, [&] {
+    int n = 0;
     DFMM_CUDA(cudaFuncSetAttribute(gemm_cx_kernel<KIND, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, CX_SMEM));
-    attr[dev] = true;
-  }
-  launch_pdl(gemm_cx_kernel<KIND, ONE>, grid, CX_THREADS, CX_SMEM, s, a, t, nblk, status);
+    DFMM_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    return n;
+  });
+  const int n = cx_block(a.M), nblk = (a.M + n - 1) / n;
+  const int64_t items = a.ntiles * nblk;
+  if (items > INT32_MAX / 2) throw Error(-5, "translation stage has too many work items");
+  launch_pdl(gemm_cx_kernel<KIND, ONE>, (unsigned)std::min<int64_t>(items, nsm), CX_THREADS, CX_SMEM, s, a, t, nblk, status);
 }
 
 void launch_gemm_stage_cx(const GemmArgs& a, const TcArgs& t, unsigned* status, bool one_acc, int kind,
@@ -639,24 +644,15 @@ void launch_gemm_stage_cx(const GemmArgs& a, const TcArgs& t, unsigned* status, 
   if (a.ntiles == 0) return;
   if (!gemm_cx_supported(a.M, a.Kd, kind) || a.src_ld != a.Kd)
     throw Error(-5, "split-complex stage needs ranks that are multiples of 16, <= 256, and dense source rows");
-  static int nsm[64] = {0};
-  int dev = 0;
-  DFMM_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) throw Error(-1, "device ordinal out of range");
-  if (!nsm[dev]) DFMM_CUDA(cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev));
-  const int n = cx_block(a.M), nblk = (a.M + n - 1) / n;
-  const int64_t items = a.ntiles * nblk;
-  if (items > INT32_MAX / 2) throw Error(-5, "translation stage has too many work items");
-  const unsigned grid = (unsigned)std::min<int64_t>(items, nsm[dev]);
   if (kind == 0) {
-    if (one_acc) launch_cx<0, true>(a, t, nblk, status, grid, s);
-    else launch_cx<0, false>(a, t, nblk, status, grid, s);
+    if (one_acc) launch_cx<0, true>(a, t, status, s);
+    else launch_cx<0, false>(a, t, status, s);
   } else if (kind == 1) {
-    if (one_acc) launch_cx<1, true>(a, t, nblk, status, grid, s);
-    else launch_cx<1, false>(a, t, nblk, status, grid, s);
+    if (one_acc) launch_cx<1, true>(a, t, status, s);
+    else launch_cx<1, false>(a, t, status, s);
   } else {
-    if (one_acc) launch_cx<2, true>(a, t, nblk, status, grid, s);
-    else launch_cx<2, false>(a, t, nblk, status, grid, s);
+    if (one_acc) launch_cx<2, true>(a, t, status, s);
+    else launch_cx<2, false>(a, t, status, s);
   }
   DFMM_CUDA(cudaGetLastError());
 }

@@ -61,6 +61,7 @@
 
 #include "apply.h"
 #include "pdl.h"
+#include "per_device.h"
 #include "tcgen05.cuh"
 
 namespace dfmm {
@@ -637,20 +638,19 @@ __global__ __launch_bounds__(SL_THREADS, 1) void gemm_sl_kernel(GemmArgs a, SlAr
 
 template <int S, class T2, class T>
 void launch_sl(const GemmArgs& a, const SlArgs& t, unsigned* status, LaunchStream s) {
-  static bool attr[64] = {false};
-  static int nsm[64] = {0};
+  static PerDevice<int> sms;   // set up with the kernel's launch attribute
   int dev = 0;
   DFMM_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) throw Error(-1, "device ordinal out of range");
-  if (!attr[dev]) {
+  const int nsm = sms.get(dev, [&] {
+    int n = 0;
     DFMM_CUDA(cudaFuncSetAttribute(gemm_sl_kernel<S, T2, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, sl_smem<S>()));
-    DFMM_CUDA(cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev));
-    attr[dev] = true;
-  }
+    DFMM_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    return n;
+  });
   const int n = block_rows<S>(a.M), nblk = (a.M + n - 1) / n;
   const int64_t items = a.ntiles * nblk;
   if (items > INT32_MAX - 1024) throw Error(-5, "translation stage has too many work items");
-  launch_pdl(gemm_sl_kernel<S, T2, T>, (unsigned)std::min<int64_t>(items, nsm[dev]), SL_THREADS, sl_smem<S>(), s, a, t, nblk, status);
+  launch_pdl(gemm_sl_kernel<S, T2, T>, (unsigned)std::min<int64_t>(items, nsm), SL_THREADS, sl_smem<S>(), s, a, t, nblk, status);
   DFMM_CUDA(cudaGetLastError());
 }
 

@@ -43,6 +43,7 @@
 #include <algorithm>
 
 #include "apply.h"
+#include "per_device.h"
 #include "tcgen05.cuh"
 
 namespace dfmm {
@@ -439,17 +440,18 @@ void launch_gemm_stage_tc(const GemmArgs& a, const TcArgs& t, unsigned* status, 
   if (a.ntiles == 0) return;
   if (!gemm_tc_supported(a.M, a.Kd) || a.src_ld != a.Kd)
     throw Error(-5, "tensor-core stage needs ranks padded to a multiple of 8 and dense source rows");
-  static int nsm[64] = {0};
+  static PerDevice<int> sms;   // set up with the kernel's launch attribute
   int dev = 0;
   DFMM_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) throw Error(-1, "device ordinal out of range");
-  if (!nsm[dev]) {
+  const int nsm = sms.get(dev, [&] {
+    int n = 0;
     DFMM_CUDA(cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-    DFMM_CUDA(cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev));
-  }
+    DFMM_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    return n;
+  });
   const int nb = (2 * a.M + TC_NMAX - 1) / TC_NMAX;
   const int64_t nitems = a.ntiles * nb;
-  const unsigned grid = (unsigned)std::min<int64_t>(nitems, nsm[dev]);
+  const unsigned grid = (unsigned)std::min<int64_t>(nitems, nsm);
   gemm_tc_kernel<<<grid, TC_THREADS, SMEM_BYTES, s>>>(a, t, nitems, nb, status);
   DFMM_CUDA(cudaGetLastError());
 }
