@@ -62,8 +62,9 @@ typedef struct {
                               pivoted QR (at least twice the largest rank) */
   double eps_op_factor;    /* [0 = 0.3 if eps >= 1e-7, else 0.1] skeleton tolerance = eps * factor */
   int32_t m2l_mode;        /* [0] translations on: 0 = automatic (tensor cores: the split of mode 2 if
-                              eps >= 1e-5, else the sliced form, which keeps the full FP32 or FP64
-                              precision; CUDA cores where neither applies), 1 = CUDA cores,
+                              eps >= 1e-5, else the sliced form, whose products are within 1e-7
+                              (FP32) or 3e-15 (FP64) of exact ones; CUDA cores where neither
+                              applies or device memory is short), 1 = CUDA cores,
                               2 = tensor cores (tcgen05, scaled FP16 hi/lo split; adds about 2e-6
                               relative error) */
   int32_t host_threads;    /* [0 = all cores] threads for the skeleton precompute */
@@ -107,7 +108,7 @@ typedef struct {
   int32_t arith;           /* [0] arithmetic of the apply: 0 = automatic (32 if eps >= 1e-6, else
                               64); 32 = the FP32 forms above (complex64 f and u); 64 = FP64
                               throughout (rows, check points and near field on the CUDA cores,
-                              translations there with m2l_mode 1 and in FP64-exact slices on the
+                              translations there with m2l_mode 1 and in slices of 56 bits on the
                               tensor cores otherwise; operators kept in complex128), for eps down
                               to 1e-8.  With 64, f and u of every apply entry point are complex128
                               [nrhs][N], m2l_mode 2 is refused and the p2p / tc options are
@@ -223,11 +224,15 @@ int dfmm_plan_stats(dfmm_plan_t plan, dfmm_stats* out);
  * buffers and work tables; the plan itself is not included).  Plans whose
  * translations are sliced (automatic form below eps 1e-5) take a source buffer
  * of their slices beside it where the memory at hand holds it, and run on the
- * CUDA cores where it does not.  -1 on a bad argument. */
+ * CUDA cores where it does not; a server's groups hold the least.  -1 on a bad
+ * argument. */
 int64_t dfmm_apply_workspace_bytes(dfmm_plan_t plan, int nrhs);
 
-/* Device bytes held by the plan (tree, lists, operators, evaluation rows);
- * the same value as dfmm_stats.plan_bytes.  -1 for a NULL plan. */
+/* Device bytes held by the plan now (tree, lists, operators, evaluation rows, tensor-core
+ * images); the same value as dfmm_stats.plan_bytes.  The images of the sliced form are taken
+ * only from memory beyond an eighth of the device, and given back (the applies then run
+ * on the CUDA cores) when an allocation of the library does not fit beside them, unless a
+ * captured apply, a batch or an apply being queued uses them.  -1 for a NULL plan. */
 int64_t dfmm_plan_bytes(dfmm_plan_t plan);
 
 /* Several independent matvecs in one call: u[k] = G_k f[k] for k < count,

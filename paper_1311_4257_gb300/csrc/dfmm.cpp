@@ -6,12 +6,14 @@
 // tables and draws the skeleton samples, the device selects the skeletons
 // (skeleton_gpu.cu; host threads with options.skeleton_host) and forms the
 // operators and evaluation rows in FP64 (operators.cu).
-// Apply (one stream, no host synchronisation): permute in, P2M, LF-M2M, the
-// top V list, then per HF level HF-M2M and HF-M2L, HF-L2L, HF->LF L2L, LF-L2L
-// and LF-M2L (V), P2L (X), L2P, M2P (W), P2P (U), permute out.  The split
-// (m2l_cx.cu, m2l_tc.cu) and sliced (m2l_sl.cu) tensor-core, FP32 (apply.cu) and
-// FP64 (apply64.cu) kernels serve the arithmetic forms.  Also here: the allocation-free and captured
-// applies, the batched forms, dfmm_validate and the live-plan registry.
+// Apply (no host synchronisation): permute in, P2M, up the LF levels LF-M2M and
+// LF-M2L (V), then per HF level HF-M2M and HF-M2L, down HF-L2L, HF->LF L2L, LF-L2L
+// and the P2L (X) projections, L2P, permute out.  The near field (P2P, U), the P2L
+// potentials and M2P (W) run on a side stream where the body is small, else in line at the
+// end.  The split (m2l_cx.cu, m2l_tc.cu), sliced (m2l_sl.cu) and few-column (gemm_few.cu), FP32
+// (apply.cu) and FP64 (apply64.cu) kernels serve the arithmetic forms.  Also here: the allocation-free
+// and captured applies, the batched forms, dfmm_validate, the live-plan registry and what is given back
+// when device memory is short.
 #include "dfmm.h"
 
 #include <algorithm>
@@ -91,7 +93,7 @@ constexpr int64_t kFusedZero = 160 << 20, kBesideNear = 200000, kEarlyLaunch = 1
 // CUDA-core stage's (8 columns: 43 against 89 and 172 us, eps 1e-6; 27 columns: both 80; a limit
 // of 20: 2.88 against 2.49 ms for the solve of sphere 4), and the split form's.  There 4 columns
 // and, with more operators than SMs, when every SM would compute several nearly empty tiles, 8
-// (applies at eps 1e-5, few against split: sphere of 2 wavelengths, 8 columns, 316 operators: 34
+// (applies at eps 1e-5, few against split: sphere of 2 wavelengths, 8 columns, 316 operators: 36
 // against 47 us; of 3, 7 columns, 62 operators: 76 against 70; of 8, 3,000 points, 10 columns: 143
 // against 136).
 constexpr int kFewColsSplit = 4, kFewColsSplitMany = 8, kFewCols = 12, kSMs = 152;
@@ -2496,8 +2498,8 @@ int dfmm_plan(const double* points, int64_t N, double K, double eps, const dfmm_
     if (!(o.eps_op_factor > 0)) o.eps_op_factor = eps >= 1e-7 ? 0.3 : 0.1;
     if (o.m2l_mode < 0 || o.m2l_mode > 2) return fail(DFMM_ERR_INVALID, "m2l_mode must be 0, 1 or 2");
     // automatic form: the split-FP16 tensor-core form adds about 2e-6
-    // relative error, so it serves eps >= 1e-5; tighter tolerances use FP32
-    // CUDA cores
+    // relative error, so it serves eps >= 1e-5; tighter tolerances start from the
+    // CUDA cores (mode 1), which the sliced form stands in for (P->sliced below)
     if (o.m2l_mode == 0) o.m2l_mode = eps >= 1e-5 ? 2 : 1;
     if (o.tc_stages < 0 || o.tc_stages > 31) return fail(DFMM_ERR_INVALID, "tc_stages must be a mask in [0, 31]");
     if (o.tc_stages == 0) o.tc_stages = 31;
@@ -2521,7 +2523,7 @@ int dfmm_plan(const double* points, int64_t N, double K, double eps, const dfmm_
     if (o.arith == 64) {
       if (opts && opts->m2l_mode == 2)
         return fail(DFMM_ERR_INVALID, "the tensor-core translations are not part of the FP64 form (arith 64)");
-      o.m2l_mode = 1;   // translations on the CUDA cores, in FP64
+      o.m2l_mode = 1;   // translations in FP64: sliced if automatic, else on the CUDA cores
       o.p2p_mode = 1;   // no FP32 near field (and no close-pair pass)
     }
     // automatic near field: FP32 coordinates with exact close-pair
@@ -2537,7 +2539,7 @@ int dfmm_plan(const double* points, int64_t N, double K, double eps, const dfmm_
     P->fp64 = o.arith == 64;
     // automatic translations below eps 1e-5: the sliced tensor-core form, with products
     // of FP32 or FP64 accuracy (m2l_sl.cu) and faster from the smallest stages on (apply,
-    // sphere of 4 wavelengths, eps 1e-6: 0.21 against 0.49 ms; of 32: 3.7 against
+    // sphere of 4 wavelengths, eps 1e-6: 0.137 against 0.50 ms; of 32: 2.96 against
     // 19.5); m2l_mode 1 asks for the CUDA cores, which also serve what the form
     // does not take
     // m2l_mode 2 keeps every stage on the tensor cores, wait_test its waits

@@ -9,7 +9,7 @@
 // and half of the columns.  Columns come in tiles of 16, since a stage lasts as long
 // as its fullest operator: with one block passing over its rows once per 8 columns, up to
 // 28 of them, the V list of a sphere of 2 wavelengths (316 operators of 131 KB, 8 columns on
-// average) took 32 us, in tiles of 16 it takes 19 and its apply 33.5 (47 in split form with
+// average) took 32 us, in tiles of 16 it takes 19 and its apply 36 (47 in split form with
 // 6 us for the split).  Five blocks per SM keep all 644 in flight; three chunks deep
 // the longer rows of eps 1e-6 lose what the sixth block gains (285 against 277 us, sphere of 8).
 // Every output is summed in the order of the CUDA-core stage kernel

@@ -50,9 +50,9 @@
 // clocks, 10k at the MMAs' own rate).
 //
 // Measured against the CUDA-core stages that served these tolerances: sphere of 32
-// wavelengths, eps 1e-6 (N = 321,699, FP32): all translations 19.2 -> 2.47 ms, 22
-// -> 174 TFLOP/s (of 330 at the MMAs' rate); sphere of 8, eps 1e-8 (FP64): 68 ->
-// 2.43 ms, 0.75 -> 21 TFLOP/s.  The warp-wide issue gave the applies 3.76 -> 2.88 and
+// wavelengths, eps 1e-6 (N = 321,699, FP32): all translations 19.2 -> 2.55 ms, 22
+// -> 168 TFLOP/s (of 327 at the MMAs' rate); sphere of 8, eps 1e-8 (FP64): 68 ->
+// 2.41 ms, 0.75 -> 21 TFLOP/s.  The warp-wide issue gave the applies 3.76 -> 2.88 and
 // 3.78 -> 3.03 ms of that.  It is bound by shared-memory bandwidth (operand reads and
 // the copies into the tiles) where tiles are full, by part-filled tiles elsewhere.
 #include <cuda_fp16.h>
