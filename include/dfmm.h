@@ -230,7 +230,7 @@ int64_t dfmm_apply_workspace_bytes(dfmm_plan_t plan, int nrhs);
 
 /* Device bytes held by the plan now (tree, lists, operators, evaluation rows, tensor-core
  * images); the same value as dfmm_stats.plan_bytes.  The images of the sliced form are taken
- * only from memory beyond an eighth of the device, and given back (the applies then run
+ * only from what is free beyond a 64th of the device (4 GB), and given back (the applies then run
  * on the CUDA cores) when an allocation of the library does not fit beside them, unless a
  * captured apply, a batch or an apply being queued uses them.  -1 for a NULL plan. */
 int64_t dfmm_plan_bytes(dfmm_plan_t plan);

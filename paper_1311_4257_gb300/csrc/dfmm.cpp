@@ -184,8 +184,9 @@ bool reclaim_images() {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   std::shared_ptr<SliceImages> most;
-  {
+  for (bool taken = false; !taken;) {
     std::lock_guard<std::mutex> g(g_images_mu);
+    most.reset();
     for (auto& w : g_images)
       if (auto im = w.lock()) {
         std::lock_guard<std::mutex> gi(im->mu);
@@ -193,8 +194,7 @@ bool reclaim_images() {
       }
     if (!most) return false;
     std::lock_guard<std::mutex> gi(most->mu);
-    if (most->users) return false;
-    most->gone = true;   // no apply queued from now on reads them
+    taken = most->gone = most->users == 0;   // no apply queued from now on reads them
   }
   if (cudaDeviceSynchronize() != cudaSuccess) {   // not allowed while this thread captures a stream
     cudaGetLastError();
@@ -2016,8 +2016,8 @@ std::vector<std::vector<GemmPlan*>> stages_by_source(dfmm_plan_s* P) {
 // Sliced images of every translation stage that has the form and that the device has room for (a stage
 // without one stays on the CUDA cores).  They come last, from the operators as the apply's other forms
 // hold them: the entries' scales need all the operators that read a buffer, and what the plan cannot
-// do without is there by then.  An eighth of the device stays free for workspaces, further plans and other
-// users of it.
+// do without is there by then.  A 64th of the device (4 GB) stays free for users of it that cannot ask the
+// images to go: other libraries, and the driver when it loads kernels.
 void build_slices(dfmm_plan_s* P, cudaStream_t s) {
   const int64_t sc = P->fp64 ? 8 : 4;
   auto images = std::make_shared<SliceImages>();
@@ -2025,7 +2025,7 @@ void build_slices(dfmm_plan_s* P, cudaStream_t s) {
   DevArena& ar = images->ar;
   size_t free = 0, total = 0;
   DFMM_CUDA(cudaMemGetInfo(&free, &total));
-  const size_t spare = free > total / 8 ? free - total / 8 : 0;
+  const size_t spare = free > total / 64 ? free - total / 64 : 0;
   uint32_t* bits = ar.try_alloc<uint32_t>(512);
   if (!bits) return;
   for (auto& list : stages_by_source(P)) {

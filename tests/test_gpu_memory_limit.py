@@ -160,3 +160,58 @@ def test_batch_fits_where_its_least_workspaces_do(nearly_full):
     for u, w in zip(us, want):
         assert _rel(u, w) < 1e-6
     b.close()
+
+
+def test_images_go_while_another_thread_applies(nearly_full):
+    """Applies of two plans go on in a thread each while the main thread needs the memory of their images:
+    every result is right, whether an apply ran before, on the images, or after, on the CUDA cores."""
+    import threading
+    import torch
+    from paper_1311_4257_gb300 import Plan, Server, dfmm
+    p = workloads.sphere(4.0, 5)
+    plans = [Plan(p, 4.0, 1e-8) for _ in range(2)]
+    f = torch.as_tensor(workloads.densities(p.shape[0], 1, 1), device="cuda").to(plans[0].dtype)
+    want = plans[0].apply(f).clone()
+    assert _rel(plans[1].apply(f), want) < 1e-13
+    us = [[torch.zeros_like(f) for _ in range(8)] for _ in plans]
+    for g, u in zip(plans, us):
+        g.apply(f, u[0])
+    held = sum(g.plan_bytes() for g in plans)
+    torch.cuda.synchronize()
+    nearly_full(64 * MB)
+    stop, failed = threading.Event(), []
+
+    def work(g, u):
+        s = torch.cuda.Stream()
+        try:
+            k = 0
+            while not stop.is_set():
+                g.apply(f, u[k % 8], stream=s)
+                k += 1
+                s.synchronize()
+        except Exception as e:   # noqa: BLE001
+            failed.append(e)
+
+    threads = [threading.Thread(target=work, args=a) for a in zip(plans, us)]
+    for t in threads:
+        t.start()
+    srv = None
+    for _ in range(200):   # the images are free to go between two applies
+        try:
+            srv = Server(streams=1, budget_bytes=256 * MB)
+            break
+        except dfmm.DfmmError as e:
+            assert e.code == dfmm.ERR_OOM
+    for _ in range(20):
+        torch.cuda.synchronize()
+    stop.set()
+    for t in threads:
+        t.join()
+    assert not failed
+    assert srv is not None and sum(g.plan_bytes() for g in plans) < held
+    srv.close()
+    nearly_full.held.clear()
+    torch.cuda.empty_cache()
+    for u in us:
+        for v in u:
+            assert _rel(v, want) < 1e-12 or not torch.any(v)
