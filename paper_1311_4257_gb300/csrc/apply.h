@@ -286,7 +286,8 @@ void launch_p2p_close(const P2PArgs& a, float delta, int32_t* cnt, unsigned* deg
 // trig_table_bytes() bytes of exp(2 pi i k / n), which the kernel evaluations read.
 int trig_table_bytes();
 void build_trig_table(void* t, cudaStream_t s);
-void launch_gemm_stage64(const GemmArgs& a, LaunchStream s);
+// parts > 1: as many operators of part_pairs pairs each, in order, with the first one's tiles
+void launch_gemm_stage64(const GemmArgs& a, int parts, int64_t part_pairs, LaunchStream s);
 void launch_permute_out64(const float2* us, const int32_t* perm, int64_t N, int nrhs, float2* u, LaunchStream s);
 void launch_p2c64(const P2CArgs& a, LaunchStream s);
 void launch_rows64(const RowsArgs& a, LaunchStream s);

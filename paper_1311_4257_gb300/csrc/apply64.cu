@@ -92,10 +92,11 @@ __device__ __forceinline__ void add_to(double2* p, double2 v) {
 
 // y[dst] += T_op x[src] over a stage's pairs: one CTA computes a 64-row x
 // 64-column block of T_op X (columns = gathered source rows x right-hand
-// sides) and adds it into the target rows with FP64 atomics.
+// sides) and adds it into the target rows with FP64 atomics.  Where a product's columns are divided over
+// several operators (P2L), gridDim.z of them with part_pairs pairs each, the tiles are the first one's.
 constexpr int GM = 64, GN = 64, GK = 8;
 
-__global__ __launch_bounds__(256) void gemm64_kernel(GemmArgs a) {
+__global__ __launch_bounds__(256) void gemm64_kernel(GemmArgs a, int64_t part_pairs) {
   pdl_begin();
   __shared__ double2 As[GK][GM + 1];
   __shared__ double2 Bs[GK][GN + 1];
@@ -103,7 +104,8 @@ __global__ __launch_bounds__(256) void gemm64_kernel(GemmArgs a) {
   __shared__ double2* dstp[GN];
   const int tid = threadIdx.x;
   const int4 tile = a.tiles[blockIdx.x];
-  const double2* A = c128(a.ops) + (size_t)tile.x * a.M * a.Kd;
+  const double2* A = c128(a.ops) + (size_t)(tile.x + blockIdx.z) * a.M * a.Kd;
+  const int2* pairs = a.pairs + blockIdx.z * part_pairs;
   const int row0 = blockIdx.y * GM;
   const int ncol = tile.z * a.nrhs;
   if (tid < GN) {
@@ -111,7 +113,7 @@ __global__ __launch_bounds__(256) void gemm64_kernel(GemmArgs a) {
     double2* dp = nullptr;
     if (tid < ncol) {
       const int p = tile.y + tid / a.nrhs, k = tid % a.nrhs;
-      const int2 pr = a.pairs[p];
+      const int2 pr = pairs[p];
       sp = c128(a.src) + ((int64_t)pr.x * a.nrhs + k) * a.src_ld;
       dp = c128(a.dst) + ((int64_t)pr.y * a.nrhs + k) * a.dst_ld;
     }
@@ -424,10 +426,10 @@ void check_rank(int R) {
 
 }  // namespace
 
-void launch_gemm_stage64(const GemmArgs& a, LaunchStream s) {
+void launch_gemm_stage64(const GemmArgs& a, int parts, int64_t part_pairs, LaunchStream s) {
   if (a.ntiles == 0) return;
-  const dim3 grid((unsigned)a.ntiles, (unsigned)((a.M + GM - 1) / GM));
-  launch_pdl(gemm64_kernel, grid, 256, 0, s, a);
+  const dim3 grid((unsigned)a.ntiles, (unsigned)((a.M + GM - 1) / GM), (unsigned)parts);
+  launch_pdl(gemm64_kernel, grid, 256, 0, s, a, part_pairs);
   DFMM_CUDA(cudaGetLastError());
 }
 

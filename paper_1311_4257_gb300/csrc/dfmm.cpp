@@ -65,7 +65,7 @@ struct GemmPlan {
   std::vector<int32_t> h_dst;      // target row of every pair (host), for tile ordering
   int64_t npairs = 0;
   int parts = 1;                   // operators that one product's columns are divided over (P2L of the FP64 form),
-                                   // as many pairs each; the CUDA cores take them in turn with the first one's tiles
+                                   // as many pairs each; on the CUDA cores the first one's tiles serve all
   int fam = 0;                     // profiling family
   __half* img = nullptr;           // tensor-core operator image (tensor form only)
   float* op_scale = nullptr;       // its per-operator power-of-two scales
@@ -1563,13 +1563,8 @@ struct Runner {
     } else {
       ProfScope ps(W, s, g.fam, g.flops_rhs * nrhs, g.bytes_fixed + g.bytes_rhs * nrhs);
       if (few) launch_gemm_stage_few(a, s);
-      else if (!P->fp64) launch_gemm_stage(a, s);
-      else
-        for (int h = 0; h < g.parts; ++h) {
-          a.ops = g.ops + (size_t)h * g.M * g.Kd * P->cw;
-          a.pairs = g.pairs + h * (g.npairs / g.parts);
-          launch_gemm_stage64(a, s);
-        }
+      else if (P->fp64) launch_gemm_stage64(a, g.parts, g.npairs / g.parts, s);
+      else launch_gemm_stage(a, s);
     }
   }
 };
